@@ -413,8 +413,7 @@ mrcm_status mrcm_measure_fp64_peak(void* stream, double* tflops);
  * two shorter edges) <= 128, longest edge x block^2 <= 262144; larger boxes
  * return MRCM_ERR_OOM.  At least one side must be Robin or Dirichlet
  * (MRCM_ERR_INVALID_ARG otherwise).  The first call on a device looks up the
- * scratch address and sets the kernel's shared-memory limit; make that first
- * call before any stream capture.  The looked-up address is kept for the
+ * scratch address; make that first call before any stream capture.  The looked-up address is kept for the
  * life of the process; calling this entry point again after cudaDeviceReset
  * is not supported.  Every call on a device shares the one
  * scratch array (nothing in it is read before the same call writes it), so

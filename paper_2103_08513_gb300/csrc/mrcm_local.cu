@@ -29,6 +29,7 @@
 
 #include "mrcm_devmath.cuh"
 #include "mrcm_internal.h"
+#include "mrcm_sweep64.cuh"
 
 namespace mrcm {
 
@@ -270,6 +271,74 @@ k_block_factor(const SubInfo* __restrict__ subs, const int* __restrict__ list, c
         __syncthreads();
     }
     if (bad && threadIdx.x == 0) atomicAdd(&status[ST_NOT_SPD], 1);
+}
+
+// FP64 form, b <= 128: the block as 4 x 4 register tiles of its lower triangle
+// (mrcm_sweep64.cuh), one CTA of NTH threads per subdomain; W_{s-1} stays in
+// the registers to form S_s.  Larger blocks keep k_block_factor: from b = 129
+// on the tiles (16 doubles a thread) no longer fit one CTA's registers.
+template <int NTH>
+__global__ void __launch_bounds__(NTH)
+k_block_factor64(const SubInfo* __restrict__ subs, const int* __restrict__ list, const double* __restrict__ coef,
+                 double* __restrict__ Wall, int* __restrict__ status, long long nct,
+                 const int* __restrict__ limit /* CTAs from *limit on have no subdomain; may be NULL */) {
+    if (limit && (int)blockIdx.x >= *limit) return;
+    const SubInfo s = subs[list[blockIdx.x]];
+    const int b = s.b, su = s.su;
+    const int nt = (b + kSw64T - 1) / kSw64T;
+    int ti, tj;
+    sweep64_tile(threadIdx.x, ti, tj);
+    const bool own = ti < nt && threadIdx.x + 32 < NTH;  // the last warp forms the pivots
+    if (!own) ti = tj = 0;                              // idle threads shadow tile (0, 0), never publish or store
+    const int i0 = ti * kSw64T, j0 = tj * kSw64T;
+    const double* cd = coef + s.cell_off;
+    const double* cu = coef + nct + s.cell_off;
+    const double* cv = coef + 2 * nct + s.cell_off;
+    const double* cs = coef + 3 * nct + s.cell_off;
+    __shared__ __align__(16) Sweep64Shared sh;
+    __shared__ double sd[kSw64B], sup[kSw64B], svp[kSw64B], st[kSw64B];
+    if (threadIdx.x == 0) sh.bad = 0;
+    double a[kSw64T][kSw64T];
+#pragma unroll
+    for (int r = 0; r < kSw64T; ++r)
+#pragma unroll
+        for (int c = 0; c < kSw64T; ++c) a[r][c] = 0.0;
+    for (int sl = 0; sl < s.ns; ++sl) {
+        const int base = sl * b;
+        __syncthreads();                                // the previous slab's last step is done with `sh`
+        for (int i = threadIdx.x; i < kSw64B; i += NTH) {
+            double d = 0.0, u = 0.0, v = 0.0, t = 0.0;
+            if (i < b) {
+                const int c = base + i;
+                d = cd[c];
+                if ((i % su) + 1 < su) u = -cu[c];
+                if (i + su < b) v = -cv[c];
+                if (sl > 0) t = cs[c - b];
+            }
+            sd[i] = d; sup[i] = u; svp[i] = v; st[i] = t;
+        }
+        __syncthreads();
+        // S_s = D_s - t o W_{s-1} o t on the tile
+#pragma unroll
+        for (int r = 0; r < kSw64T; ++r) {
+            const int i = i0 + r;
+#pragma unroll
+            for (int c = 0; c < kSw64T; ++c) {
+                const int j = j0 + c;
+                double dij = 0.0;
+                if (j == i) dij += sd[i];
+                if (j == i + 1) dij += sup[i];
+                if (j + 1 == i) dij += sup[j];
+                if (j == i + su) dij += svp[i];
+                if (j + su == i) dij += svp[j];
+                a[r][c] = (i < b && j < b) ? fma(-st[i] * st[j], a[r][c], dij) : 0.0;
+            }
+        }
+        sweep64_invert(a, ti, tj, own, b, sh);
+        sweep64_store(a, ti, tj, own, b, Wall + s.w_off + (long long)sl * wstride<double>(b));
+    }
+    __syncthreads();
+    if (threadIdx.x == 0 && sh.bad) atomicAdd(&status[ST_NOT_SPD], 1);
 }
 
 template <typename T>
@@ -2082,6 +2151,22 @@ Geo make_geo(const mrcm_config& c) {
 // b <= 64, packed shared-memory kernel otherwise; one launch per class).
 int num_solve_variants() { return kNumSolveVariants; }
 
+// FP64 block factors of n listed subdomains whose blocks are at most bmax
+// (limit: see the kernels; big: packed triangles of blocks above kMaxBlock64, or NULL).
+static void launch_factor64(const SubInfo* subs, const int* list, int n, int bmax, const double* coef,
+                            const double* scale, double* W, int* status, long long nct, const int* limit, double* big,
+                            const char* name, cudaStream_t st, Prof& P) {
+    switch (sweep64_threads(bmax)) {
+    case 128: MRCM_LAUNCH(P, name, st, k_block_factor64<128><<<n, 128, 0, st>>>(subs, list, coef, W, status, nct, limit)); break;
+    case 192: MRCM_LAUNCH(P, name, st, k_block_factor64<192><<<n, 192, 0, st>>>(subs, list, coef, W, status, nct, limit)); break;
+    case 352: MRCM_LAUNCH(P, name, st, k_block_factor64<352><<<n, 352, 0, st>>>(subs, list, coef, W, status, nct, limit)); break;
+    case 576: MRCM_LAUNCH(P, name, st, k_block_factor64<576><<<n, 576, 0, st>>>(subs, list, coef, W, status, nct, limit)); break;
+    default:
+        MRCM_LAUNCH(P, name, st, k_block_factor<double, false><<<n, kThreads, factor_smem<double>(std::min(bmax, kMaxBlock64)), st>>>(
+                    subs, list, coef, scale, W, status, nct, nullptr, nullptr, limit, big));
+    }
+}
+
 static void launch_factor_wave(const Tables& t, const DeviceTables& d, const Layout& L, char* ws, int precision,
                                int w, cudaStream_t st, Prof& P) {
     double* coef = (double*)(ws + L.coef);
@@ -2091,11 +2176,15 @@ static void launch_factor_wave(const Tables& t, const DeviceTables& d, const Lay
     const int o0 = wc[0], o1 = wc[1], o2 = wc[2], o3 = wc[3];
     const int n_small = o1 - o0, n_mid = o2 - o1, n_large = o3 - o2;
     if (precision == MRCM_FP64) {
-        if (n_large > 0) {
-            size_t sm = factor_smem<double>(std::min(t.max_b, kMaxBlock64));   // larger blocks: global slot
-            MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor<double, false><<<n_large, kThreads, sm, st>>>(d.subs, d.class_list + o2, coef, scale,
-                (double*)(ws + L.W), status, t.n_cells, (float*)(ws + L.scf), (float*)(ws + L.tsc), nullptr,
-                (double*)(ws + L.big)));
+        (void)n_large;
+        // ordered by b, largest first: one launch per run of subdomains that share a CTA size
+        for (int q = o2; q < o3;) {
+            const int b0 = t.subs[t.class_list[q]].b, nth = sweep64_threads(b0);
+            int e = q + 1;
+            while (e < o3 && sweep64_threads(t.subs[t.class_list[e]].b) == nth) ++e;
+            launch_factor64(d.subs, d.class_list + q, e - q, b0, coef, scale, (double*)(ws + L.W), status, t.n_cells, nullptr,
+                            (double*)(ws + L.big), "k_block_factor", st, P);
+            q = e;
         }
     } else {
         if (n_small > 0) {
@@ -2275,9 +2364,8 @@ static void launch_fallback(const Tables& t, const DeviceTables& d, const Layout
                 g0.conv, status, fb_subs, fb_list, cap, wstride_slot, ystride_slot));
     int bmax = 0;
     for (const SubInfo& s : t.subs) if (s.b <= kMaxBlock64) bmax = std::max(bmax, s.b);
-    MRCM_LAUNCH(P, "k_fb_factor", st, k_block_factor<double, false><<<cap, kThreads, factor_smem<double>(bmax), st>>>(
-                fb_subs, fb_list, g0.coef, g0.scale, (double*)(ws + L.fb_W), status, t.n_cells, nullptr, nullptr,
-                status + ST_FB_WAVE, nullptr));
+    launch_factor64(fb_subs, fb_list, cap, bmax, g0.coef, g0.scale, (double*)(ws + L.fb_W), status, t.n_cells,
+                    status + ST_FB_WAVE, nullptr, "k_fb_factor", st, P);
     LocalArgs g = g0;
     g.subs = fb_subs;
     g.list = fb_list;
@@ -2425,9 +2513,8 @@ int launch_postprocess(const Tables& t, const DeviceTables& d, const Layout& L, 
             MRCM_LAUNCH(P, "k_set_int", st, k_set_int<<<1, 1, 0, st>>>(cnt, 0));
             MRCM_LAUNCH(P, "k_pp_unconverged", st, k_pp_unconverged<<<(n + 127) / 128, 128, 0, st>>>(d.subs,
                         d.solve_list + t.pp_wave_off[w], n, g.conv, plist, cnt, status + ST_FB_TOTAL));
-            MRCM_LAUNCH(P, "k_pp_factor", st, k_block_factor<double, false><<<n, kThreads, factor_smem<double>(bmax), st>>>(
-                        d.pp_subs, plist, coef, (const double*)(ws + L.scale), (double*)(ws + L.W), status, t.n_cells,
-                        nullptr, nullptr, cnt, nullptr));
+            launch_factor64(d.pp_subs, plist, n, bmax, coef, (const double*)(ws + L.scale), (double*)(ws + L.W), status,
+                            t.n_cells, cnt, nullptr, "k_pp_factor", st, P);
             const int grid = std::max(1, std::min(n, d.sms * d.f64_occ));
             void* args[] = {(void*)&g, (void*)&W};
             g.count_unconverged = 0;

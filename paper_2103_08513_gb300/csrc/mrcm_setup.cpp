@@ -289,9 +289,9 @@ mrcm_status build_tables(const mrcm_config* cfg, Tables& t, std::string& err) {
                 const SubInfo& s = t.subs[l];
                 const double cost = (double)s.ns * s.b * s.b * s.b;
                 const int k = cfg->precision == MRCM_FP64 ? 2 : s.b <= kRegBlock ? 0 : s.b <= kTileBlock ? 1 : 2;
-                // mixed large class: ordered by b first (its factor launches
+                // large class and FP64: ordered by b first (its factor launches
                 // one CTA size per run of b), then by cost
-                cls[k].push_back({k == 2 && cfg->precision != MRCM_FP64 ? -s.b : 0, -cost, l});
+                cls[k].push_back({k == 2 ? -s.b : 0, -cost, l});
             }
             for (int k = 0; k < 3; ++k) {
                 std::sort(cls[k].begin(), cls[k].end());
