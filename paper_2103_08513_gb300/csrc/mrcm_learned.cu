@@ -21,6 +21,7 @@
 #include <cstring>
 #include <vector>
 
+#include "mrcm_conv_tc.cuh"
 #include "mrcm_internal.h"
 
 struct mrcm_net {
@@ -31,7 +32,11 @@ struct mrcm_net {
     std::vector<long long> act_off;      // offsets (floats per sample) of stored activations
     long long act_per_sample = 0;
     int max_ch = 0;
-    bool mma_ok = false;                 // 32 -> 32 layers take the tensor-core forward (its shared memory fits)
+    bool mma_ok = false;                 // 32 -> 32 layers take the per-layer tensor-core forward (its shared memory fits)
+    bool tc_ok = false;                  // all layers take the fused tensor-core passes (at most 8 input channels,
+                                         // the box's planes fit shared memory)
+    int C = 32;                          // hidden channels of those passes, padded (16 or 32)
+    int wg_zc_max = 0;                   // most slices per work item of the weight gradients that fit
 };
 
 namespace mrcm {
@@ -417,11 +422,154 @@ NetPtrs net_ptrs(const mrcm_net* n, const float* state) {
     return p;
 }
 
-// Workspace per sample: stored activations (input copy not needed: given),
-// then two gradient buffers of max_ch x S, plus loss partials.
+// Workspace: per sample the stored activations (input copy not needed: given)
+// and two gradient buffers of max_ch x S, then loss partials, the gradient, and
+// for the tensor-core passes the packed weights (forward, backward data), the
+// pre-activation gradients of every layer and the weight gradients' partial sums.
+constexpr int kWgCtas = 152;             // CTAs (partial sums) of the weight gradients: one per SM
+size_t net_pack_bytes(const mrcm_net* n) { return (size_t)n->layers * mrcm::tc_weight_bytes(mrcm::kTcHidden, 32); }
+size_t net_part_floats(const mrcm_net* n, int batch) {   // every weight per CTA, every bias per sample
+    size_t s = 0;
+    for (int l = 0; l < n->layers; ++l) s += (size_t)kWgCtas * 27 * n->cin[l] * n->cout[l] + (size_t)batch * n->cout[l];
+    return s;
+}
 size_t net_ws_bytes(const mrcm_net* n, int batch) {
     const size_t per = (size_t)n->act_per_sample + 2 * (size_t)n->max_ch * n->S;
-    return sizeof(float) * (per * (size_t)batch + 1024 + (size_t)n->P) + 256;
+    size_t s = sizeof(float) * (per * (size_t)batch + 1024 + (size_t)n->P) + 256;
+    s += 2 * net_pack_bytes(n) + sizeof(float) * ((size_t)n->act_per_sample * batch + net_part_floats(n, batch)) + 256;
+    return s;
+}
+struct TcWs { unsigned char* pack_f; unsigned char* pack_b; float* g; float* part; };
+TcWs tc_ws(const mrcm_net* n, void* ws, int batch) {
+    const size_t per = (size_t)n->act_per_sample + 2 * (size_t)n->max_ch * n->S;
+    uintptr_t a = (uintptr_t)ws + sizeof(float) * (per * (size_t)batch + 1024 + (size_t)n->P);
+    a = (a + 255) & ~(uintptr_t)255;     // bulk copies start on 16-byte boundaries
+    TcWs t;
+    t.pack_f = (unsigned char*)a;
+    t.pack_b = t.pack_f + net_pack_bytes(n);
+    t.g = (float*)(t.pack_b + net_pack_bytes(n));
+    t.part = t.g + (size_t)n->act_per_sample * batch;
+    return t;
+}
+
+int sm_count() {
+    int dev = 0, sms = 1;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return sms;
+}
+
+void tc_launch(const mrcm_net* n, const mrcm::TcNet& net, cudaStream_t st) {
+    const mrcm::TcGeo g(n->D, n->H, n->W);
+    const size_t sm = mrcm::tc_plane_bytes(g, n->C) + mrcm::tc_wregion_bytes(g, n->C);
+    const int grid = std::max(1, std::min(net.batch, sm_count()));
+    if (n->C == 16) mrcm::k_tc_net<16><<<grid, mrcm::kTcThreads, sm, st>>>(net);
+    else mrcm::k_tc_net<32><<<grid, mrcm::kTcThreads, sm, st>>>(net);
+}
+
+// All layers in one launch.  y: where the output goes; keep: store the hidden
+// activations at their places in `acts` (a training step needs them).
+void forward_tc(const mrcm_net* n, const NetPtrs& p, const float* x, int batch, float* acts, float* y, bool keep,
+                void* ws, cudaStream_t st) {
+    const TcWs w = tc_ws(n, ws, batch);
+    mrcm::TcPack pk;
+    mrcm::TcNet net;
+    pk.layers = net.layers = n->layers;
+    pk.C = n->C;
+    pk.flip = 0;
+    net.D = n->D; net.H = n->H; net.W = n->W; net.batch = batch; net.x = x; net.wpack = w.pack_f;
+    uint32_t off = 0;
+    for (int l = 0; l < n->layers; ++l) {
+        mrcm::TcLayer& L = net.l[l];
+        const bool last = l + 1 == n->layers;
+        L.kind = last ? mrcm::kTcOut : l == 0 ? mrcm::kTcFirst : mrcm::kTcHidden;
+        L.cin = n->cin[l]; L.cout = n->cout[l]; L.w_off = off;
+        L.bias = p.w + n->b_off[l];
+        L.mask = nullptr;
+        L.out = last ? y : keep ? acts + (long long)batch * n->act_off[l] : nullptr;
+        L.leaky = last ? 0 : 1;
+        L.last = last ? 1 : 0;
+        pk.kind[l] = L.kind; pk.cin[l] = L.cin; pk.cout[l] = L.cout; pk.w[l] = n->w_off[l]; pk.off[l] = off;
+        off += mrcm::tc_weight_bytes(L.kind, n->C);
+    }
+    mrcm::k_tc_pack<<<dim3(32, n->layers), 256, 0, st>>>(pk, p.wb, w.pack_f);
+    tc_launch(n, net, st);
+}
+
+// Gradients of every layer's pre-activation from the output's (g_out, one
+// channel) into w.g at the layers' activation offsets, one launch.
+void backward_data_tc(const mrcm_net* n, const NetPtrs& p, const float* g_out, int batch, const float* acts, void* ws,
+                      cudaStream_t st) {
+    const TcWs w = tc_ws(n, ws, batch);
+    mrcm::TcPack pk;
+    mrcm::TcNet net;
+    pk.layers = net.layers = n->layers - 1;
+    pk.C = n->C;
+    pk.flip = 1;
+    net.D = n->D; net.H = n->H; net.W = n->W; net.batch = batch; net.x = g_out; net.wpack = w.pack_b;
+    uint32_t off = 0;
+    for (int i = 0; i + 1 < n->layers; ++i) {
+        const int l = n->layers - 1 - i;                 // this network layer's transposed convolution
+        mrcm::TcLayer& L = net.l[i];
+        L.kind = i == 0 ? mrcm::kTcFirst : mrcm::kTcHidden;
+        L.cin = n->cout[l]; L.cout = n->cin[l]; L.w_off = off;
+        L.bias = nullptr;
+        L.mask = acts + (long long)batch * n->act_off[l - 1];
+        L.out = w.g + (long long)batch * n->act_off[l - 1];
+        L.leaky = 0;
+        L.last = l == 1 ? 1 : 0;
+        pk.kind[i] = L.kind; pk.cin[i] = L.cin; pk.cout[i] = L.cout; pk.w[i] = n->w_off[l]; pk.off[i] = off;
+        off += mrcm::tc_weight_bytes(L.kind, n->C);
+    }
+    mrcm::k_tc_pack<<<dim3(32, n->layers - 1), 256, 0, st>>>(pk, p.wb, w.pack_b);
+    tc_launch(n, net, st);
+}
+
+template <int MT, int NT>
+void wgrad_launch(const mrcm_net* n, int zc, int batch, int ci, int co, const float* g, const float* in, float* part,
+                  int grid, cudaStream_t st) {
+    mrcm::k_tc_wgrad<MT, NT><<<grid, mrcm::kWgThreads, mrcm::wg_smem(n->H, n->W, zc, MT, NT), st>>>(
+        n->D, n->H, n->W, zc, batch, ci, co, g, in, part);
+}
+
+// Slices per work item: the rounds of the persistent grid against the halo each item stages again.
+int wgrad_slices(const mrcm_net* n, int batch, int zmax) {
+    int zc = 1;
+    double best = 1e30;
+    for (int z = 1; z <= zmax; ++z) {
+        const int items = batch * ((n->D + z - 1) / z), rounds = (items + kWgCtas - 1) / kWgCtas;
+        const double cost = rounds * (z + 0.25 * (z + 2));
+        if (cost < best) { best = cost; zc = z; }
+    }
+    return zc;
+}
+
+// Weight gradients of one layer as partial sums of up to kWgCtas CTAs (the count is returned).
+int wgrad_tc(const mrcm_net* n, int l, int batch, const float* g, const float* in, float* part, cudaStream_t st) {
+    const int ci = n->cin[l], co = n->cout[l], HW = n->H * n->W;
+    if (co == 1) {                                       // taps as rows of the one-channel operand
+        const int nt = ci > 16 ? 4 : 2;
+        int zmax = 0;
+        for (int z = 1; z <= n->D; ++z)
+            if (mrcm::im_smem(HW, z, 2, nt) <= mrcm::kTcSmemMax) zmax = z;
+        if (zmax > 0) {
+            const int zc = wgrad_slices(n, batch, zmax), grid = std::min(kWgCtas, batch * ((n->D + zc - 1) / zc));
+            const uint32_t sm = mrcm::im_smem(HW, zc, 2, nt);
+            if (nt == 4) mrcm::k_tc_wgrad_out<4><<<grid, mrcm::kImThreads, sm, st>>>(n->D, n->H, n->W, zc, batch, ci, g, in, part);
+            else mrcm::k_tc_wgrad_out<2><<<grid, mrcm::kImThreads, sm, st>>>(n->D, n->H, n->W, zc, batch, ci, g, in, part);
+            return grid;
+        }
+    }
+    const int MT = co > 16 ? 2 : 1, NT = ci > 16 ? 4 : ci > 8 ? 2 : 1;
+    const int zc = wgrad_slices(n, batch, n->wg_zc_max);
+    const int grid = std::min(kWgCtas, batch * ((n->D + zc - 1) / zc));
+    if (MT == 2 && NT == 4) wgrad_launch<2, 4>(n, zc, batch, ci, co, g, in, part, grid, st);
+    else if (MT == 2 && NT == 2) wgrad_launch<2, 2>(n, zc, batch, ci, co, g, in, part, grid, st);
+    else if (MT == 2) wgrad_launch<2, 1>(n, zc, batch, ci, co, g, in, part, grid, st);
+    else if (NT == 4) wgrad_launch<1, 4>(n, zc, batch, ci, co, g, in, part, grid, st);
+    else if (NT == 2) wgrad_launch<1, 2>(n, zc, batch, ci, co, g, in, part, grid, st);
+    else wgrad_launch<1, 1>(n, zc, batch, ci, co, g, in, part, grid, st);
+    return grid;
 }
 
 void forward(const mrcm_net* n, const NetPtrs& p, const float* x, int batch, float* acts, cudaStream_t st) {
@@ -431,10 +579,7 @@ void forward(const mrcm_net* n, const NetPtrs& p, const float* x, int batch, flo
         float* out = acts + (long long)batch * n->act_off[l];
         const int mode = l + 1 == n->layers ? 1 : 0;
         if (n->cin[l] == mrcm::kMmaCh && n->cout[l] == mrcm::kMmaCh && n->mma_ok) {
-            int dev = 0, sms = 1;
-            cudaGetDevice(&dev);
-            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-            mrcm::k_conv_forward_mma<<<std::max(1, std::min(batch, sms)), mrcm::kMmaThreads, mrcm::conv_mma_smem(sh), st>>>(
+            mrcm::k_conv_forward_mma<<<std::max(1, std::min(batch, sm_count())), mrcm::kMmaThreads, mrcm::conv_mma_smem(sh), st>>>(
                 sh, batch, p.wb + n->w_off[l], p.w + n->b_off[l], in, out, mode);
         } else {
             const size_t sm = mrcm::conv_smem(n->cin[l], n->cout[l], n->S);
@@ -449,9 +594,16 @@ void forward(const mrcm_net* n, const NetPtrs& p, const float* x, int batch, flo
     }
 }
 
+// Forward pass of a training step: every activation kept at its place in the workspace.
+void forward_train(const mrcm_net* n, const NetPtrs& p, const float* x, int batch, void* ws, cudaStream_t st) {
+    float* acts = (float*)ws;
+    if (n->tc_ok) forward_tc(n, p, x, batch, acts, acts + (long long)batch * n->act_off[n->layers - 1], true, ws, st);
+    else forward(n, p, x, batch, acts, st);
+}
+
 // loss and gradient of the parameters into `grad` (P floats)
 void backward(const mrcm_net* n, const NetPtrs& p, const float* x, const float* target, const float* weight,
-              int batch, float* acts, float* gbuf0, float* gbuf1, float* grad, float* partial, float* loss,
+              int batch, float* acts, float* gbuf0, float* gbuf1, float* grad, float* partial, float* loss, void* ws,
               cudaStream_t st) {
     ConvShape sh{n->D, n->H, n->W, n->S};
     const int L = n->layers;
@@ -460,8 +612,33 @@ void backward(const mrcm_net* n, const NetPtrs& p, const float* x, const float* 
     const int nb = 128;
     mrcm::k_mse_loss<<<nb, mrcm::kNetThreads, 0, st>>>(nout, y, target, weight, gbuf0, partial);
     mrcm::k_sum_partials<<<1, 32, 0, st>>>(nout, nb, partial, loss);
-    float* g = gbuf0;
+    const float* g = gbuf0;
     float* gnext = gbuf1;
+    if (n->tc_ok) {                       // (its slabs fit whenever the fused pass does)
+        const TcWs w = tc_ws(n, ws, batch);
+        backward_data_tc(n, p, gbuf0, batch, acts, ws, st);
+        mrcm::TcSum sum;
+        mrcm::TcOffs goff;
+        sum.layers = L;
+        sum.batch = batch;
+        long long off = 0, blocks = 0;
+        for (int l = 0; l < L; ++l) {
+            const long long cnt = 27LL * n->cin[l] * n->cout[l];
+            sum.cin[l] = n->cin[l]; sum.cout[l] = n->cout[l];
+            sum.w_off[l] = n->w_off[l]; sum.b_off[l] = n->b_off[l];
+            goff.o[l] = (long long)batch * n->act_off[l];
+            sum.part[l] = off;
+            sum.parts[l] = wgrad_tc(n, l, batch, l + 1 == L ? gbuf0 : w.g + goff.o[l],
+                                    l == 0 ? x : acts + (long long)batch * n->act_off[l - 1], w.part + off, st);
+            off += kWgCtas * cnt;
+            sum.bpart[l] = off;
+            off += (long long)batch * n->cout[l];
+            blocks += (cnt + n->cout[l] + 31) / 32;
+        }
+        mrcm::k_tc_bias<<<dim3(152, L), 256, 0, st>>>(sum, n->S, gbuf0, w.g, goff, w.part);
+        mrcm::k_tc_sum<<<(int)blocks, 256, 0, st>>>(sum, w.part, w.part, grad);
+        return;
+    }
     for (int l = L - 1; l >= 0; --l) {
         const float* in = l == 0 ? x : acts + (long long)batch * n->act_off[l - 1];
         mrcm::k_conv_backward_weights<<<n->cout[l] * n->cin[l], mrcm::kNetThreads, 0, st>>>(
@@ -470,7 +647,8 @@ void backward(const mrcm_net* n, const NetPtrs& p, const float* x, const float* 
             const size_t sm = mrcm::conv_smem(n->cout[l], n->cin[l], n->S);
             mrcm::k_conv_backward_data<<<batch, mrcm::kNetThreads, sm, st>>>(sh, n->cin[l], n->cout[l],
                                                                            p.wb + n->w_off[l], g, in, gnext, 1);
-            float* t = g; g = gnext; gnext = t;
+            g = gnext;
+            gnext = gnext == gbuf1 ? gbuf0 : gbuf1;
         }
     }
 }
@@ -512,6 +690,22 @@ mrcm_status mrcm_net_create(int in_channels, int hidden, int layers, int D, int 
         cudaGetLastError();
     }
     cudaFuncSetAttribute(mrcm::k_conv_backward_data, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    {
+        const mrcm::TcGeo g(D, H, W);
+        n->C = hidden > 16 ? 32 : 16;
+        const size_t smt = mrcm::tc_plane_bytes(g, n->C) + mrcm::tc_wregion_bytes(g, n->C);
+        n->tc_ok = in_channels <= 8 && 3 * n->C * g.tiles <= 512 && smt <= mrcm::kTcSmemMax;
+        for (int z = 1; z <= D; ++z)
+            if (mrcm::wg_smem(H, W, z, 2, 4) <= mrcm::kTcSmemMax) n->wg_zc_max = z;
+        if (n->wg_zc_max == 0) n->tc_ok = false;
+        const void* tk[] = {(const void*)mrcm::k_tc_net<16>, (const void*)mrcm::k_tc_net<32>,
+                            (const void*)mrcm::k_tc_wgrad<2, 4>, (const void*)mrcm::k_tc_wgrad<2, 2>, (const void*)mrcm::k_tc_wgrad<2, 1>,
+                            (const void*)mrcm::k_tc_wgrad<1, 4>, (const void*)mrcm::k_tc_wgrad<1, 2>, (const void*)mrcm::k_tc_wgrad<1, 1>,
+                            (const void*)mrcm::k_tc_wgrad_out<4>, (const void*)mrcm::k_tc_wgrad_out<2>};
+        for (const void* k : tk)
+            if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)mrcm::kTcSmemMax) != cudaSuccess) n->tc_ok = false;
+        cudaGetLastError();
+    }
     *out = n;
     return MRCM_OK;
 }
@@ -566,6 +760,10 @@ mrcm_status mrcm_net_forward(mrcm_net* n, const float* state, const float* x, fl
     cudaStream_t st = (cudaStream_t)stream;
     NetPtrs p = net_ptrs(n, state);
     float* acts = (float*)ws;
+    if (n->tc_ok) {
+        forward_tc(n, p, x, batch, acts, y, false, ws, st);
+        return cudaGetLastError() == cudaSuccess ? MRCM_OK : MRCM_ERR_CUDA;
+    }
     forward(n, p, x, batch, acts, st);
     cudaMemcpyAsync(y, acts + (long long)batch * n->act_off[n->layers - 1], sizeof(float) * batch * n->S,
                     cudaMemcpyDeviceToDevice, st);
@@ -588,8 +786,8 @@ mrcm_status mrcm_net_gradient(mrcm_net* n, const float* state, const float* x, c
     NetPtrs p = net_ptrs(n, state);
     float *g0, *g1, *partial;
     ws_grad(n, ws, batch, &g0, &g1, &partial);
-    forward(n, p, x, batch, (float*)ws, st);
-    backward(n, p, x, target, weight, batch, (float*)ws, g0, g1, grad, partial, loss, st);
+    forward_train(n, p, x, batch, ws, st);
+    backward(n, p, x, target, weight, batch, (float*)ws, g0, g1, grad, partial, loss, ws, st);
     return cudaGetLastError() == cudaSuccess ? MRCM_OK : MRCM_ERR_CUDA;
 }
 
@@ -601,8 +799,8 @@ mrcm_status mrcm_net_train_step(mrcm_net* n, float* state, const float* x, const
     NetPtrs p = net_ptrs(n, state);
     float *g0, *g1, *partial;
     float* grad = ws_grad(n, ws, batch, &g0, &g1, &partial);
-    forward(n, p, x, batch, (float*)ws, st);
-    backward(n, p, x, target, weight, batch, (float*)ws, g0, g1, grad, partial, loss, st);
+    forward_train(n, p, x, batch, ws, st);
+    backward(n, p, x, target, weight, batch, (float*)ws, g0, g1, grad, partial, loss, ws, st);
     const float b1 = 0.9f, b2 = 0.999f;
     const float c1 = 1.0f - std::pow(b1, (float)step), c2 = 1.0f - std::pow(b2, (float)step);
     mrcm::k_adam<<<128, 256, 0, st>>>(n->P, p.w, p.m, p.v, grad, p.wb, lr, b1, b2, 1e-8f, c1, c2);

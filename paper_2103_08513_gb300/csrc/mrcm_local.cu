@@ -170,124 +170,35 @@ k_coefficients(const SubInfo* __restrict__ subs, const FaceInfo* __restrict__ fa
 
 // ---------------------------------------------------------------------------
 // Slab block factorisation: W_s = S_s^{-1} by in-place Gauss-Jordan on the
-// SPD block pivot (no pivoting needed for SPD), one CTA per subdomain.
+// SPD block pivot (no pivoting needed for SPD).
 //
 // Gauss-Jordan on a symmetric matrix keeps M[i][j] = sigma_i sigma_j M[j][i]
 // with sigma = -1 on the indices already pivoted (the "sweep operator"), so
-// only the lower triangle is stored (packed, row i at i(i+1)/2) and updated:
-// step k, with r_j = M[k][j] read from the lower triangle and
-// c_i = M[i][k] = sigma_i r_i,
+// only the lower triangle has to be held and updated: step k, with
+// r_j = M[k][j] and c_i = M[i][k] = sigma_i r_i,
 //   M[i][j] -= c_i r_j / p  (i, j != k),  M[k][j] = r_j / p,
 //   M[i][k] = -c_i / p,  M[k][k] = 1 / p.
 // After the last pivot every sigma is -1 and the triangle holds S_s^{-1}.
 // W_s is written to global memory as a full b x b matrix.
 // ---------------------------------------------------------------------------
-__host__ __device__ inline size_t packed_len(int b) { return (size_t)b * (b + 1) / 2; }
 
-template <typename T, bool kScaled>
-__global__ void __launch_bounds__(kThreads)
-k_block_factor(const SubInfo* __restrict__ subs, const int* __restrict__ list, const double* __restrict__ coef,
-               const double* __restrict__ scale, T* __restrict__ Wall, int* __restrict__ status,
-               long long nct, float* __restrict__ scf_all, float* __restrict__ tsc_all,
-               const int* __restrict__ limit /* CTAs from *limit on have no subdomain; may be NULL */,
-               T* __restrict__ big /* packed triangles of the blocks with a global slot; may be NULL */) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    if (limit && (int)blockIdx.x >= *limit) return;
-    const SubInfo s = subs[list[blockIdx.x]];
-    const int b = s.b, su = s.su;
-    T* rk = reinterpret_cast<T*>(smem_raw);                    // row k
-    T* tv = rk + b;                                            // scaled couplings to the previous slab
-    // packed lower triangle: shared memory, or the subdomain's global slot (L2-resident) when it is too large
-    T* Lp = (big && s.big_slot >= 0) ? big + (size_t)s.big_slot * packed_len(kMaxBlock)
-                                     : tv + ((b + 1) & ~1);
-    const double* cd = coef + s.cell_off;
-    const double* cu = coef + nct + s.cell_off;
-    const double* cv = coef + 2 * nct + s.cell_off;
-    const double* cs = coef + 3 * nct + s.cell_off;
-    const double* sc = scale + s.cell_off;
-    T* W = Wall + s.w_off;
-    const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;    // 32 x 8 threads
-    int bad = 0;
-    for (int i = threadIdx.x; i < (int)packed_len(b); i += blockDim.x) Lp[i] = (T)0;
-    for (int sl = 0; sl < s.ns; ++sl) {
-        const int base = sl * b;
-        for (int i = threadIdx.x; i < b; i += blockDim.x) {
-            const int c = base + i;
-            double t = 0.0;
-            if (sl > 0) t = cs[c - b] * (kScaled ? sc[c - b] * sc[c] : 1.0);
-            tv[i] = (T)t;
-            if (kScaled) {
-                scf_all[s.cell_off + c] = (float)sc[c];
-                tsc_all[s.cell_off + c] = sl + 1 < s.ns ? (float)(cs[c] * sc[c] * sc[c + b]) : 0.0f;
-            }
-        }
-        __syncthreads();
-        // S_s = D_s - t o W_{s-1} o t on the lower triangle
-        for (int i = ty; i < b; i += 8) {
-            const int ci = base + i;
-            const int ui = i % su;
-            const double si = kScaled ? sc[ci] : 1.0;
-            T* row = Lp + packed_len(i);
-            for (int j = tx; j <= i; j += 32) {
-                const int cj = base + j;
-                double dij = 0.0;
-                if (i == j) dij = cd[ci];
-                if (i == j + 1 && ui > 0) dij = -cu[cj];
-                if (i == j + su) dij = -cv[cj];
-                if (kScaled) dij *= si * sc[cj];
-                row[j] = (T)(dij - (double)tv[i] * (double)tv[j] * (double)row[j]);
-            }
-        }
-        __syncthreads();
-        // sweep operator on the packed triangle
-        for (int k = 0; k < b; ++k) {
-            for (int j = threadIdx.x; j < b; j += blockDim.x) rk[j] = j <= k ? Lp[packed_len(k) + j] : Lp[packed_len(j) + k];
-            __syncthreads();
-            T p = rk[k];
-            if (!(p > (T)0)) { bad = 1; p = (T)1; }
-            const T ip = (T)1 / p;
-            for (int i = ty; i < b; i += 8) {
-                const T ci = i < k ? -rk[i] : rk[i];
-                T* row = Lp + packed_len(i);
-                for (int j = tx; j <= i; j += 32) {
-                    T v;
-                    if (i == k) v = j == k ? ip : rk[j] * ip;
-                    else if (j == k) v = -ci * ip;
-                    else v = row[j] - ci * rk[j] * ip;
-                    row[j] = v;
-                }
-            }
-            __syncthreads();
-        }
-        // W_s as a full matrix (both triangles)
-        T* Ws = W + (long long)sl * wstride<T>(b);
-        for (int i = ty; i < b; i += 8) {
-            const T* row = Lp + packed_len(i);
-            for (int j = tx; j <= i; j += 32) {
-                Ws[(long long)i * b + j] = row[j];
-                Ws[(long long)j * b + i] = row[j];
-            }
-        }
-        __syncthreads();
-    }
-    if (bad && threadIdx.x == 0) atomicAdd(&status[ST_NOT_SPD], 1);
-}
-
-// FP64 form, b <= 128: the block as 4 x 4 register tiles of its lower triangle
-// (mrcm_sweep64.cuh), one CTA of NTH threads per subdomain; W_{s-1} stays in
-// the registers to form S_s.  Larger blocks keep k_block_factor: from b = 129
-// on the tiles (16 doubles a thread) no longer fit one CTA's registers.
-template <int NTH>
+// FP64 form: the block as 4 x 4 register tiles of its lower triangle
+// (mrcm_sweep64.cuh), one CTA of NTH threads per subdomain up to b = 128, a cluster
+// of CL CTAs above (16 doubles a thread no longer fit one SM's registers there);
+// W_{s-1} stays in the registers to form S_s.
+template <int NTH, int CL>
 __global__ void __launch_bounds__(NTH)
 k_block_factor64(const SubInfo* __restrict__ subs, const int* __restrict__ list, const double* __restrict__ coef,
                  double* __restrict__ Wall, int* __restrict__ status, long long nct,
-                 const int* __restrict__ limit /* CTAs from *limit on have no subdomain; may be NULL */) {
-    if (limit && (int)blockIdx.x >= *limit) return;
-    const SubInfo s = subs[list[blockIdx.x]];
+                 const int* __restrict__ limit /* only the first *limit subdomains of the list; may be NULL */) {
+    const int item = (int)blockIdx.x / CL, rank = (int)blockIdx.x % CL;
+    if (limit && item >= *limit) return;
+    const SubInfo s = subs[list[item]];
     const int b = s.b, su = s.su;
     const int nt = (b + kSw64T - 1) / kSw64T;
+    constexpr int B = CL == 1 ? kSw64B : kSw64BC;
     int ti, tj;
-    sweep64_tile(threadIdx.x, ti, tj);
+    sweep64_tile((int)threadIdx.x * CL + rank, ti, tj);
     const bool own = ti < nt && threadIdx.x + 32 < NTH;  // the last warp forms the pivots
     if (!own) ti = tj = 0;                              // idle threads shadow tile (0, 0), never publish or store
     const int i0 = ti * kSw64T, j0 = tj * kSw64T;
@@ -295,8 +206,8 @@ k_block_factor64(const SubInfo* __restrict__ subs, const int* __restrict__ list,
     const double* cu = coef + nct + s.cell_off;
     const double* cv = coef + 2 * nct + s.cell_off;
     const double* cs = coef + 3 * nct + s.cell_off;
-    __shared__ __align__(16) Sweep64Shared sh;
-    __shared__ double sd[kSw64B], sup[kSw64B], svp[kSw64B], st[kSw64B];
+    __shared__ __align__(16) Sweep64Shared<CL> sh;
+    __shared__ double sd[B], sup[B], svp[B], st[B];
     if (threadIdx.x == 0) sh.bad = 0;
     double a[kSw64T][kSw64T];
 #pragma unroll
@@ -305,8 +216,8 @@ k_block_factor64(const SubInfo* __restrict__ subs, const int* __restrict__ list,
         for (int c = 0; c < kSw64T; ++c) a[r][c] = 0.0;
     for (int sl = 0; sl < s.ns; ++sl) {
         const int base = sl * b;
-        __syncthreads();                                // the previous slab's last step is done with `sh`
-        for (int i = threadIdx.x; i < kSw64B; i += NTH) {
+        sweep64_barrier<CL>();                          // the previous slab's last step is done with `sh`
+        for (int i = threadIdx.x; i < B; i += NTH) {
             double d = 0.0, u = 0.0, v = 0.0, t = 0.0;
             if (i < b) {
                 const int c = base + i;
@@ -334,15 +245,12 @@ k_block_factor64(const SubInfo* __restrict__ subs, const int* __restrict__ list,
                 a[r][c] = (i < b && j < b) ? fma(-st[i] * st[j], a[r][c], dij) : 0.0;
             }
         }
-        sweep64_invert(a, ti, tj, own, b, sh);
+        sweep64_invert<CL>(a, ti, tj, own, b, sh);
         sweep64_store(a, ti, tj, own, b, Wall + s.w_off + (long long)sl * wstride<double>(b));
     }
-    __syncthreads();
-    if (threadIdx.x == 0 && sh.bad) atomicAdd(&status[ST_NOT_SPD], 1);
+    sweep64_barrier<CL>();                              // (every CTA of a cluster has formed the same pivots)
+    if (threadIdx.x == 0 && rank == 0 && sh.bad) atomicAdd(&status[ST_NOT_SPD], 1);
 }
-
-template <typename T>
-size_t factor_smem(int b) { return sizeof(T) * (packed_len(b) + 2 * (size_t)b + 4); }
 
 // ---------------------------------------------------------------------------
 // Register-resident variant of the block factorisation for b <= 64 (FP32,
@@ -788,10 +696,10 @@ k_block_factor_tc(const SubInfo* __restrict__ subs, const int* __restrict__ list
 constexpr int kTriB = 256;                 // largest block
 
 // CTA size of the triangle factor for a b x b block: whole warps covering the
-// nt (nt + 1) / 2 tiles; 0 = beyond kTriB (packed kernel)
+// nt (nt + 1) / 2 tiles
 static int tri_threads(int b) {
     const int nt = (b + 7) / 8, T = nt * (nt + 1) / 2;
-    return b > kTriB ? 0 : T <= 192 ? 192 : T <= 320 ? 320 : T <= 512 ? 512 : 544;
+    return T <= 192 ? 192 : T <= 320 ? 320 : T <= 512 ? 512 : 544;
 }
 
 // NTH threads: 192 cover b <= 144, 320 b <= 192, 512 b <= 248 (496 tiles),
@@ -2147,24 +2055,30 @@ Geo make_geo(const mrcm_config& c) {
 
 }  // namespace
 
-// Block factors of one wave's subdomains (register-resident FP32 kernel for
-// b <= 64, packed shared-memory kernel otherwise; one launch per class).
+// Block factors of one wave's subdomains (one launch per class and CTA size).
 int num_solve_variants() { return kNumSolveVariants; }
 
 // FP64 block factors of n listed subdomains whose blocks are at most bmax
-// (limit: see the kernels; big: packed triangles of blocks above kMaxBlock64, or NULL).
-static void launch_factor64(const SubInfo* subs, const int* list, int n, int bmax, const double* coef,
-                            const double* scale, double* W, int* status, long long nct, const int* limit, double* big,
-                            const char* name, cudaStream_t st, Prof& P) {
-    switch (sweep64_threads(bmax)) {
-    case 128: MRCM_LAUNCH(P, name, st, k_block_factor64<128><<<n, 128, 0, st>>>(subs, list, coef, W, status, nct, limit)); break;
-    case 192: MRCM_LAUNCH(P, name, st, k_block_factor64<192><<<n, 192, 0, st>>>(subs, list, coef, W, status, nct, limit)); break;
-    case 352: MRCM_LAUNCH(P, name, st, k_block_factor64<352><<<n, 352, 0, st>>>(subs, list, coef, W, status, nct, limit)); break;
-    case 576: MRCM_LAUNCH(P, name, st, k_block_factor64<576><<<n, 576, 0, st>>>(subs, list, coef, W, status, nct, limit)); break;
-    default:
-        MRCM_LAUNCH(P, name, st, k_block_factor<double, false><<<n, kThreads, factor_smem<double>(std::min(bmax, kMaxBlock64)), st>>>(
-                    subs, list, coef, scale, W, status, nct, nullptr, nullptr, limit, big));
-    }
+// (limit: only the first *limit of them, read on the device, or NULL).
+static void launch_factor64(const SubInfo* subs, const int* list, int n, int bmax, const double* coef, double* W,
+                            int* status, long long nct, const int* limit, const char* name, cudaStream_t st, Prof& P) {
+    const int nth = sweep64_threads(bmax), cl = bmax > kSw64B ? kSw64Cl : 1;
+    const void* k = cl > 1 ? (nth == 160 ? (const void*)k_block_factor64<160, kSw64Cl> : (const void*)k_block_factor64<320, kSw64Cl>)
+                  : nth == 128 ? (const void*)k_block_factor64<128, 1> : nth == 192 ? (const void*)k_block_factor64<192, 1>
+                  : nth == 352 ? (const void*)k_block_factor64<352, 1> : (const void*)k_block_factor64<576, 1>;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(n * cl);
+    cfg.blockDim = dim3(nth);
+    cfg.stream = st;
+    cudaLaunchAttribute at[1];
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = cl;
+    at[0].val.clusterDim.y = 1;
+    at[0].val.clusterDim.z = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = cl > 1 ? 1 : 0;
+    void* args[] = {(void*)&subs, (void*)&list, (void*)&coef, (void*)&W, (void*)&status, (void*)&nct, (void*)&limit};
+    MRCM_LAUNCH(P, name, st, cudaLaunchKernelExC(&cfg, k, args));
 }
 
 static void launch_factor_wave(const Tables& t, const DeviceTables& d, const Layout& L, char* ws, int precision,
@@ -2182,8 +2096,8 @@ static void launch_factor_wave(const Tables& t, const DeviceTables& d, const Lay
             const int b0 = t.subs[t.class_list[q]].b, nth = sweep64_threads(b0);
             int e = q + 1;
             while (e < o3 && sweep64_threads(t.subs[t.class_list[e]].b) == nth) ++e;
-            launch_factor64(d.subs, d.class_list + q, e - q, b0, coef, scale, (double*)(ws + L.W), status, t.n_cells, nullptr,
-                            (double*)(ws + L.big), "k_block_factor", st, P);
+            launch_factor64(d.subs, d.class_list + q, e - q, b0, coef, (double*)(ws + L.W), status, t.n_cells, nullptr,
+                            "k_block_factor", st, P);
             q = e;
         }
     } else {
@@ -2207,7 +2121,7 @@ static void launch_factor_wave(const Tables& t, const DeviceTables& d, const Lay
                     (float*)(ws + L.W), status, t.n_cells, (float*)(ws + L.scf), (float*)(ws + L.tsc)));
         }
         // the large class is ordered by b, largest first: one launch per run of
-        // subdomains that share a thread count (packed kernel above kTriB)
+        // subdomains that share a thread count
         for (int q = o2; q < o3;) {
             const int nth = tri_threads(t.subs[t.class_list[q]].b);
             int e = q + 1;
@@ -2222,10 +2136,6 @@ static void launch_factor_wave(const Tables& t, const DeviceTables& d, const Lay
             case 320: MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_tri<320><<<n, 320, 0, st>>>(d.subs, lst, coef, scale, W, status, t.n_cells, scf, tsc)); break;
             case 512: MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_tri<512><<<n, 512, 0, st>>>(d.subs, lst, coef, scale, W, status, t.n_cells, scf, tsc)); break;
             case 544: MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_tri<544><<<n, 544, 0, st>>>(d.subs, lst, coef, scale, W, status, t.n_cells, scf, tsc)); break;
-            default: {
-                size_t sm = factor_smem<float>(t.max_b);
-                MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor<float, true><<<n, kThreads, sm, st>>>(d.subs, lst, coef, scale, W, status, t.n_cells, scf, tsc, nullptr, nullptr));
-            }
             }
             q = e;
         }
@@ -2302,10 +2212,6 @@ int configure_local(const Tables& t, DeviceTables& d) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k1, variant_threads(0), d.f64_solve_smem);
         d.f64_occ = std::max(1, occ);
     }
-    cudaFuncSetAttribute(k_block_factor<double, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)factor_smem<double>(std::min(t.max_b, kMaxBlock64)));
-    cudaFuncSetAttribute(k_block_factor<float, true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)factor_smem<float>(t.max_b));
     cudaFuncSetAttribute(k_block_factor_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
     return (int)cudaGetLastError();
 }
@@ -2364,8 +2270,8 @@ static void launch_fallback(const Tables& t, const DeviceTables& d, const Layout
                 g0.conv, status, fb_subs, fb_list, cap, wstride_slot, ystride_slot));
     int bmax = 0;
     for (const SubInfo& s : t.subs) if (s.b <= kMaxBlock64) bmax = std::max(bmax, s.b);
-    launch_factor64(fb_subs, fb_list, cap, bmax, g0.coef, g0.scale, (double*)(ws + L.fb_W), status, t.n_cells,
-                    status + ST_FB_WAVE, nullptr, "k_fb_factor", st, P);
+    launch_factor64(fb_subs, fb_list, cap, bmax, g0.coef, (double*)(ws + L.fb_W), status, t.n_cells, status + ST_FB_WAVE,
+                    "k_fb_factor", st, P);
     LocalArgs g = g0;
     g.subs = fb_subs;
     g.list = fb_list;
@@ -2513,8 +2419,7 @@ int launch_postprocess(const Tables& t, const DeviceTables& d, const Layout& L, 
             MRCM_LAUNCH(P, "k_set_int", st, k_set_int<<<1, 1, 0, st>>>(cnt, 0));
             MRCM_LAUNCH(P, "k_pp_unconverged", st, k_pp_unconverged<<<(n + 127) / 128, 128, 0, st>>>(d.subs,
                         d.solve_list + t.pp_wave_off[w], n, g.conv, plist, cnt, status + ST_FB_TOTAL));
-            launch_factor64(d.pp_subs, plist, n, bmax, coef, (const double*)(ws + L.scale), (double*)(ws + L.W), status,
-                            t.n_cells, cnt, nullptr, "k_pp_factor", st, P);
+            launch_factor64(d.pp_subs, plist, n, bmax, coef, (double*)(ws + L.W), status, t.n_cells, cnt, "k_pp_factor", st, P);
             const int grid = std::max(1, std::min(n, d.sms * d.f64_occ));
             void* args[] = {(void*)&g, (void*)&W};
             g.count_unconverged = 0;

@@ -79,7 +79,7 @@ k_box_solve_noalloc(BoxArgs a, const double* __restrict__ K, const double* __res
                     const double* __restrict__ g, const double* __restrict__ beta, double* __restrict__ p,
                     double* __restrict__ q, double* scratch, int* __restrict__ not_spd) {
     using namespace mrcm;
-    __shared__ __align__(16) Sweep64Shared sh;
+    __shared__ __align__(16) Sweep64Shared<1> sh;
     __shared__ double z[kNaMaxBlock], tv[kNaMaxBlock], tw[kNaMaxBlock];
     __shared__ double part[NTH];
     __shared__ int other_bad;
@@ -206,7 +206,7 @@ k_box_solve_noalloc(BoxArgs a, const double* __restrict__ K, const double* __res
                 m[r][c] = fma(-tv[i] * tv[j], m[r][c], dij);
             }
         }
-        sweep64_invert(m, ti, tj, own, b, sh);
+        sweep64_invert<1>(m, ti, tj, own, b, sh);
         sweep64_store(m, ti, tj, own, b, W + (long long)sl * b * b);
         __syncthreads();
         gemv(sl, [&](int i, double v) { y[base + i] = v; });

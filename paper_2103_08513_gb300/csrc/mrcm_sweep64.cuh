@@ -2,7 +2,8 @@
 // batched factor kernel and the allocation-free box solve.
 //
 // The block is held as 4 x 4 tiles of its lower triangle, one tile per thread
-// (b <= 128: at most 528 tiles), and swept by the sign-symmetric Gauss-Jordan
+// (b <= 128: at most 528 tiles in one CTA; up to 256: at most 2080 tiles over a
+// cluster of eight), and swept by the sign-symmetric Gauss-Jordan
 // step M[i][j] -= M[i][k] M[k][j] / p (M[i][k] = sigma_i M[k][i], sigma = -1 on
 // pivoted indices).
 //
@@ -18,6 +19,9 @@
 // diagonal tile's thread doing it after its updates, 376 us with the warp, 318 us
 // once no sign was flipped by an FP64 instruction).  2244 blocks of 10 slabs,
 // b = 50: 19.3 ms with the packed triangle, 4.5 ms now.
+// Blocks above 128 (the tiles no longer fit one SM's registers) are spread over a
+// cluster of eight CTAs, tile t on CTA t mod 8; the pivot row goes into every
+// CTA's shared memory and the step's barrier is the cluster's.  @CL@
 // 8 x 8 tiles would scale less (72 instead of 80 per 64 entries) but waste more
 // on the diagonal and leave one warp per block of 50.
 #pragma once
@@ -27,14 +31,17 @@
 
 namespace mrcm {
 
-constexpr int kSw64B = 128;        // largest block
+constexpr int kSw64B = 128;        // largest block of one CTA
+constexpr int kSw64BC = 256;       // largest block of a cluster
+constexpr int kSw64Cl = 8;         // CTAs of a cluster
 constexpr int kSw64T = 4;          // tile edge
 
-// Threads: whole warps that hold a b x b block, one tile each, and the pivot
-// warp (the last one); 0 = too large.
+// Threads per CTA: whole warps that hold a b x b block (or a cluster's eighth of
+// it), one tile each, and the pivot warp (the last one).
 __host__ __device__ inline int sweep64_threads(int b) {
     const int nt = (b + kSw64T - 1) / kSw64T, T = nt * (nt + 1) / 2;
-    return b > kSw64B ? 0 : T <= 96 ? 128 : T <= 160 ? 192 : T <= 320 ? 352 : 576;
+    if (b > kSw64B) return T <= 128 * kSw64Cl ? 160 : 320;
+    return T <= 96 ? 128 : T <= 160 ? 192 : T <= 320 ? 352 : 576;
 }
 
 // Tile (ti >= tj) of thread t.
@@ -45,8 +52,9 @@ __device__ __forceinline__ void sweep64_tile(int t, int& ti, int& tj) {
     tj = t - ti * (ti + 1) / 2;
 }
 
+template <int CL>
 struct Sweep64Shared {
-    double prow[2][kSw64B];        // the pivot row, double-buffered: one barrier per pivot
+    double prow[2][CL == 1 ? kSw64B : kSw64BC];        // the pivot row, double-buffered: one barrier per pivot
     double pinv[2];                // 1 / p of the step
     double dnext[2];               // the next pivot's entry before the step's update
     int bad;                       // a pivot was not positive (replaced by 1)
@@ -60,17 +68,48 @@ __device__ __forceinline__ double sweep64_pivot(double p, int* bad) {
     return rcp64c(p);
 }
 
+template <int CL>
+__device__ __forceinline__ void sweep64_barrier() {
+    if constexpr (CL == 1) __syncthreads();
+    else asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+}
+// *dst = v (and dst[1] = w) here, or at the same place in every CTA of the cluster
+template <int CL>
+__device__ __forceinline__ void sweep64_put(double* dst, double v) {
+    if constexpr (CL == 1) { *dst = v; return; }
+    const unsigned la = (unsigned)__cvta_generic_to_shared(dst);
+#pragma unroll
+    for (int t = 0; t < CL; ++t) {
+        unsigned ra;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(la), "r"(t));
+        asm volatile("st.shared::cluster.f64 [%0], %1;" :: "r"(ra), "d"(v) : "memory");
+    }
+}
+template <int CL>
+__device__ __forceinline__ void sweep64_put2(double* dst, double v, double w) {
+    if constexpr (CL == 1) { *reinterpret_cast<double2*>(dst) = make_double2(v, w); return; }
+    const unsigned la = (unsigned)__cvta_generic_to_shared(dst);
+#pragma unroll
+    for (int t = 0; t < CL; ++t) {
+        unsigned ra;
+        asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(ra) : "r"(la), "r"(t));
+        asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" :: "r"(ra), "d"(v), "d"(w) : "memory");
+    }
+}
+
 // a <- inverse of the block whose lower-triangle tiles the threads hold
 // (diagonal tiles: both triangles; rows and columns past b are never pivoted).
-// Every thread of the CTA calls it; `own` marks the threads with a tile (not the
-// pivot warp's, the last of the CTA).  The last step's readers of `sh` are not
-// waited for.
+// Every thread of the CTA (cluster) calls it; `own` marks the threads with a tile
+// (not the pivot warp's, the last of each CTA).  The last step's readers of `sh`
+// are not waited for.
+template <int CL>
 __device__ __forceinline__ void sweep64_invert(double (&a)[kSw64T][kSw64T], int ti, int tj, bool own, int b,
-                                               Sweep64Shared& sh) {
+                                               Sweep64Shared<CL>& sh) {
     const int i0 = ti * kSw64T, j0 = tj * kSw64T;
     const int nt = (b + kSw64T - 1) / kSw64T;
     const bool pivot_warp = threadIdx.x + 32 >= blockDim.x;
-    if (own && ti == 0) sh.pinv[0] = sweep64_pivot(a[0][0], &sh.bad);
+    const bool idle_warp = !__any_sync(0xffffffffu, own);      // no tile: its FP64 instructions would cost all the same
+    if (own && ti == 0) sweep64_put<CL>(&sh.pinv[0], sweep64_pivot(a[0][0], &sh.bad));
 #pragma unroll 1
     for (int kt = 0; kt < nt; ++kt) {
         const bool rowt = own && ti == kt, colt = own && tj == kt;
@@ -80,16 +119,16 @@ __device__ __forceinline__ void sweep64_invert(double (&a)[kSw64T][kSw64T], int 
             if (k >= b) break;
             double* pr = sh.prow[kr & 1];
             if (rowt) {                                     // M[k][x], x in or left of the diagonal tile
-                reinterpret_cast<double2*>(pr + j0)[0] = make_double2(a[kr][0], a[kr][1]);
-                reinterpret_cast<double2*>(pr + j0)[1] = make_double2(a[kr][2], a[kr][3]);
+                sweep64_put2<CL>(pr + j0, a[kr][0], a[kr][1]);
+                sweep64_put2<CL>(pr + j0 + 2, a[kr][2], a[kr][3]);
             }
             if (colt && ti > kt) {                          // M[x][k] = M[k][x] below it
-                reinterpret_cast<double2*>(pr + i0)[0] = make_double2(a[0][kr], a[1][kr]);
-                reinterpret_cast<double2*>(pr + i0)[1] = make_double2(a[2][kr], a[3][kr]);
+                sweep64_put2<CL>(pr + i0, a[0][kr], a[1][kr]);
+                sweep64_put2<CL>(pr + i0 + 2, a[2][kr], a[3][kr]);
             }
             if (kr + 1 < kSw64T ? rowt && colt : own && ti == kt + 1 && tj == ti)
-                sh.dnext[kr & 1] = a[(kr + 1) & 3][(kr + 1) & 3];
-            __syncthreads();
+                sweep64_put<CL>(&sh.dnext[kr & 1], a[(kr + 1) & 3][(kr + 1) & 3]);
+            sweep64_barrier<CL>();
             const double ip = sh.pinv[kr & 1];
             if (pivot_warp) {                               // p_{k+1} as its tile forms it, and its reciprocal
                 if (k + 1 < b && (threadIdx.x & 31) == 0) {
@@ -98,6 +137,7 @@ __device__ __forceinline__ void sweep64_invert(double (&a)[kSw64T][kSw64T], int 
                 }
                 continue;
             }
+            if (idle_warp) continue;
             const double2 q0 = reinterpret_cast<const double2*>(pr + j0)[0], q1 = reinterpret_cast<const double2*>(pr + j0)[1];
             const double2 c0 = reinterpret_cast<const double2*>(pr + i0)[0], c1 = reinterpret_cast<const double2*>(pr + i0)[1];
             double rk[4] = {q0.x * ip, q0.y * ip, q1.x * ip, q1.y * ip};
