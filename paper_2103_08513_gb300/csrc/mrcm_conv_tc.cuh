@@ -30,7 +30,7 @@ namespace mrcm {
 constexpr int kTcMaxLayers = 16;
 constexpr int kTcThreads = 512;
 constexpr int kTcPairs = 5;             // the nine (dz, dy) shifts two by two (first layer)
-constexpr size_t kTcSmemMax = 227 * 1024 - 8192;
+constexpr size_t kTcSmemMax = 227 * 1024 - 9216;      // dynamic; the kernels' static part stays below 9 KB
 
 // Padded geometry of a D x H x W box.
 struct TcGeo {
@@ -62,8 +62,8 @@ struct TcGeo {
 // D_dx[v] = sum w(dz, dy, dx) x[v + shift(dz, dy)] and the output of voxel p is
 // D_-1[p - 1] + D_0[p] + D_+1[p + 1] (padding rows give 0).  Nine shifts instead
 // of 27 taps: an MMA reads its 128 x 16 A tile from shared memory whatever its N,
-// and with N = C = 32 that read bounded it (83 us per 5 x 10 x 10 sample and
-// network with one MMA per tap, @DX@ with three).
+// and with N = C = 32 that read bounded it (162 x 73 cycles per tile
+// and layer with one MMA per tap, 54 x 57 cycles with three).
 //
 // The first layer has at most 8 input channels: one 8-channel chunk per piece,
 // and an MMA (K = 16) takes two shifts, the second one as the second chunk at the
@@ -165,15 +165,19 @@ __device__ __forceinline__ void tcs_mma(uint32_t d, uint64_t a, uint64_t b, uint
                  " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}"
                  :: "r"(d), "l"(a), "l"(b), "r"(idesc), "r"(acc) : "memory");
 }
-__device__ __forceinline__ void tcs_ld16(uint32_t taddr, float* v) {
-    uint32_t r[16];
+// 16 accumulator columns of this lane's row; the values are valid after tcs_ld_wait
+__device__ __forceinline__ void tcs_ld16(uint32_t taddr, uint32_t (&r)[16]) {
     asm volatile("tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
                  : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
                    "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
                  : "r"(taddr));
-    asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-#pragma unroll
-    for (int q = 0; q < 16; ++q) v[q] = __uint_as_float(r[q]);
+}
+// (the registers pass through the wait, so that no use moves before it)
+__device__ __forceinline__ void tcs_ld_wait(uint32_t (&r)[16]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+                 :: "memory");
 }
 // three BF16 pieces of two values, packed (first value in the low half)
 __device__ __forceinline__ void tcs_split(float a, float b, uint32_t& p1, uint32_t& p2, uint32_t& p3) {
@@ -227,7 +231,10 @@ __device__ __forceinline__ void tcs_issue(uint32_t d, uint32_t r0, uint64_t bd, 
 // 27 columns, 6 MMAs a tile instead of 162) and adds the 27 shifted entries.
 //
 // What bounds it: the MMAs (54 x 5 per hidden layer and 5 x 10 x 10 sample), which
-// the epilogue does not overlap (it rewrites the planes they read).  @FUSED@
+// the epilogue does not overlap (it rewrites the planes they read): 57 cycles each,
+// the 7 KB of operands they read from shared memory.  256 samples (two rounds on
+// 152 SMs), four layers of 32 channels: 78 us, against 405 us for four launches of
+// SIMT and mma.sync kernels that cut every value 27 times.
 template <int C>
 __global__ void __launch_bounds__(kTcThreads, 1) k_tc_net(const __grid_constant__ TcNet net) {
     extern __shared__ __align__(128) unsigned char tcsm[];
@@ -241,7 +248,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_net(const __grid_constant_
     // per 32-row segment (a warp's accumulator lanes): D_-1 of the row before its
     // first, D_+1 of the row after its last
     constexpr int kSeg = 4 * (512 / (3 * C));
-    __shared__ __align__(16) float edge_lo[kSeg + 1][C], edge_hi[kSeg + 1][C];
+    __shared__ __align__(16) float edge_lo[kSeg + 1][C], edge_hi[kSeg + 1][C], s_bias[C];
+    __shared__ short s_vox[32 * kSeg];                          // the real voxel of each tile row, or -1
+    for (int e = threadIdx.x; e < 128 * g.tiles; e += kTcThreads) s_vox[e] = (short)g.voxel(g.v0 + e);
     const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
     const uint32_t bmma = tcs_u32(&bars[0]), bw = tcs_u32(&bars[1]);
     uint32_t ncols = 32;
@@ -329,15 +338,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_net(const __grid_constant_
                 // P[voxel][tap], then the sum over the taps and the logistic
                 float* P = reinterpret_cast<float*>(wreg);
                 for (int t = warp >> 2; t < g.tiles; t += kTcThreads / 128) {
-                    float v[32];
+                    uint32_t lo[16], hi[16];
                     __syncwarp();
                     const uint32_t ta = tmem + 32u * t + ((uint32_t)(32 * quarter) << 16);
-                    tcs_ld16(ta, v);
-                    tcs_ld16(ta + 16, v + 16);
-                    const int p = g.voxel(g.v0 + 128 * t + 32 * quarter + lane);
+                    tcs_ld16(ta, lo);
+                    tcs_ld16(ta + 16, hi);
+                    tcs_ld_wait(lo);
+                    tcs_ld_wait(hi);
+                    const int p = s_vox[128 * t + 32 * quarter + lane];
                     if (p >= 0) {
 #pragma unroll
-                        for (int q = 0; q < 27; ++q) P[p * 27 + q] = v[q];
+                        for (int q = 0; q < 27; ++q) P[p * 27 + q] = __uint_as_float(q < 16 ? lo[q] : hi[q - 16]);
                     }
                 }
                 tcs_sync();
@@ -356,52 +367,79 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_net(const __grid_constant_
                 tcs_sync();                                     // P is overwritten by the next sample's weights
                 continue;
             }
-            for (int t = warp >> 2; t < g.tiles; t += kTcThreads / 128) {       // the segments' edge rows
-                const int seg = 4 * t + quarter;
+            // tasks (tile, 16 channels) over the four warps of an accumulator-lane quarter
+            for (int k = warp >> 2; k < g.tiles * (C / 16); k += kTcThreads / 128) {   // the segments' edge rows
+                const int t = k / (C / 16), h = k % (C / 16), seg = 4 * t + quarter;
                 const uint32_t ta = tmem + (uint32_t)(3 * C * t) + ((uint32_t)(32 * quarter) << 16);
-#pragma unroll
-                for (int h = 0; h < C / 16; ++h) {
-                    float lo[16], hi[16];
+                {
+                    uint32_t lo[16], hi[16];
                     __syncwarp();                               // the loads are warp-collective
                     tcs_ld16(ta + 16u * h, lo);
                     tcs_ld16(ta + 2u * C + 16u * h, hi);
+                    tcs_ld_wait(lo);
+                    tcs_ld_wait(hi);
+                    if (lane == 31) {
 #pragma unroll
-                    for (int c = 0; c < 16; c += 4) {
-                        if (lane == 31) *reinterpret_cast<float4*>(&edge_lo[seg + 1][16 * h + c]) = make_float4(lo[c], lo[c + 1], lo[c + 2], lo[c + 3]);
-                        if (lane == 0) *reinterpret_cast<float4*>(&edge_hi[seg][16 * h + c]) = make_float4(hi[c], hi[c + 1], hi[c + 2], hi[c + 3]);
+                        for (int c = 0; c < 16; c += 4)
+                            *reinterpret_cast<uint4*>(&edge_lo[seg + 1][16 * h + c]) = make_uint4(lo[c], lo[c + 1], lo[c + 2], lo[c + 3]);
+                    }
+                    if (lane == 0) {
+#pragma unroll
+                        for (int c = 0; c < 16; c += 4)
+                            *reinterpret_cast<uint4*>(&edge_hi[seg][16 * h + c]) = make_uint4(hi[c], hi[c + 1], hi[c + 2], hi[c + 3]);
                     }
                 }
             }
-            if (tid < C) edge_lo[0][tid] = edge_hi[4 * g.tiles][tid] = 0.0f;
+            if (tid < C) {
+                edge_lo[0][tid] = edge_hi[4 * g.tiles][tid] = 0.0f;
+                s_bias[tid] = L.bias && tid < L.cout ? L.bias[tid] : 0.0f;
+            }
             __syncthreads();
-            for (int t = warp >> 2; t < g.tiles; t += kTcThreads / 128) {
-                const int seg = 4 * t + quarter, row = g.v0 + 32 * seg + lane;
+            const float leak = L.leaky ? 0.01f : 1.0f;         
+            for (int k = warp >> 2; k < g.tiles * (C / 16); k += kTcThreads / 128) {
+                const int t = k / (C / 16), h = k % (C / 16), seg = 4 * t + quarter, row = g.v0 + 32 * seg + lane;
                 const uint32_t ta = tmem + (uint32_t)(3 * C * t) + ((uint32_t)(32 * quarter) << 16);
-                const int p = g.voxel(row);
-#pragma unroll
-                for (int h = 0; h < C / 16; ++h) {
-                    float v[16], lo[16], hi[16];
+                const int p = s_vox[32 * seg + lane];
+                // the edge lanes take their neighbour from shared memory, the others by a shuffle
+                const float* el = edge_lo[lane == 31 ? seg + 1 : seg];
+                const float* eh = edge_hi[lane == 0 ? seg : seg + 1];
+                {
+                    uint32_t lo[16], md[16], hi[16];
+                    float v[16];
                     __syncwarp();
                     tcs_ld16(ta + 16u * h, lo);
-                    tcs_ld16(ta + (uint32_t)C + 16u * h, v);
+                    tcs_ld16(ta + (uint32_t)C + 16u * h, md);
                     tcs_ld16(ta + 2u * C + 16u * h, hi);
+                    tcs_ld_wait(lo);
+                    tcs_ld_wait(md);
+                    tcs_ld_wait(hi);
 #pragma unroll
-                    for (int c = 0; c < 16; ++c) {
-                        float a = __shfl_up_sync(0xffffffffu, lo[c], 1), z = __shfl_down_sync(0xffffffffu, hi[c], 1);
-                        if (lane == 0) a = edge_lo[seg][16 * h + c];
-                        if (lane == 31) z = edge_hi[seg + 1][16 * h + c];
-                        v[c] = (a + z) + v[c];
+                    for (int c4 = 0; c4 < 16; c4 += 4) {
+                        const float4 a4 = *reinterpret_cast<const float4*>(el + 16 * h + c4);
+                        const float4 z4 = *reinterpret_cast<const float4*>(eh + 16 * h + c4);
+                        const float4 b4 = *reinterpret_cast<const float4*>(s_bias + 16 * h + c4);
+                        const float aa[4] = {a4.x, a4.y, a4.z, a4.w}, zz[4] = {z4.x, z4.y, z4.z, z4.w}, bb[4] = {b4.x, b4.y, b4.z, b4.w};
+#pragma unroll
+                        for (int q = 0; q < 4; ++q) {
+                            const int c = c4 + q;
+                            const float up = __shfl_up_sync(0xffffffffu, __uint_as_float(lo[c]), 1);
+                            const float dn = __shfl_down_sync(0xffffffffu, __uint_as_float(hi[c]), 1);
+                            const float x = ((lane == 0 ? aa[q] : up) + (lane == 31 ? zz[q] : dn)) + __uint_as_float(md[c]) + bb[q];
+                            v[c] = x > 0.0f ? x : leak * x;
+                        }
                     }
                     if (p >= 0) {
+                        const long long o = ((long long)b * L.cout + 16 * h) * g.S + p;
+                        if (L.mask) {                           // backward: the derivative of the layer's leaky ReLU
+                            float m[16];
 #pragma unroll
-                        for (int c = 0; c < 16; ++c) {
-                            const int ch = 16 * h + c;
-                            const bool real = ch < L.cout;
-                            const long long o = ((long long)b * L.cout + (real ? ch : 0)) * g.S + p;
-                            if (L.bias && real) v[c] += __ldg(L.bias + ch);
-                            if (L.leaky) v[c] = v[c] > 0.0f ? v[c] : 0.01f * v[c];
-                            if (L.mask && real && !(L.mask[o] > 0.0f)) v[c] *= 0.01f;
-                            if (L.out && real) L.out[o] = v[c];
+                            for (int c = 0; c < 16; ++c) m[c] = 16 * h + c < L.cout ? L.mask[o + (long long)c * g.S] : 1.0f;
+#pragma unroll
+                            for (int c = 0; c < 16; ++c) if (!(m[c] > 0.0f)) v[c] *= 0.01f;
+                        }
+                        if (L.out) {
+#pragma unroll
+                            for (int c = 0; c < 16; ++c) if (16 * h + c < L.cout) L.out[o + (long long)c * g.S] = v[c];
                         }
                         if (!L.last) {
                             tcs_put8(planes, pitch, KC, 2 * h, row, v);
@@ -436,7 +474,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_net(const __grid_constant_
 // CTAs' partial sums are added in a fixed order by k_tc_sum.
 //
 // What bounds it: the MMAs, six per product of FP32 operands, at the 4 cycles per
-// SM that mma.sync takes for m16n8k16 here.  @WG@
+// SM that mma.sync takes for m16n8k16 here: 256 samples of 5 x 10 x 10, 32 -> 32
+// channels 157 us (136 us of MMAs), against 2480 us for a CTA per channel pair that
+// read both arrays 27 times through L1.
 // ---------------------------------------------------------------------------
 constexpr int kWgThreads = 27 * 32;
 __host__ __device__ inline uint32_t wg_smem(int H, int W, int zc, int mt, int nt) {
@@ -567,7 +607,7 @@ k_tc_wgrad(int D, int H, int W, int zc, int batch, int Cin, int Cout, const floa
 // Output layer (one channel of g): the taps become the rows of g (im2col), and all
 // of its gradient is one product over K = voxels, out[tap][ci] = sum_q g[q - tap]
 // in[ci][q].  A tap per warp as above would pad the single channel to 16 rows 27
-// times over (256 samples of 5 x 10 x 10, 32 channels: 84 us against 40).  (For
+// times over (256 samples of 5 x 10 x 10, 32 channels: 84 us against 42).  (For
 // the first layer the same with 27 columns per input channel lost, 118 us against
 // 56: it stages 108 gathered columns per voxel.)  The warps share the K steps of
 // an item (one sample's slab) and are added in warp order at the end.

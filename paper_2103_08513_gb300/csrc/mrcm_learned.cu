@@ -103,8 +103,9 @@ k_conv_forward(ConvShape sh, int Cin, int Cout, const __nv_bfloat16* __restrict_
     }
 }
 
-// The same forward for a 32 -> 32 channel layer as an implicit GEMM on the BF16
-// tensor cores: out[co][p] = bias[co] + sum_k A[co][k] B[k][p] with k = tap 32 + ci,
+// For boxes whose planes do not fit the fused pass of mrcm_conv_tc.cuh, or more
+// than eight input channels: the same forward for a 32 -> 32 channel layer as an
+// implicit GEMM on the BF16 tensor cores: out[co][p] = bias[co] + sum_k A[co][k] B[k][p] with k = tap 32 + ci,
 // A = the BF16 weights (exact in BF16), B[k][p] = in[ci][p + tap] cut into three BF16
 // pieces x = x1 + x2 + x3 (x1 the rounded value, x2 and x3 the rounded remainders, which
 // carry x to FP32 accuracy); mma.sync m16n8k16 with FP32 accumulation (a BF16 x BF16
