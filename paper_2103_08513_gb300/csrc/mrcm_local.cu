@@ -89,8 +89,10 @@ k_coefficients(const SubInfo* __restrict__ subs, const FaceInfo* __restrict__ fa
                double3 bc_lo, double3 bc_hi,
                double* __restrict__ coef, double* __restrict__ scale, double* __restrict__ rhs_dir,
                double* __restrict__ face_tr, double* __restrict__ face_beta, double* __restrict__ face_u,
-               double* __restrict__ face_bst, long long ncell_total) {
+               double* __restrict__ face_bst, long long ncell_total,
+               short* __restrict__ cface /* [cell][6] face of each cell side, for the subdomains with frag; or NULL */) {
     const SubInfo s = subs[blockIdx.x];
+    int* cw = cface && s.frag ? reinterpret_cast<int*>(cface + 6 * s.cell_off) : nullptr;
     const long long ncells = (long long)geo.n[0] * geo.n[1] * geo.n[2];
     const double* Kc[3] = {K, K + ncells, K + 2 * ncells};
     const long long stride[3] = {1, geo.n[0], (long long)geo.n[0] * geo.n[1]};
@@ -118,6 +120,7 @@ k_coefficients(const SubInfo* __restrict__ subs, const FaceInfo* __restrict__ fa
             }
             tp[a][c] = T;
         }
+        if (cw) { cw[3 * c] = -1; cw[3 * c + 1] = -1; cw[3 * c + 2] = -1; }
     }
     __syncthreads();                                   // the high-side cells read their "-" faces
     for (int c = threadIdx.x; c < s.N; c += blockDim.x) {
@@ -165,6 +168,7 @@ k_coefficients(const SubInfo* __restrict__ subs, const FaceInfo* __restrict__ fa
         face_beta[s.face_off + q] = beta;
         face_u[s.face_off + q] = -beta * fi.s * tr;     // U-MBF right-hand side on this face
         face_bst[s.face_off + q] = beta * fi.s * tr;     // weight of the face's flux in the U row
+        if (cw) cface[6 * (s.cell_off + fi.cell) + 2 * a + (fi.s > 0 ? 1 : 0)] = (short)q;   // one face per cell side
     }
 }
 
@@ -664,11 +668,20 @@ k_block_factor_tc(const SubInfo* __restrict__ subs, const int* __restrict__ list
         if (stop_s) break;
         // W_s: row i of the swept matrix (every lane loads: the TMEM loads are warp-collective)
         {
+            const int nt16 = (b + 15) >> 4;
+            float* Wf = W + (long long)sl * frag_stride(b);
             float* row = W + (long long)sl * wstride<float>(b) + (long long)min(i, b - 1) * b;
             for (int c0 = 0; c0 < kTcN; c0 += 16) {
                 float v[16];
                 tm_ld16(trow + c0, v);
-                if (i < b) {
+                if (s.frag) {
+                    if (i < 16 * nt16 && c0 < 16 * nt16) {
+#pragma unroll
+                        for (int q = 0; q < 16; q += 2)
+                            *reinterpret_cast<float2*>(Wf + frag_off(nt16, i, c0 + q)) =
+                                make_float2(i < b && c0 + q < b ? v[q] : 0.0f, i < b && c0 + q + 1 < b ? v[q + 1] : 0.0f);
+                    }
+                } else if (i < b) {
 #pragma unroll
                     for (int q = 0; q < 16; ++q)
                         if (c0 + q < b) row[c0 + q] = v[q];
@@ -694,6 +707,56 @@ k_block_factor_tc(const SubInfo* __restrict__ subs, const int* __restrict__ list
 // same sweep-operator step to its tile; W_s is written as a full matrix.
 // ---------------------------------------------------------------------------
 constexpr int kTriB = 256;                 // largest block
+
+// An 8 x 8 tile (rows i0 .., columns j0 .., multiples of 8) of a block in fragment
+// order, zero past b, and its transpose when asked for (an odd count of 8-row tiles
+// leaves the last half of the padding to the tile before it).
+__device__ __forceinline__ void store_frag8(float* __restrict__ Wf, int b, int i0, int j0, const float (&a)[8][8], bool transposed) {
+    const int nt = (b + 15) >> 4, n8 = (b + 7) >> 3;
+    if (i0 >= 8 * n8 || j0 >= 8 * n8) return;
+    // entry (i0 + r, j0 + c) of the aligned tile lies at its (i0, j0) + 16 r + 2 c (c even), the next column beside it
+    float* q = Wf + frag_off(nt, i0, j0);
+    const bool whole = i0 + 8 <= b && j0 + 8 <= b;
+#pragma unroll
+    for (int r = 0; r < 8; ++r)
+#pragma unroll
+        for (int c = 0; c < 8; c += 2) {
+            float2 v = make_float2(a[r][c], a[r][c + 1]);
+            if (!whole) {
+                if (i0 + r >= b || j0 + c >= b) v.x = 0.0f;
+                if (i0 + r >= b || j0 + c + 1 >= b) v.y = 0.0f;
+            }
+            *reinterpret_cast<float2*>(q + 16 * r + 2 * c) = v;
+        }
+    if (transposed) {
+        q = Wf + frag_off(nt, j0, i0);
+#pragma unroll
+        for (int c = 0; c < 8; ++c)
+#pragma unroll
+            for (int r = 0; r < 8; r += 2) {
+                float2 v = make_float2(a[r][c], a[r + 1][c]);
+                if (!whole) {
+                    if (i0 + r >= b || j0 + c >= b) v.x = 0.0f;
+                    if (i0 + r + 1 >= b || j0 + c >= b) v.y = 0.0f;
+                }
+                *reinterpret_cast<float2*>(q + 16 * c + 2 * r) = v;
+            }
+    }
+    if (n8 & 1) {                                  // rows and columns 8 n8 .. 8 n8 + 7 of the padding
+        const int e = 8 * n8;
+        auto zero = [&](int i, int j) {
+            float* z = Wf + frag_off(nt, i, j);
+#pragma unroll 1
+            for (int r = 0; r < 8; ++r)
+#pragma unroll 1
+                for (int c = 0; c < 8; c += 2) *reinterpret_cast<float2*>(z + 16 * r + 2 * c) = make_float2(0.0f, 0.0f);
+        };
+        if (i0 == e - 8) zero(e, j0);
+        if (j0 == e - 8) zero(i0, e);
+        else if (transposed && i0 == e - 8) zero(j0, e);
+        if (i0 == e - 8 && j0 == e - 8) zero(e, e);
+    }
+}
 
 // CTA size of the triangle factor for a b x b block: whole warps covering the
 // nt (nt + 1) / 2 tiles
@@ -817,7 +880,9 @@ k_block_factor_tri(const SubInfo* __restrict__ subs, const int* __restrict__ lis
         }
         // W_s as a full matrix: the tile and, below the diagonal, its transpose
         float* Ws = W + (long long)sl * wstride<float>(b);
-        if (own) {
+        if (own && s.frag) {
+            store_frag8(W + (long long)sl * frag_stride(b), b, i0, j0, a, !diag);
+        } else if (own) {
 #pragma unroll
             for (int r = 0; r < 8; ++r) {
                 const int i = i0 + r;
@@ -945,6 +1010,13 @@ k_block_factor_tile(const SubInfo* __restrict__ subs, const int* __restrict__ li
         }
         // store W_s (full symmetric matrix, row major)
         float* Ws = W + (long long)sl * wstride<float>(b);
+        if constexpr (TPT == 8) {
+            if (s.frag) {
+                store_frag8(W + (long long)sl * frag_stride(b), b, i0, j0, a, false);
+                __syncthreads();
+                continue;
+            }
+        }
 #pragma unroll
         for (int r = 0; r < TPT; ++r) {
             const int i = i0 + r;
@@ -1275,6 +1347,7 @@ struct LocalArgs {
     const int* nlist_dev; // when set: the list holds min(nlist, *nlist_dev) subdomains (written by an earlier kernel)
     int col_groups;       // > 1: up to this many CTAs share a subdomain, each taking the columns j = grp mod G
                           // (G = min(col_groups, grid / subdomains)); 1: one CTA per subdomain
+    const short* cface;   // [cell][6] face of each cell side (fragment-order subdomains)
     int passes;           // refinement sweeps run back to back on each subdomain by one launch (sweeps only)
 };
 
@@ -1634,6 +1707,8 @@ k_local_solve(LocalArgs g, const T* __restrict__ Wall) {
     }
     drain_pipe(pipe, bar);
 }
+
+#include "mrcm_solve_tc.cuh"
 
 // Tunable variants of the local solve: threads per CTA x block-product path
 // (SIMT with 2, 1 or 4 rows per thread, the pair tile, or 3xTF32 tensor
@@ -2162,7 +2237,8 @@ int launch_factor(const Tables& t, const DeviceTables& d, const Layout& L, char*
                                              c.beta_const, bcm, blo, bhi, coef, scale,
                                              (double*)(ws + L.rhs_part), (double*)(ws + L.face_tr),
                                              (double*)(ws + L.face_beta), (double*)(ws + L.face_u),
-                                             (double*)(ws + L.face_bst), t.n_cells));
+                                             (double*)(ws + L.face_bst), t.n_cells,
+                                             precision == MRCM_FP64 ? nullptr : (short*)(ws + L.cface)));
     // the learned form solves the local problems iteratively: coefficients only
     if (t.n_waves == 1 && precision != MRCM_LEARNED_PCG) launch_factor_wave(t, d, L, ws, precision, 0, st, P);
     return (int)cudaGetLastError();
@@ -2172,9 +2248,22 @@ static size_t solve_smem_bytes(const Tables& t, int precision) {
     const int mpad = (t.max_m + 3) & ~3;
     size_t sm = 0;
     for (const SubInfo& sb : t.subs)
-        sm = std::max(sm, precision == MRCM_FP64 ? solve_smem_layout<double>(sb.b, mpad, sb.N).total
+        if (!sb.frag) sm = std::max(sm, precision == MRCM_FP64 ? solve_smem_layout<double>(sb.b, mpad, sb.N).total
                                                  : solve_smem_layout<float>(sb.b, mpad, sb.N).total);
     return sm + 16;                                // + the two mbarriers, after the largest layout
+}
+
+static BigSmem big_smem(const Tables& t) {
+    BigSmem b;
+    for (const SubInfo& s : t.subs) if (s.frag) b.add(s.b, s.m);
+    return b;
+}
+static const void* big_kernel(bool sweep, int units) {
+    const int U = (units + kBigWarps - 1) / kBigWarps;
+    if (sweep) return U <= 1 ? (const void*)k_solve_big<true, 1> : U <= 2 ? (const void*)k_solve_big<true, 2>
+                    : U <= 4 ? (const void*)k_solve_big<true, 4> : (const void*)k_solve_big<true, 8>;
+    return U <= 1 ? (const void*)k_solve_big<false, 1> : U <= 2 ? (const void*)k_solve_big<false, 2>
+         : U <= 4 ? (const void*)k_solve_big<false, 4> : (const void*)k_solve_big<false, 8>;
 }
 
 // One-time kernel configuration (dynamic shared memory limits, persistent
@@ -2196,6 +2285,16 @@ int configure_local(const Tables& t, DeviceTables& d) {
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ1, k1, variant_threads(v), d.solve_smem);
         d.solve_occ[v] = std::max(1, occ0);
         d.sweep_occ[v] = std::max(1, occ1);
+    }
+    const BigSmem big = big_smem(t);
+    if (big.units > 0) {
+        for (int sw = 0; sw < 2; ++sw) {
+            const void* k = big_kernel(sw == 1, big.units);
+            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)big.total());
+            int occ = 0;
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, kBigThreads, big.total());
+            d.big_occ[sw] = std::max(1, occ);
+        }
     }
     if (!f64) {
         // the FP64 solve kernels of the mixed modes' fallback and post-processing (variant 0)
@@ -2236,21 +2335,60 @@ static LocalArgs local_args(const Tables& t, const DeviceTables& d, const Layout
     g.nlist_dev = nullptr;
     g.col_groups = 1;
     g.passes = 1;
+    g.cface = (const short*)(ws + L.cface);
     return g;
 }
 
-// Launch one local-solve pass (first solve or refinement sweep) with variant v.
-static void launch_local_pass(const Tables& t, const DeviceTables& d, LocalArgs& g, const void* W, bool sweep,
-                              int v, cudaStream_t st, Prof& P) {
+// CTAs that share a subdomain (by columns) when there are too few subdomains to
+// fill the SMs: as many as give every SM two CTAs, each with eight columns or more.
+// The columns are independent, so the results are those of one CTA.  40 x 40 x 8
+// cells in FP64 (32 subdomains, 53 columns: 7 groups): first solve 769 -> 317 us,
+// sweep 838 -> 342 us; 45 x 38 x 27 (100 subdomains, mixed, 3 groups): 453 -> 259
+// and 1313 -> 698 us.
+static int column_groups(const DeviceTables& d, const LocalArgs& g, int max_m) {
+    if (g.last_only || g.nlist <= 0) return 1;
+    return std::max(1, std::min(2 * d.sms / g.nlist, max_m / 8));
+}
+
+// Launch one local-solve pass (first solve or refinement sweeps) over g.list, whose
+// first nbig subdomains have fragment-order factors; v: variant of the others.
+static void launch_local_pass(const Tables& t, const DeviceTables& d, const LocalArgs& g0, int nbig, const void* W,
+                              bool sweep, int v, cudaStream_t st, Prof& P) {
     const bool f64 = t.cfg.precision == MRCM_FP64;
-    const void* k = f64 ? (sweep ? solve_kernel<double, false, true>(v) : solve_kernel<double, false, false>(v))
-                        : (sweep ? solve_kernel<float, true, true>(v) : solve_kernel<float, true, false>(v));
-    const int occ = sweep ? d.sweep_occ[v] : d.solve_occ[v];
-    const int grid = std::max(1, std::min(g.nlist, d.sms * occ));
-    MRCM_LAUNCH(P, "k_set_int", st, k_set_int<<<1, 1, 0, st>>>(g.queue, 0));
-    void* args[] = {(void*)&g, (void*)&W};
-    MRCM_LAUNCH(P, sweep ? "k_ir_sweep" : "k_local_solve", st,
-                cudaLaunchKernel(k, dim3(grid), dim3(variant_threads(v)), args, d.solve_smem, st));
+    const char* name = sweep ? "k_ir_sweep" : "k_local_solve";
+    if (nbig > 0) {
+        const BigSmem big = big_smem(t);
+        BigArgs a;
+        a.g = g0;
+        a.g.nlist = nbig;
+        a.g.col_groups = column_groups(d, a.g, t.max_m);
+        a.stages = big.stages();
+        a.stage_bytes = big.nt * 1024;
+        size_t o = (size_t)a.stages * a.stage_bytes;
+        a.ring = 0;
+        a.zp = (int)o; o += BigSmem::al(big.zp);
+        a.p = (int)o; o += BigSmem::al(big.p);
+        a.co = (int)o; o += BigSmem::al(big.co);
+        a.cols = (int)o; o += BigSmem::al(big.cols);
+        a.bars = (int)o;
+        const int grid = std::max(1, std::min(nbig * a.g.col_groups, d.sms * d.big_occ[sweep]));
+        MRCM_LAUNCH(P, "k_set_int", st, k_set_int<<<1, 1, 0, st>>>(g0.queue, 0));
+        void* args[] = {(void*)&a, (void*)&W};
+        MRCM_LAUNCH(P, name, st, cudaLaunchKernel(big_kernel(sweep, big.units), dim3(grid), dim3(kBigThreads), args, big.total(), st));
+    }
+    if (g0.nlist > nbig) {
+        LocalArgs g = g0;
+        g.list += nbig;
+        g.nlist -= nbig;
+        g.col_groups = column_groups(d, g, t.max_m);
+        const void* k = f64 ? (sweep ? solve_kernel<double, false, true>(v) : solve_kernel<double, false, false>(v))
+                            : (sweep ? solve_kernel<float, true, true>(v) : solve_kernel<float, true, false>(v));
+        const int occ = sweep ? d.sweep_occ[v] : d.solve_occ[v];
+        const int grid = std::max(1, std::min(g.nlist * g.col_groups, d.sms * occ));
+        MRCM_LAUNCH(P, "k_set_int", st, k_set_int<<<1, 1, 0, st>>>(g.queue, 0));
+        void* args[] = {(void*)&g, (void*)&W};
+        MRCM_LAUNCH(P, name, st, cudaLaunchKernel(k, dim3(grid), dim3(variant_threads(v)), args, d.solve_smem, st));
+    }
 }
 
 // FP64 fallback of one wave (see k_fb_collect): slots, FP64 block factors of
@@ -2316,7 +2454,7 @@ int launch_solve_mbf(const Tables& t, const DeviceTables& d, const Layout& L, ch
         g.list = d.solve_list + t.wave_off[w];
         g.nlist = t.wave_off[w + 1] - t.wave_off[w];
         g.count_unconverged = 0;
-        launch_local_pass(t, d, g, W, false, d.solve_variant, st, P);
+        launch_local_pass(t, d, g, t.wave_big[w], W, false, d.solve_variant, st, P);
         if (precision != MRCM_FP64) {
             // all sweeps in one launch, each subdomain's back to back (a subdomain that needs more
             // sweeps than most no longer holds up a launch of its own per sweep), or one launch per
@@ -2325,7 +2463,7 @@ int launch_solve_mbf(const Tables& t, const DeviceTables& d, const Layout& L, ch
                 const int np = d.sweeps_separate ? 1 : sweeps - it;
                 g.passes = np;
                 g.count_unconverged = it + np == sweeps && fb_cap == 0 ? 1 : 0;
-                launch_local_pass(t, d, g, W, true, d.sweep_variant, st, P);
+                launch_local_pass(t, d, g, t.wave_big[w], W, true, d.sweep_variant, st, P);
                 it += np;
             }
             g.passes = 1;
@@ -2334,7 +2472,7 @@ int launch_solve_mbf(const Tables& t, const DeviceTables& d, const Layout& L, ch
             // FP64 form: the direct solve through the explicit block inverses plus one
             // FP64 refinement step (the same residual sweep), for FP64-level MBFs
             g.count_unconverged = 0;
-            launch_local_pass(t, d, g, W, true, d.sweep_variant, st, P);
+            launch_local_pass(t, d, g, t.wave_big[w], W, true, d.sweep_variant, st, P);
         }
     }
     MRCM_LAUNCH(P, "k_set_int", st, k_set_int<<<1, 1, 0, st>>>(status + ST_SWEEPS, precision == MRCM_FP64 ? 1 : sweeps));
@@ -2373,12 +2511,12 @@ int launch_postprocess(const Tables& t, const DeviceTables& d, const Layout& L, 
             g.list = d.solve_list + t.wave_off[w];
             g.nlist = t.wave_off[w + 1] - t.wave_off[w];
             g.count_unconverged = 0;
-            launch_local_pass(t, d, g, W, false, d.solve_variant, st, P);
+            launch_local_pass(t, d, g, t.wave_big[w], W, false, d.solve_variant, st, P);
             MRCM_LAUNCH(P, "k_pp_scale", st, k_pp_scale<<<g.nlist, kThreads, 0, st>>>(g.subs, g.list, coef, g.rhs_dir,
                         f, geo, t.n_cells, g.X, g.bnorm, nullptr));
             for (int it = 0; it < sweeps; ++it) {
                 g.count_unconverged = it + 1 == sweeps ? 1 : 0;
-                launch_local_pass(t, d, g, W, true, d.sweep_variant, st, P);
+                launch_local_pass(t, d, g, t.wave_big[w], W, true, d.sweep_variant, st, P);
             }
         }
     } else {
@@ -2390,12 +2528,12 @@ int launch_postprocess(const Tables& t, const DeviceTables& d, const Layout& L, 
             g.list = d.solve_list + t.wave_off[w];
             g.nlist = t.wave_off[w + 1] - t.wave_off[w];
             g.count_unconverged = 0;
-            launch_local_pass(t, d, g, W, false, d.solve_variant, st, P);
+            launch_local_pass(t, d, g, t.wave_big[w], W, false, d.solve_variant, st, P);
             MRCM_LAUNCH(P, "k_pp_scale", st, k_pp_scale<<<g.nlist, kThreads, 0, st>>>(g.subs, g.list, coef, g.rhs_dir,
                         f, geo, t.n_cells, g.X, g.bnorm, nullptr));
             g.passes = kPpMixedSweeps;
             g.tol2 = kPpMixedTol * kPpMixedTol;
-            launch_local_pass(t, d, g, W, true, d.sweep_variant, st, P);
+            launch_local_pass(t, d, g, t.wave_big[w], W, true, d.sweep_variant, st, P);
             g.passes = 1;
             g.tol2 = tol * tol;
         }
@@ -2544,10 +2682,10 @@ int autotune_local(const Tables& t, DeviceTables& d, const Layout& L, char* ws, 
             }
             // convergence of the refinement with this factor (wave 0)
             k_set_int<<<1, 1, 0, st>>>(status + ST_UNCONVERGED, 0);
-            launch_local_pass(t, d, g, W, false, d.solve_variant, st, dummy);
+            launch_local_pass(t, d, g, t.wave_big[0], W, false, d.solve_variant, st, dummy);
             for (int it = 0; it < t.cfg.ir_max_sweeps; ++it) {
                 g.count_unconverged = it + 1 == t.cfg.ir_max_sweeps ? 1 : 0;
-                launch_local_pass(t, d, g, W, true, d.sweep_variant, st, dummy);
+                launch_local_pass(t, d, g, t.wave_big[0], W, true, d.sweep_variant, st, dummy);
             }
             g.count_unconverged = 0;
             cudaMemcpyAsync(&unconv[fv], status + ST_UNCONVERGED, sizeof(int), cudaMemcpyDeviceToHost, st);
@@ -2566,7 +2704,7 @@ int autotune_local(const Tables& t, DeviceTables& d, const Layout& L, char* ws, 
         std::vector<float> t0;
         for (int r = 0; r < reps; ++r) {
             cudaEventRecord(e0, st);
-            launch_local_pass(t, d, g, W, false, v, st, dummy);
+            launch_local_pass(t, d, g, t.wave_big[0], W, false, v, st, dummy);
             cudaEventRecord(e1, st);
             cudaEventSynchronize(e1);
             float ms = 0.f;
@@ -2581,10 +2719,10 @@ int autotune_local(const Tables& t, DeviceTables& d, const Layout& L, char* ws, 
         for (int v = 0; v < kNumSolveVariants; ++v) {
             std::vector<float> t1;
             for (int r = 0; r < reps; ++r) {
-                launch_local_pass(t, d, g, W, false, *best_solve, st, dummy);
+                launch_local_pass(t, d, g, t.wave_big[0], W, false, *best_solve, st, dummy);
                 cudaEventRecord(e0, st);
                 g.passes = t.cfg.ir_max_sweeps;          // all sweeps in one launch
-                if (g.passes > 0) launch_local_pass(t, d, g, W, true, v, st, dummy);
+                if (g.passes > 0) launch_local_pass(t, d, g, t.wave_big[0], W, true, v, st, dummy);
                 g.passes = 1;
                 cudaEventRecord(e1, st);
                 cudaEventSynchronize(e1);
@@ -2599,9 +2737,9 @@ int autotune_local(const Tables& t, DeviceTables& d, const Layout& L, char* ws, 
         // the chosen variant with one launch per sweep
         std::vector<float> t2;
         for (int r = 0; r < reps && t.cfg.ir_max_sweeps > 0; ++r) {
-            launch_local_pass(t, d, g, W, false, *best_solve, st, dummy);
+            launch_local_pass(t, d, g, t.wave_big[0], W, false, *best_solve, st, dummy);
             cudaEventRecord(e0, st);
-            for (int it = 0; it < t.cfg.ir_max_sweeps; ++it) launch_local_pass(t, d, g, W, true, *best_sweep, st, dummy);
+            for (int it = 0; it < t.cfg.ir_max_sweeps; ++it) launch_local_pass(t, d, g, t.wave_big[0], W, true, *best_sweep, st, dummy);
             cudaEventRecord(e1, st);
             cudaEventSynchronize(e1);
             float ms = 0.f;

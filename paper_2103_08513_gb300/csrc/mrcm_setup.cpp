@@ -257,7 +257,9 @@ mrcm_status build_tables(const mrcm_config* cfg, Tables& t, std::string& err) {
         long long wcur = 0, wmax = 0;
         for (int q = 0; q < nsub; ++q) {
             SubInfo& s = t.subs[t.solve_list[q]];
-            const long long need = (long long)s.ns * (t.cfg.precision == MRCM_FP64 ? wstride<double>(s.b) : wstride<float>(s.b));
+            s.frag = cfg->precision != MRCM_FP64 && big_ok(s.b, s.m) ? 1 : 0;
+            const long long need = (long long)s.ns * (t.cfg.precision == MRCM_FP64 ? wstride<double>(s.b)
+                                                      : s.frag ? frag_stride(s.b) : wstride<float>(s.b));
             if (cfg->wave_bytes > 0 && q > t.wave_off.back() && (size_t)(wcur + need) * welem > cfg->wave_bytes) {
                 t.wave_off.push_back(q);
                 wcur = 0;
@@ -269,6 +271,12 @@ mrcm_status build_tables(const mrcm_config* cfg, Tables& t, std::string& err) {
         t.wave_off.push_back(nsub);
         t.n_waves = (int)t.wave_off.size() - 1;
         t.total_w = wmax;
+        // within a wave, the fragment-order subdomains first (each kind has its own solve kernel)
+        for (int w = 0; w < t.n_waves; ++w) {
+            const auto mid = std::stable_partition(t.solve_list.begin() + t.wave_off[w], t.solve_list.begin() + t.wave_off[w + 1],
+                                                   [&](int l) { return t.subs[l].frag != 0; });
+            t.wave_big.push_back((int)(mid - t.solve_list.begin()) - t.wave_off[w]);
+        }
         t.class_list.clear();
         for (int w = 0; w < t.n_waves; ++w) {
             std::vector<std::tuple<int, double, int>> cls[3];
@@ -497,6 +505,9 @@ void compute_layout(const Tables& t, Layout& L) {
     L.scf = take(nc * sizeof(float));
     L.tsc = take(nc * sizeof(float));
     L.rhs_part = take(nc * sizeof(double));
+    bool any_frag = false;
+    for (const SubInfo& s : t.subs) any_frag = any_frag || s.frag;
+    L.cface = take(any_frag ? 6 * nc * sizeof(short) : 0);
     L.face_tr = take(t.faces.size() * sizeof(double));
     L.face_beta = take(t.faces.size() * sizeof(double));
     L.face_u = take(t.faces.size() * sizeof(double));
