@@ -99,7 +99,7 @@ struct Tables {
     std::vector<int> wave_big;         // per wave: its first so many subdomains have SubInfo::frag
     std::vector<int> wave_class_off;   // 4 entries per wave (class boundaries)
     int n_waves = 1;
-    int class_off[4] = {0, 0, 0, 0};  // class 0: b <= kRegBlock, 1: b <= kTileBlock, 2: larger (mixed); FP64: all in 2
+    int class_off[4] = {0, 0, 0, 0};  // class 0: b <= kRegBlock, 1: fragment-order factors, 2: the other larger blocks (mixed); FP64: all in 2
     long long n_cells = 0, total_x = 0, total_w = 0, total_el = 0;
     int total_elb = 0;
     int max_m = 0, max_b = 0, max_el = 0, max_N = 0;

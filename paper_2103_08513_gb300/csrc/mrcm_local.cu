@@ -708,56 +708,6 @@ k_block_factor_tc(const SubInfo* __restrict__ subs, const int* __restrict__ list
 // ---------------------------------------------------------------------------
 constexpr int kTriB = 256;                 // largest block
 
-// An 8 x 8 tile (rows i0 .., columns j0 .., multiples of 8) of a block in fragment
-// order, zero past b, and its transpose when asked for (an odd count of 8-row tiles
-// leaves the last half of the padding to the tile before it).
-__device__ __forceinline__ void store_frag8(float* __restrict__ Wf, int b, int i0, int j0, const float (&a)[8][8], bool transposed) {
-    const int nt = (b + 15) >> 4, n8 = (b + 7) >> 3;
-    if (i0 >= 8 * n8 || j0 >= 8 * n8) return;
-    // entry (i0 + r, j0 + c) of the aligned tile lies at its (i0, j0) + 16 r + 2 c (c even), the next column beside it
-    float* q = Wf + frag_off(nt, i0, j0);
-    const bool whole = i0 + 8 <= b && j0 + 8 <= b;
-#pragma unroll
-    for (int r = 0; r < 8; ++r)
-#pragma unroll
-        for (int c = 0; c < 8; c += 2) {
-            float2 v = make_float2(a[r][c], a[r][c + 1]);
-            if (!whole) {
-                if (i0 + r >= b || j0 + c >= b) v.x = 0.0f;
-                if (i0 + r >= b || j0 + c + 1 >= b) v.y = 0.0f;
-            }
-            *reinterpret_cast<float2*>(q + 16 * r + 2 * c) = v;
-        }
-    if (transposed) {
-        q = Wf + frag_off(nt, j0, i0);
-#pragma unroll
-        for (int c = 0; c < 8; ++c)
-#pragma unroll
-            for (int r = 0; r < 8; r += 2) {
-                float2 v = make_float2(a[r][c], a[r + 1][c]);
-                if (!whole) {
-                    if (i0 + r >= b || j0 + c >= b) v.x = 0.0f;
-                    if (i0 + r + 1 >= b || j0 + c >= b) v.y = 0.0f;
-                }
-                *reinterpret_cast<float2*>(q + 16 * c + 2 * r) = v;
-            }
-    }
-    if (n8 & 1) {                                  // rows and columns 8 n8 .. 8 n8 + 7 of the padding
-        const int e = 8 * n8;
-        auto zero = [&](int i, int j) {
-            float* z = Wf + frag_off(nt, i, j);
-#pragma unroll 1
-            for (int r = 0; r < 8; ++r)
-#pragma unroll 1
-                for (int c = 0; c < 8; c += 2) *reinterpret_cast<float2*>(z + 16 * r + 2 * c) = make_float2(0.0f, 0.0f);
-        };
-        if (i0 == e - 8) zero(e, j0);
-        if (j0 == e - 8) zero(i0, e);
-        else if (transposed && i0 == e - 8) zero(j0, e);
-        if (i0 == e - 8 && j0 == e - 8) zero(e, e);
-    }
-}
-
 // CTA size of the triangle factor for a b x b block: whole warps covering the
 // nt (nt + 1) / 2 tiles
 static int tri_threads(int b) {
@@ -880,9 +830,7 @@ k_block_factor_tri(const SubInfo* __restrict__ subs, const int* __restrict__ lis
         }
         // W_s as a full matrix: the tile and, below the diagonal, its transpose
         float* Ws = W + (long long)sl * wstride<float>(b);
-        if (own && s.frag) {
-            store_frag8(W + (long long)sl * frag_stride(b), b, i0, j0, a, !diag);
-        } else if (own) {
+        if (own) {
 #pragma unroll
             for (int r = 0; r < 8; ++r) {
                 const int i = i0 + r;
@@ -1010,13 +958,6 @@ k_block_factor_tile(const SubInfo* __restrict__ subs, const int* __restrict__ li
         }
         // store W_s (full symmetric matrix, row major)
         float* Ws = W + (long long)sl * wstride<float>(b);
-        if constexpr (TPT == 8) {
-            if (s.frag) {
-                store_frag8(W + (long long)sl * frag_stride(b), b, i0, j0, a, false);
-                __syncthreads();
-                continue;
-            }
-        }
 #pragma unroll
         for (int r = 0; r < TPT; ++r) {
             const int i = i0 + r;
@@ -1709,6 +1650,7 @@ k_local_solve(LocalArgs g, const T* __restrict__ Wall) {
 }
 
 #include "mrcm_solve_tc.cuh"
+#include "mrcm_factor_tc.cuh"
 
 // Tunable variants of the local solve: threads per CTA x block-product path
 // (SIMT with 2, 1 or 4 rows per thread, the pair tile, or 3xTF32 tensor
@@ -2156,6 +2098,10 @@ static void launch_factor64(const SubInfo* subs, const int* list, int n, int bma
     MRCM_LAUNCH(P, name, st, cudaLaunchKernelExC(&cfg, k, args));
 }
 
+// CTA shape of k_block_factor_mma: 8 warps of up to 5 tiles (b <= 128: 36 tiles), 16 of 5
+// (b <= 192: 78) or 16 of 9 (136).
+static int factor_mma_shape(int b) { return b <= 128 ? 0 : b <= 192 ? 1 : 2; }
+
 static void launch_factor_wave(const Tables& t, const DeviceTables& d, const Layout& L, char* ws, int precision,
                                int w, cudaStream_t st, Prof& P) {
     double* coef = (double*)(ws + L.coef);
@@ -2187,26 +2133,42 @@ static void launch_factor_wave(const Tables& t, const DeviceTables& d, const Lay
                 MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_tile<4, 16><<<n_small, 256, 0, st>>>(d.subs, d.class_list + o0, coef, scale,
                     (float*)(ws + L.W), status, t.n_cells, (float*)(ws + L.scf), (float*)(ws + L.tsc)));
         }
-        if (n_mid > 0) {
-            if (d.factor_mid_variant == 1)       // tensor cores; its shared memory keeps <= 4 CTAs (4 x 128 TMEM columns) per SM
-                MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_tc<<<n_mid, kTcN, kTcSmem, st>>>(d.subs, d.class_list + o1, coef, scale,
-                    (float*)(ws + L.W), status, t.n_cells, (float*)(ws + L.scf), (float*)(ws + L.tsc)));
-            else
-                MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_tile<8, 16><<<n_mid, 256, 0, st>>>(d.subs, d.class_list + o1, coef, scale,
-                    (float*)(ws + L.W), status, t.n_cells, (float*)(ws + L.scf), (float*)(ws + L.tsc)));
-        }
-        // the large class is ordered by b, largest first: one launch per run of
-        // subdomains that share a thread count
-        for (int q = o2; q < o3;) {
-            const int nth = tri_threads(t.subs[t.class_list[q]].b);
+        // 64 < b: fragment-order factors first (ordered by b, largest first, one launch per CTA
+        // shape; up to b = 128 the tuner may choose the kernel with the block in tensor memory),
+        // then the blocks with too many right-hand sides for k_solve_big
+        float* W = (float*)(ws + L.W);
+        float* scf = (float*)(ws + L.scf);
+        float* tsc = (float*)(ws + L.tsc);
+        int q = o1;
+        while (q < o3 && t.subs[t.class_list[q]].frag) {
+            const int b0 = t.subs[t.class_list[q]].b, shape = factor_mma_shape(b0);
             int e = q + 1;
-            while (e < o3 && tri_threads(t.subs[t.class_list[e]].b) == nth) ++e;
+            while (e < o3 && t.subs[t.class_list[e]].frag && factor_mma_shape(t.subs[t.class_list[e]].b) == shape) ++e;
             const int n = e - q;
             const int* lst = d.class_list + q;
-            float* W = (float*)(ws + L.W);
-            float* scf = (float*)(ws + L.scf);
-            float* tsc = (float*)(ws + L.tsc);
+            const size_t sm = factor_mma_smem(b0);
+            if (shape == 0 && d.factor_mid_variant == 1)    // its shared memory keeps <= 4 CTAs (4 x 128 TMEM columns) per SM
+                MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_tc<<<n, kTcN, kTcSmem, st>>>(d.subs, lst, coef, scale, W, status, t.n_cells, scf, tsc));
+            else if (shape == 0)
+                MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_mma<8, 5><<<n, 256, sm, st>>>(d.subs, lst, coef, scale, W, status, t.n_cells, scf, tsc));
+            else if (shape == 1)
+                MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_mma<16, 5><<<n, 512, sm, st>>>(d.subs, lst, coef, scale, W, status, t.n_cells, scf, tsc));
+            else
+                MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_mma<16, 9><<<n, 512, sm, st>>>(d.subs, lst, coef, scale, W, status, t.n_cells, scf, tsc));
+            q = e;
+        }
+        (void)n_mid;
+        // the large class is ordered by b, largest first: one launch per run of
+        // subdomains that share a thread count
+        while (q < o3) {
+            auto cta = [&](int k) { const int b = t.subs[t.class_list[k]].b; return b <= kTileBlock ? 256 : tri_threads(b); };
+            const int nth = cta(q);
+            int e = q + 1;
+            while (e < o3 && cta(e) == nth) ++e;
+            const int n = e - q;
+            const int* lst = d.class_list + q;
             switch (nth) {
+            case 256: MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_tile<8, 16><<<n, 256, 0, st>>>(d.subs, lst, coef, scale, W, status, t.n_cells, scf, tsc)); break;
             case 192: MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_tri<192><<<n, 192, 0, st>>>(d.subs, lst, coef, scale, W, status, t.n_cells, scf, tsc)); break;
             case 320: MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_tri<320><<<n, 320, 0, st>>>(d.subs, lst, coef, scale, W, status, t.n_cells, scf, tsc)); break;
             case 512: MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_tri<512><<<n, 512, 0, st>>>(d.subs, lst, coef, scale, W, status, t.n_cells, scf, tsc)); break;
@@ -2312,6 +2274,9 @@ int configure_local(const Tables& t, DeviceTables& d) {
         d.f64_occ = std::max(1, occ);
     }
     cudaFuncSetAttribute(k_block_factor_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
+    cudaFuncSetAttribute(k_block_factor_mma<8, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)factor_mma_smem(128));
+    cudaFuncSetAttribute(k_block_factor_mma<16, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)factor_mma_smem(192));
+    cudaFuncSetAttribute(k_block_factor_mma<16, 9>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)factor_mma_smem(256));
     return (int)cudaGetLastError();
 }
 

@@ -284,10 +284,10 @@ mrcm_status build_tables(const mrcm_config* cfg, Tables& t, std::string& err) {
                 const int l = t.solve_list[q];
                 const SubInfo& s = t.subs[l];
                 const double cost = (double)s.ns * s.b * s.b * s.b;
-                const int k = cfg->precision == MRCM_FP64 ? 2 : s.b <= kRegBlock ? 0 : s.b <= kTileBlock ? 1 : 2;
-                // large class and FP64: ordered by b first (its factor launches
-                // one CTA size per run of b), then by cost
-                cls[k].push_back({k == 2 ? -s.b : 0, -cost, l});
+                // small blocks; fragment-order factors; the others (and FP64).  The last two are ordered
+                // by b first (their factors launch one CTA shape per run of b), then by cost
+                const int k = cfg->precision == MRCM_FP64 ? 2 : s.b <= kRegBlock ? 0 : s.frag ? 1 : 2;
+                cls[k].push_back({k > 0 ? -s.b : 0, -cost, l});
             }
             for (int k = 0; k < 3; ++k) {
                 std::sort(cls[k].begin(), cls[k].end());
