@@ -8,17 +8,19 @@
 // step.  With P the pivot block, G = M_PP^{-1}, C_i = M_iP, A_i = C_i G and
 // sigma_j = -1 on swept blocks:
 //   M_ij -= sigma_j A_i C_j^T,   M_iP <- -A_i (i > P),   M_Pj <- -A_j^T (j < P),   M_PP <- G.
-// Per step: the pivot row's and column's tiles are published as C_i, one warp
-// inverts M_PP (16 FP32 pivots in registers), the A_i are formed (one tile a warp),
-// and every warp updates its tiles.  Products are m16n8k16 BF16 MMAs on three-piece
+// Per step: the pivot row's and column's tiles are published as C_i, the A_i are
+// formed (one tile a warp), and every warp updates its tiles, the next diagonal
+// tile's warp inverting it (16 FP32 pivots in registers) meanwhile.  Products are m16n8k16 BF16 MMAs on three-piece
 // operands (24 bits; six products), summed per step in a fresh accumulator and
 // added in FP32: rounding as in the FP32 sweep, pivot block by pivot block.  (The
 // variant with the block in tensor memory accumulates there over the whole sweep
 // with truncation, which costs the refinement convergence on ill-conditioned blocks.)
 //
-// What bounds it: per step the chain publish -> invert -> A_i -> update with its four
-// barriers, hidden by several CTAs per SM.  One FP32 FMA per entry and pivot and a
-// barrier per pivot before: @FB@
+// What bounds it: per step the chain publish -> A_i -> update and inversion with its
+// three barriers, hidden by several CTAs per SM (issue 40 %, shared-memory pipe 51 %,
+// tensor pipe 21 % at b = 128).  One FP32 FMA per entry and pivot and a barrier per pivot
+// before: 8192 subdomains of 16 slabs, b = 128: 24.6 -> 16.0 ms; 256 x 256 x 128 uneven
+// (b 65 .. 256): 17.9 -> 10.0 ms.
 #pragma once
 
 constexpr int kFmRow = 48;            // bytes of a 16-column BF16 plane row (padded: conflict-free ldmatrix)
@@ -27,27 +29,29 @@ __host__ __device__ inline size_t factor_mma_smem(int b) {
     return 3 * nt * 16 * kFmRow       // C planes
          + 3 * nt * 512               // A_i as A operands
          + nt * 16 * 17 * 4           // A_i in FP32
-         + 3 * 16 * kFmRow            // G planes
-         + 2 * 16 * 17 * 4            // M_PP, G
+         + 2 * 3 * 16 * kFmRow        // G planes (this step's and the next)
+         + 3 * 16 * 17 * 4            // M_PP, G (two)
          + 4 * nt * 16 * 4 + 64;      // diagonal, couplings
 }
 
-template <int NW, int TPW>
-__global__ void __launch_bounds__(32 * NW, NW == 8 ? 3 : 1)
+// NW warps of TPW tiles each, the first ND of them diagonal (tile d: warp d mod NW,
+// slot d / NW), MINB CTAs per SM.
+template <int NW, int TPW, int ND, int MINB>
+__global__ void __launch_bounds__(32 * NW, MINB)
 k_block_factor_mma(const SubInfo* __restrict__ subs, const int* __restrict__ list, const double* __restrict__ coef,
                    const double* __restrict__ scale, float* __restrict__ Wall, int* __restrict__ status,
                    long long nct, float* __restrict__ scf_all, float* __restrict__ tsc_all) {
     extern __shared__ __align__(128) unsigned char smem_ls[];
     const SubInfo s = subs[list[blockIdx.x]];
-    const int b = s.b, su = s.su, nt = (b + 15) >> 4, B = 16 * nt, ntiles = nt * (nt + 1) / 2;
+    const int b = s.b, su = s.su, nt = (b + 15) >> 4, B = 16 * nt, ntiles = nt * (nt - 1) / 2;
     unsigned char* Cp = smem_ls;                                        // [piece][row][k] BF16
     const uint32_t cpl = (uint32_t)B * kFmRow;
     uint4* Af = reinterpret_cast<uint4*>(Cp + 3 * cpl);                 // [piece][tile][lane]
     float* Ap = reinterpret_cast<float*>(Af + 3 * nt * 32);             // [tile][16][17]
     unsigned char* Gp = reinterpret_cast<unsigned char*>(Ap + nt * 16 * 17);   // [piece][row][k] BF16
-    float* D = reinterpret_cast<float*>(Gp + 3 * 16 * kFmRow);          // [16][17]
-    float* Gs = D + 16 * 17;
-    float* sd = Gs + 16 * 17;
+    float* D = reinterpret_cast<float*>(Gp + 2 * 3 * 16 * kFmRow);      // [16][17]
+    float* Gs = D + 16 * 17;                                            // [2][16][17]
+    float* sd = Gs + 2 * 16 * 17;
     float* sup = sd + B;
     float* svp = sup + B;
     float* st = svp + B;
@@ -63,12 +67,13 @@ k_block_factor_mma(const SubInfo* __restrict__ subs, const int* __restrict__ lis
     int ti[TPW], tj[TPW];
 #pragma unroll
     for (int q = 0; q < TPW; ++q) {
-        const int x = warp + NW * q;
+        // the diagonal tiles of this warp, then its share of those below them, row by row
+        const int x = q < ND ? 0 : warp + NW * (q - ND), d = warp + NW * q;
         int i = (int)((sqrtf(8.0f * (float)x + 1.0f) - 1.0f) * 0.5f);
         while (i * (i + 1) / 2 > x) --i;
         while ((i + 1) * (i + 2) / 2 <= x) ++i;
-        ti[q] = x < ntiles ? i : -1;
-        tj[q] = x - i * (i + 1) / 2;
+        ti[q] = q < ND ? (d < nt ? d : -1) : x < ntiles ? i + 1 : -1;
+        tj[q] = q < ND ? d : x - i * (i + 1) / 2;
 #pragma unroll
         for (int e = 0; e < 8; ++e) acc[q][e] = 0.0f;
     }
@@ -96,7 +101,7 @@ k_block_factor_mma(const SubInfo* __restrict__ subs, const int* __restrict__ lis
         // S_s = D_s - t o W_{s-1} o t
 #pragma unroll
         for (int q = 0; q < TPW; ++q) {
-            if (ti[q] < 0) break;
+            if (ti[q] < 0) continue;
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
                 const int i = 16 * ti[q] + g + 8 * ((e >> 1) & 1), j = 16 * tj[q] + 8 * (e >> 2) + 2 * t + (e & 1);
@@ -109,16 +114,65 @@ k_block_factor_mma(const SubInfo* __restrict__ subs, const int* __restrict__ lis
                 acc[q][e] = v;
             }
         }
+        // G = M_PP^{-1} of the diagonal tile that this warp left in D, into buffer `buf`: lane r + 16 h
+        // holds columns 8 h .. 8 h + 7 of row r.  The next pivot is formed by every lane from entries
+        // fetched before the step's update, so that a pivot's chain is multiply, FMA, reciprocal
+        // (an approximation and a Newton step; the IEEE division and a shuffle of the updated pivot
+        // took about four times as long).
+        auto leave = [&](const float (&v)[8]) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) D[(g + 8 * ((e >> 1) & 1)) * 17 + 8 * (e >> 2) + 2 * t + (e & 1)] = v[e];
+        };
+        auto invert = [&](int buf) {
+            __syncwarp();
+            const int r = lane & 15, h = lane >> 4;
+            float a[8];
+#pragma unroll
+            for (int c = 0; c < 8; ++c) a[c] = D[r * 17 + 8 * h + c];
+            float p = D[0];
+#pragma unroll
+            for (int q = 0; q < 16; ++q) {
+                const int ql = q & 7, qh = q >> 3, nl = (q + 1) & 7, nh = (q + 1) >> 3;
+                if (!(p > 0.0f)) { bad = 1; p = 1.0f; }
+                float inv;
+                asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(inv) : "f"(p));
+                inv = fmaf(inv, fmaf(-p, inv, 1.0f), inv);
+                const float cr = __shfl_sync(0xffffffffu, a[ql], r + 16 * qh);
+                if (q < 15) {
+                    const float dn = __shfl_sync(0xffffffffu, a[nl], q + 1 + 16 * nh);      // M[q+1][q+1]
+                    const float un = __shfl_sync(0xffffffffu, a[nl], q + 16 * nh);          // M[q][q+1]
+                    const float ln = __shfl_sync(0xffffffffu, a[ql], q + 1 + 16 * qh);      // M[q+1][q]
+                    p = fmaf(-ln, un * inv, dn);
+                }
+#pragma unroll
+                for (int c = 0; c < 8; ++c) {
+                    const float rq = __shfl_sync(0xffffffffu, a[c], q + 16 * h) * inv;
+                    if (r == q) a[c] = rq; else a[c] = fmaf(-cr, rq, a[c]);
+                }
+                if (h == qh) a[ql] = r == q ? inv : -cr * inv;
+            }
+            float* go = Gs + buf * 16 * 17 + r * 17 + 8 * h;
+            unsigned char* gq = Gp + buf * 3 * 16 * kFmRow + r * kFmRow + 16 * h;
+#pragma unroll
+            for (int c = 0; c < 8; c += 2) {
+                go[c] = a[c];
+                go[c + 1] = a[c + 1];
+                uint32_t w[3];
+                cut3(a[c], a[c + 1], w[0], w[1], w[2]);
+#pragma unroll
+                for (int k = 0; k < 3; ++k) *reinterpret_cast<uint32_t*>(gq + k * 16 * kFmRow + 2 * c) = w[k];
+            }
+        };
+        if (warp == 0) { leave(acc[0]); invert(0); }
 #pragma unroll 1
         for (int kb = 0; kb < nt; ++kb) {
-            // (a) publish M_PP and the C_i
+            const float* Gk = Gs + (kb & 1) * 16 * 17;
+            const uint32_t gk = gbase + (kb & 1) * 3 * 16 * kFmRow;
+            // (a) publish the C_i
 #pragma unroll
-            for (int q = 0; q < TPW; ++q) {
-                if (ti[q] < 0) break;
-                if (ti[q] == kb && tj[q] == kb) {
-#pragma unroll
-                    for (int e = 0; e < 8; ++e) D[(g + 8 * ((e >> 1) & 1)) * 17 + 8 * (e >> 2) + 2 * t + (e & 1)] = acc[q][e];
-                } else if (tj[q] == kb) {                     // C_i = M_iP
+            for (int q = ND; q < TPW; ++q) {
+                if (ti[q] < 0) continue;
+                if (tj[q] == kb) {                     // C_i = M_iP
 #pragma unroll
                     for (int h = 0; h < 4; ++h) {             // pairs: (row half h & 1, column half h >> 1)
                         uint32_t p[3];
@@ -142,45 +196,14 @@ k_block_factor_mma(const SubInfo* __restrict__ subs, const int* __restrict__ lis
                 }
             }
             __syncthreads();
-            // (b) G = M_PP^{-1}: lane r + 16 h holds columns 8 h .. 8 h + 7 of row r
-            if (warp == kb % NW) {
-                const int r = lane & 15, h = lane >> 4;
-                float a[8];
-#pragma unroll
-                for (int c = 0; c < 8; ++c) a[c] = D[r * 17 + 8 * h + c];
-#pragma unroll
-                for (int q = 0; q < 16; ++q) {
-                    const int ql = q & 7, qh = q >> 3;
-                    float p = __shfl_sync(0xffffffffu, a[ql], q + 16 * qh);
-                    const float cr = __shfl_sync(0xffffffffu, a[ql], r + 16 * qh);
-                    if (!(p > 0.0f)) { bad = 1; p = 1.0f; }
-                    const float inv = 1.0f / p;
-#pragma unroll
-                    for (int c = 0; c < 8; ++c) {
-                        const float rq = __shfl_sync(0xffffffffu, a[c], q + 16 * h) * inv;
-                        if (r == q) a[c] = rq; else a[c] = fmaf(-cr, rq, a[c]);
-                    }
-                    if (h == qh) a[ql] = r == q ? inv : -cr * inv;
-                }
-#pragma unroll
-                for (int c = 0; c < 8; c += 2) {
-                    Gs[r * 17 + 8 * h + c] = a[c];
-                    Gs[r * 17 + 8 * h + c + 1] = a[c + 1];
-                    uint32_t p[3];
-                    cut3(a[c], a[c + 1], p[0], p[1], p[2]);
-#pragma unroll
-                    for (int k = 0; k < 3; ++k) *reinterpret_cast<uint32_t*>(Gp + k * 16 * kFmRow + r * kFmRow + 16 * h + 2 * c) = p[k];
-                }
-            }
-            __syncthreads();
-            // (c) A_i = C_i G
+            // (b) A_i = C_i G
             for (int i = warp; i < nt; i += NW) {
                 if (i == kb) continue;
                 uint32_t ca[3][4], gb[3][4];
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
                     ldsm4(cbase + k * cpl + (uint32_t)(16 * i) * kFmRow + la, ca[k]);
-                    ldsm4(gbase + k * 16 * kFmRow + lb, gb[k]);
+                    ldsm4(gk + k * 16 * kFmRow + lb, gb[k]);
                 }
                 float t0[4] = {0.f, 0.f, 0.f, 0.f}, t1[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
@@ -202,16 +225,17 @@ k_block_factor_mma(const SubInfo* __restrict__ subs, const int* __restrict__ lis
                 o[8] = t1[0]; o[9] = t1[1]; o[8 * 17 + 8] = t1[2]; o[8 * 17 + 9] = t1[3];
             }
             __syncthreads();
-            // (d) the tiles
+            // (c) the tiles; the next diagonal one first, whose warp then inverts it
 #pragma unroll
             for (int q = 0; q < TPW; ++q) {
-                if (ti[q] < 0) break;
+                if (q == ND && kb + 1 < nt && warp == (kb + 1) % NW) invert((kb + 1) & 1);
+                if (ti[q] < 0) continue;
                 const int i = ti[q], j = tj[q];
                 if (i == kb || j == kb) {
 #pragma unroll
                     for (int e = 0; e < 8; ++e) {
                         const int r = g + 8 * ((e >> 1) & 1), c = 8 * (e >> 2) + 2 * t + (e & 1);
-                        acc[q][e] = i == j ? Gs[r * 17 + c] : j == kb ? -Ap[i * 16 * 17 + r * 17 + c] : -Ap[j * 16 * 17 + c * 17 + r];
+                        acc[q][e] = i == j ? Gk[r * 17 + c] : j == kb ? -Ap[i * 16 * 17 + r * 17 + c] : -Ap[j * 16 * 17 + c * 17 + r];
                     }
                     continue;
                 }
@@ -233,6 +257,7 @@ k_block_factor_mma(const SubInfo* __restrict__ subs, const int* __restrict__ lis
                 const float sg = j < kb ? 1.0f : -1.0f;       // -sigma_j
 #pragma unroll
                 for (int e = 0; e < 4; ++e) { acc[q][e] = fmaf(sg, t0[e], acc[q][e]); acc[q][4 + e] = fmaf(sg, t1[e], acc[q][4 + e]); }
+                if (q < ND && i == kb + 1) leave(acc[q]);
             }
             __syncthreads();                                  // the step's planes are read
         }
@@ -242,7 +267,7 @@ k_block_factor_mma(const SubInfo* __restrict__ subs, const int* __restrict__ lis
         float* T = reinterpret_cast<float*>(Cp) + warp * 16 * 17;
 #pragma unroll
         for (int q = 0; q < TPW; ++q) {
-            if (ti[q] < 0) break;
+            if (ti[q] < 0) continue;
             const int i = ti[q], j = tj[q];
             float v[8];
 #pragma unroll

@@ -2098,9 +2098,16 @@ static void launch_factor64(const SubInfo* subs, const int* list, int n, int bma
     MRCM_LAUNCH(P, name, st, cudaLaunchKernelExC(&cfg, k, args));
 }
 
-// CTA shape of k_block_factor_mma: 8 warps of up to 5 tiles (b <= 128: 36 tiles), 16 of 5
-// (b <= 192: 78) or 16 of 9 (136).
-static int factor_mma_shape(int b) { return b <= 128 ? 0 : b <= 192 ? 1 : 2; }
+// CTA shape of k_block_factor_mma by the number of tile rows: as few warps as hold the
+// tiles in registers, so that as many blocks as possible are in flight on an SM (the step
+// is a chain; 8 warps of 5 tiles for b = 128, three CTAs, took 17.3 ms where 4 of 9, four
+// CTAs, take 16.0): nt <= 8: 4 warps of 2 + 7, nt = 9: 8 of 2 + 5, nt <= 12: 16 of 1 + 5,
+// nt <= 16: 16 of 1 + 8.
+static int factor_mma_shape(int b) { return b <= 128 ? 0 : b <= 144 ? 1 : b <= 192 ? 2 : 3; }
+static const void* factor_mma_kernel(int shape) {
+    return shape == 0 ? (const void*)k_block_factor_mma<4, 9, 2, 4> : shape == 1 ? (const void*)k_block_factor_mma<8, 7, 2, 2>
+         : shape == 2 ? (const void*)k_block_factor_mma<16, 6, 1, 1> : (const void*)k_block_factor_mma<16, 9, 1, 1>;
+}
 
 static void launch_factor_wave(const Tables& t, const DeviceTables& d, const Layout& L, char* ws, int precision,
                                int w, cudaStream_t st, Prof& P) {
@@ -2149,12 +2156,11 @@ static void launch_factor_wave(const Tables& t, const DeviceTables& d, const Lay
             const size_t sm = factor_mma_smem(b0);
             if (shape == 0 && d.factor_mid_variant == 1)    // its shared memory keeps <= 4 CTAs (4 x 128 TMEM columns) per SM
                 MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_tc<<<n, kTcN, kTcSmem, st>>>(d.subs, lst, coef, scale, W, status, t.n_cells, scf, tsc));
-            else if (shape == 0)
-                MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_mma<8, 5><<<n, 256, sm, st>>>(d.subs, lst, coef, scale, W, status, t.n_cells, scf, tsc));
-            else if (shape == 1)
-                MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_mma<16, 5><<<n, 512, sm, st>>>(d.subs, lst, coef, scale, W, status, t.n_cells, scf, tsc));
-            else
-                MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_mma<16, 9><<<n, 512, sm, st>>>(d.subs, lst, coef, scale, W, status, t.n_cells, scf, tsc));
+            else {
+                const void* k = factor_mma_kernel(shape);
+                void* args[] = {(void*)&d.subs, (void*)&lst, (void*)&coef, (void*)&scale, (void*)&W, (void*)&status, (void*)&t.n_cells, (void*)&scf, (void*)&tsc};
+                MRCM_LAUNCH(P, "k_block_factor", st, cudaLaunchKernel(k, dim3(n), dim3(shape == 0 ? 128 : shape == 1 ? 256 : 512), args, sm, st));
+            }
             q = e;
         }
         (void)n_mid;
@@ -2274,9 +2280,8 @@ int configure_local(const Tables& t, DeviceTables& d) {
         d.f64_occ = std::max(1, occ);
     }
     cudaFuncSetAttribute(k_block_factor_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
-    cudaFuncSetAttribute(k_block_factor_mma<8, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)factor_mma_smem(128));
-    cudaFuncSetAttribute(k_block_factor_mma<16, 5>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)factor_mma_smem(192));
-    cudaFuncSetAttribute(k_block_factor_mma<16, 9>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)factor_mma_smem(256));
+    for (int b : {128, 144, 192, 256})
+        cudaFuncSetAttribute(factor_mma_kernel(factor_mma_shape(b)), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)factor_mma_smem(b));
     return (int)cudaGetLastError();
 }
 
