@@ -827,60 +827,57 @@ __device__ __forceinline__ void slab_coords(const SubInfo& s, int c, int lc[3]) 
     lc[s.va] = v;
 }
 
+// One CTA per subdomain and part: part y writes the columns c = y (mod gridDim.y).
+// The FP64 logarithms (what bounds the gather: about 40 FP64 instructions each) are
+// taken once per CTA, not once per column.  32 subdomains of 500 cells, 896
+// samples: 331 us with one CTA per subdomain and the logarithms per column, 31 us now.
 __global__ void __launch_bounds__(256)
 k_gather_samples(const SubInfo* __restrict__ subs, const FaceInfo* __restrict__ faces, const int* __restrict__ soff,
                  const double* __restrict__ K, const double* __restrict__ X, int nx, int ny, long long ncells,
                  int max_samples, float* __restrict__ xs, float* __restrict__ ts) {
+    extern __shared__ __align__(16) float sm[];
     const SubInfo s = subs[blockIdx.x];
     const int base = soff[blockIdx.x];
-    if (base < 0) return;
+    if (base < 0 || (int)blockIdx.y >= s.nI || base + (int)blockIdx.y >= max_samples) return;
     const int N = s.N;
-    for (int c = 0; c < s.nI; ++c) {
-        const int smp = base + c;
-        if (smp >= max_samples) return;
-        float* xin = xs + (long long)smp * 4 * N;
-        float* tg = ts ? ts + (long long)smp * N : nullptr;
-        for (int e = threadIdx.x; e < N; e += blockDim.x) {
-            int lc[3];
-            slab_coords(s, e, lc);
-            const int lex = lc[0] + s.sz[0] * (lc[1] + s.sz[1] * lc[2]);
-            const long long gcell = (s.o[0] + lc[0]) + (long long)nx * ((s.o[1] + lc[1]) + (long long)ny * (s.o[2] + lc[2]));
-            xin[lex] = kLogKScale * (float)log(K[gcell]);
-            xin[N + lex] = kLogKScale * (float)log(K[2 * ncells + gcell]);
-            xin[2 * N + lex] = 0.0f;
-            xin[3 * N + lex] = 0.0f;
-            if (tg) tg[lex] = (float)X[s.x_off + (long long)c * N + e];
-        }
-        __syncthreads();
-        for (int q = threadIdx.x; q < s.nface; q += blockDim.x) {
-            const FaceInfo fi = faces[s.face_off + q];
-            int lc[3];
-            slab_coords(s, fi.cell, lc);
-            const int lex = lc[0] + s.sz[0] * (lc[1] + s.sz[1] * lc[2]);
-            if (fi.col == c) xin[2 * N + lex] = 1.0f;            // one face per cell for a basis
-        }
-        __syncthreads();
-    }
-}
-
-// Robin mask: cells with at least one Robin face (the same for every sample
-// of a subdomain), written after the gather for each sample.
-__global__ void __launch_bounds__(256)
-k_gather_mask(const SubInfo* __restrict__ subs, const FaceInfo* __restrict__ faces, const int* __restrict__ soff,
-              int max_samples, float* __restrict__ xs) {
-    const SubInfo s = subs[blockIdx.x];
-    const int base = soff[blockIdx.x];
-    if (base < 0) return;
-    const int N = s.N;
-    for (int q = threadIdx.x; q < s.nface; q += blockDim.x) {
-        const FaceInfo fi = faces[s.face_off + q];
+    float* lx = sm;                                            // log Kx, log Kz (scaled), Robin mask, this column's
+    float* lz = lx + N;                                        // faces, by box-lexicographic cell
+    float* mask = lz + N;
+    float* ind = mask + N;
+    auto lex_of = [&](int cell) {
         int lc[3];
-        slab_coords(s, fi.cell, lc);
-        const int lex = lc[0] + s.sz[0] * (lc[1] + s.sz[1] * lc[2]);
-        for (int c = 0; c < s.nI; ++c) {
-            const int smp = base + c;
-            if (smp < max_samples) xs[(long long)smp * 4 * N + 3 * N + lex] = 1.0f;
+        slab_coords(s, cell, lc);
+        return lc[0] + s.sz[0] * (lc[1] + s.sz[1] * lc[2]);
+    };
+    for (int e = threadIdx.x; e < N; e += blockDim.x) {
+        const int z = e / (s.sz[0] * s.sz[1]), r = e - z * s.sz[0] * s.sz[1], y = r / s.sz[0], x = r - y * s.sz[0];
+        const long long gcell = (s.o[0] + x) + (long long)nx * ((s.o[1] + y) + (long long)ny * (s.o[2] + z));
+        lx[e] = kLogKScale * (float)log(K[gcell]);
+        lz[e] = kLogKScale * (float)log(K[2 * ncells + gcell]);
+        mask[e] = 0.0f;
+        ind[e] = 0.0f;
+    }
+    __syncthreads();
+    for (int q = threadIdx.x; q < s.nface; q += blockDim.x) mask[lex_of(faces[s.face_off + q].cell)] = 1.0f;
+    for (int c = blockIdx.y; c < s.nI && base + c < max_samples; c += gridDim.y) {
+        for (int q = threadIdx.x; q < s.nface; q += blockDim.x) {   // one face per cell for a basis
+            const FaceInfo fi = faces[s.face_off + q];
+            if (fi.col == c) ind[lex_of(fi.cell)] = 1.0f;
         }
+        __syncthreads();
+        float* xin = xs + (long long)(base + c) * 4 * N;
+        for (int e = threadIdx.x; e < N; e += blockDim.x) {
+            xin[e] = lx[e];
+            xin[N + e] = lz[e];
+            xin[2 * N + e] = ind[e];
+            xin[3 * N + e] = mask[e];
+            ind[e] = 0.0f;
+        }
+        if (ts) {
+            float* tg = ts + (long long)(base + c) * N;
+            for (int e = threadIdx.x; e < N; e += blockDim.x) tg[lex_of(e)] = (float)X[s.x_off + (long long)c * N + e];
+        }
+        __syncthreads();
     }
 }
 
@@ -1022,17 +1019,18 @@ k_pcg_sample(const SubInfo* __restrict__ subs, const FaceInfo* __restrict__ face
 // constant on the patch), zero for the particular column.  A column whose
 // FP64 residual reaches ||r|| <= tol ||b|| gets conv = 1; the others are left
 // to the FP64 direct fallback.
-__device__ __forceinline__ double block_sum_d(double v, double* red) {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-    __syncthreads();
-    if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = v;
-    __syncthreads();
-    double t = 0.0;
-    for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
-    return t;
-}
-
-__global__ void __launch_bounds__(256)
+//
+// Four cells a thread, T threads (T = 128 covers 512 cells, 1024 all of them):
+// the vectors and each cell's seven couplings stay in registers, only the search
+// direction goes through shared memory (with b zero cells on both sides, so no
+// bounds tests), three barriers a CG step.  Bound: the step's latency chain (two
+// reductions) and its ~110 instructions a warp.  1824 columns of 500 cells, 122
+// steps each: 933 us with couplings in shared memory and two cells a thread (an
+// index division per neighbour test, eight barriers a step), 1022 us with a warp
+// per column and 16 cells a lane, 342 us now.
+constexpr int kLcCells = 4;
+template <int T>
+__global__ void __launch_bounds__(T)
 k_learned_column(const SubInfo* __restrict__ subs, const FaceInfo* __restrict__ faces, const int* __restrict__ col_list,
                  const double* __restrict__ coef, const double* __restrict__ scale,
                  const double* __restrict__ face_tr, const double* __restrict__ face_u,
@@ -1041,136 +1039,174 @@ k_learned_column(const SubInfo* __restrict__ subs, const FaceInfo* __restrict__ 
                  const int* __restrict__ soff, const float* __restrict__ pred, int n_pred, int cg_maxit,
                  int max_outer, double tol, double* __restrict__ X, int* __restrict__ conv, int* __restrict__ status) {
     extern __shared__ __align__(16) unsigned char lsm[];
+    constexpr int NWP = T / 32;
     const int l = col_list[2 * blockIdx.x], j = col_list[2 * blockIdx.x + 1];
     const SubInfo s = subs[l];
     const int N = s.N, b = s.b, su = s.su, nI = s.nI, m = s.m;
-    double* x = reinterpret_cast<double*>(lsm);
-    double* bb = x + N;
-    float* dd = reinterpret_cast<float*>(bb + N);
-    float* tu = dd + N;
-    float* tv = tu + N;
-    float* ts = tv + N;
-    float* z = ts + N;
-    float* r = z + N;
-    float* p = r + N;
-    float* q = p + N;
-    __shared__ float red[32];
-    __shared__ double redd[32];
-    __shared__ double wscale_s;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    double* x = reinterpret_cast<double*>(lsm) + b;                           // index c in [-b, N + b)
+    float* ps = reinterpret_cast<float*>(lsm + sizeof(double) * (size_t)(N + 2 * b)) + b;
+    __shared__ double redd[NWP];
+    __shared__ __align__(16) float red[2][NWP < 4 ? 4 : NWP];
     const double* cd = coef + s.cell_off;
     const double* cu = coef + nct + s.cell_off;
     const double* cv = coef + 2 * nct + s.cell_off;
     const double* cs = coef + 3 * nct + s.cell_off;
     const double* sc = scale + s.cell_off;
-    for (int c = threadIdx.x; c < N; c += blockDim.x) {
-        const int i = c % b, u = i % su;
-        dd[c] = (float)(cd[c] * sc[c] * sc[c]);
-        tu[c] = u + 1 < su ? (float)(cu[c] * sc[c] * sc[c + 1]) : 0.0f;
-        tv[c] = i + su < b ? (float)(cv[c] * sc[c] * sc[c + su]) : 0.0f;
-        ts[c] = c + b < N ? (float)(cs[c] * sc[c] * sc[c + b]) : 0.0f;
-        double bv = 0.0;
-        if (j == m - 1) {
-            int lc[3];
-            slab_coords(s, c, lc);
-            const long long g = (s.o[0] + lc[0]) + (long long)nx * ((s.o[1] + lc[1]) + (long long)ny * (s.o[2] + lc[2]));
-            bv = rhs_part[s.cell_off + c] + f[g] * vol;
-        }
-        bb[c] = bv;
-        x[c] = 0.0;
-    }
-    if (threadIdx.x == 0) wscale_s = 1.0;
-    __syncthreads();
-    const int pc = j < nI ? j : (j < 2 * nI ? j - nI : -1);       // the basis of an MBF column
-    if (j < m - 1) {
-        for (int e = threadIdx.x; e < s.nface; e += blockDim.x) {
-            const FaceInfo fi = faces[s.face_off + e];
-            if (fi.col != pc) continue;
-            bb[fi.cell] = j < nI ? face_tr[s.face_off + e] : face_u[s.face_off + e];
-            if (j >= nI) wscale_s = -face_beta[s.face_off + e] * fi.s;    // any face of the basis (a benign race)
-        }
-    }
-    __syncthreads();
-    if (pred && soff && pc >= 0 && soff[l] >= 0 && soff[l] + pc < n_pred) {
-        const float* pr = pred + (long long)(soff[l] + pc) * N;
-        const double ws = j < nI ? 1.0 : wscale_s;
-        for (int c = threadIdx.x; c < N; c += blockDim.x) {
-            int lc[3];
-            slab_coords(s, c, lc);
-            x[c] = ws * (double)pr[lc[0] + s.sz[0] * (lc[1] + s.sz[1] * lc[2])];
-        }
-    }
-    __syncthreads();
-    auto matvec = [&](const float* v, float* out) {
-        for (int c = threadIdx.x; c < N; c += blockDim.x) {
-            const int i = c % b, u = i % su;
-            float a = dd[c] * v[c];
-            if (u + 1 < su) a -= tu[c] * v[c + 1];
-            if (u > 0) a -= tu[c - 1] * v[c - 1];
-            if (i + su < b) a -= tv[c] * v[c + su];
-            if (i >= su) a -= tv[c - su] * v[c - su];
-            if (c + b < N) a -= ts[c] * v[c + b];
-            if (c >= b) a -= ts[c - b] * v[c - b];
-            out[c] = a;
-        }
-    };
-    auto dot = [&](const float* a, const float* bv) -> float {
-        float acc = 0.0f;
-        for (int c = threadIdx.x; c < N; c += blockDim.x) acc = fmaf(a[c], bv[c], acc);
-        for (int o = 16; o > 0; o >>= 1) acc += __shfl_down_sync(0xffffffffu, acc, o);
+    auto sum_d = [&](double v) {
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
         __syncthreads();
-        if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
+        if (lane == 0) redd[warp] = v;
         __syncthreads();
-        float t = 0.0f;
-        for (int w = 0; w < (int)(blockDim.x >> 5); ++w) t += red[w];
+        double t = 0.0;
+        for (int w = 0; w < NWP; ++w) t += redd[w];
         return t;
     };
-    double bn = 0.0;
-    for (int c = threadIdx.x; c < N; c += blockDim.x) bn += bb[c] * bb[c];
-    bn = block_sum_d(bn, redd);
-    long long iters = 0;
-    int ok = 0;
+    auto sum_f = [&](float v, int buf) {                 // the two buffers alternate: one barrier
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+        if (lane == 0) red[buf][warp] = v;
+        __syncthreads();
+        float t = 0.0f;
+#pragma unroll
+        for (int w = 0; w < NWP; w += 4) {
+            const float4 q = *reinterpret_cast<const float4*>(&red[buf][w]);
+            t += (q.x + q.y) + (q.z + q.w);
+        }
+        return t;
+    };
+    static_assert(NWP % 4 == 0, "sum_f reads four partial sums at a time");
+    // first iterate and right-hand side (through shared memory: faces are scattered)
+    const int pc = j < nI ? j : (j < 2 * nI ? j - nI : -1);       // the basis of an MBF column
+    for (int c = tid - b; c < N + b; c += T) { x[c] = 0.0; ps[c] = 0.0f; }
+    __syncthreads();
+    double ws = 1.0;
+    if (pc >= 0) {
+        int last = -1;                                   // any face of the basis: the last one in face order
+        for (int e = tid; e < s.nface; e += T) {
+            const FaceInfo fi = faces[s.face_off + e];
+            if (fi.col != pc) continue;
+            x[fi.cell] = j < nI ? face_tr[s.face_off + e] : face_u[s.face_off + e];
+            last = e;
+        }
+        if (j >= nI) {
+            for (int o = 16; o > 0; o >>= 1) last = max(last, __shfl_xor_sync(0xffffffffu, last, o));
+            if (lane == 0) redd[warp] = (double)last;
+            __syncthreads();
+            for (int w = 0; w < NWP; ++w) last = max(last, (int)redd[w]);
+            if (last >= 0) ws = -face_beta[s.face_off + last] * faces[s.face_off + last].s;
+        }
+    }
+    __syncthreads();
+    const bool guess = pred && soff && pc >= 0 && soff[l] >= 0 && soff[l] + pc < n_pred;
+    const float* pr = guess ? pred + (long long)(soff[l] + pc) * N : nullptr;
+    double bb[kLcCells], bn = 0.0;
+    float d[kLcCells], up[kLcCells], um[kLcCells], vp[kLcCells], vm[kLcCells], sp[kLcCells], sm[kLcCells];
+    unsigned nbr = 0;                                    // in-slab neighbours of each cell (+u, -u, +v, -v), four bits a cell
+#pragma unroll
+    for (int k = 0; k < kLcCells; ++k) {
+        const int c = tid + T * k;
+        bb[k] = 0.0;
+        d[k] = up[k] = um[k] = vp[k] = vm[k] = sp[k] = sm[k] = 0.0f;
+        if (c < N) {
+            const int i = c % b, u = i % su;
+            const double sx = sc[c];
+            if (u + 1 < su) nbr |= 1u << (4 * k);
+            if (u > 0) nbr |= 2u << (4 * k);
+            if (i + su < b) nbr |= 4u << (4 * k);
+            if (i >= su) nbr |= 8u << (4 * k);
+            d[k] = (float)(cd[c] * sx * sx);
+            if (u + 1 < su) up[k] = (float)(cu[c] * sx * sc[c + 1]);
+            if (u > 0) um[k] = (float)(cu[c - 1] * sc[c - 1] * sx);
+            if (i + su < b) vp[k] = (float)(cv[c] * sx * sc[c + su]);
+            if (i >= su) vm[k] = (float)(cv[c - su] * sc[c - su] * sx);
+            if (c + b < N) sp[k] = (float)(cs[c] * sx * sc[c + b]);
+            if (c >= b) sm[k] = (float)(cs[c - b] * sc[c - b] * sx);
+            bb[k] = x[c];
+            int lc[3];
+            slab_coords(s, c, lc);
+            if (j == m - 1) {
+                const long long g = (s.o[0] + lc[0]) + (long long)nx * ((s.o[1] + lc[1]) + (long long)ny * (s.o[2] + lc[2]));
+                bb[k] = rhs_part[s.cell_off + c] + f[g] * vol;
+            }
+            x[c] = guess ? ws * (double)pr[lc[0] + s.sz[0] * (lc[1] + s.sz[1] * lc[2])] : 0.0;   // (own cells only)
+        }
+        bn = fma(bb[k], bb[k], bn);
+    }
+    bn = sum_d(bn);                                      // (its barriers publish x)
+    int iters = 0, ok = 0;
+    float r[kLcCells], p[kLcCells], z[kLcCells];
     for (int o = 0; o <= max_outer; ++o) {
         // FP64 residual of the unscaled system, the scaled right-hand side of the correction
         double rr = 0.0;
-        for (int c = threadIdx.x; c < N; c += blockDim.x) {
-            const int i = c % b, u = i % su;
-            double a = cd[c] * x[c];
-            if (u + 1 < su) a = fma(-cu[c], x[c + 1], a);
-            if (u > 0) a = fma(-cu[c - 1], x[c - 1], a);
-            if (i + su < b) a = fma(-cv[c], x[c + su], a);
-            if (i >= su) a = fma(-cv[c - su], x[c - su], a);
-            if (c + b < N) a = fma(-cs[c], x[c + b], a);
-            if (c >= b) a = fma(-cs[c - b], x[c - b], a);
-            const double res = bb[c] - a;
-            rr = fma(res, res, rr);
-            r[c] = (float)(res * sc[c]);
-            z[c] = 0.0f;
-            p[c] = r[c];
+        float rho = 0.0f;
+#pragma unroll
+        for (int k = 0; k < kLcCells; ++k) {
+            const int c = tid + T * k;
+            r[k] = z[k] = 0.0f;
+            if (c < N) {
+                const unsigned nb = nbr >> (4 * k);
+                double a = cd[c] * x[c];
+                if (nb & 1u) a = fma(-cu[c], x[c + 1], a);
+                if (nb & 2u) a = fma(-cu[c - 1], x[c - 1], a);
+                if (nb & 4u) a = fma(-cv[c], x[c + su], a);
+                if (nb & 8u) a = fma(-cv[c - su], x[c - su], a);
+                if (c + b < N) a = fma(-cs[c], x[c + b], a);
+                if (c >= b) a = fma(-cs[c - b], x[c - b], a);
+                const double res = bb[k] - a;
+                rr = fma(res, res, rr);
+                r[k] = (float)(res * sc[c]);
+            }
+            p[k] = r[k];
+            rho = fmaf(r[k], r[k], rho);
         }
-        rr = block_sum_d(rr, redd);
+        rr = sum_d(rr);
         if (rr <= tol * tol * bn) { ok = 1; break; }
         if (o == max_outer) break;
-        float rho = dot(r, r);
+        rho = sum_f(rho, 1);
         const float stop = 1e-8f * rho;                  // relative residual 1e-4
-        for (int k = 0; k < cg_maxit && rho > stop; ++k) {
-            matvec(p, q);
+        for (int it = 0; it < cg_maxit && rho > stop; ++it) {
+#pragma unroll
+            for (int k = 0; k < kLcCells; ++k) if (tid + T * k < N) ps[tid + T * k] = p[k];
             __syncthreads();
-            const float alpha = rho / dot(p, q);
-            for (int c = threadIdx.x; c < N; c += blockDim.x) { z[c] = fmaf(alpha, p[c], z[c]); r[c] = fmaf(-alpha, q[c], r[c]); }
-            __syncthreads();
-            const float rho2 = dot(r, r);
+            float q[kLcCells], pq = 0.0f;
+#pragma unroll
+            for (int k = 0; k < kLcCells; ++k) {
+                const int c = min(tid + T * k, N - 1);   // (zero couplings past the end)
+                float a = d[k] * p[k];
+                a = fmaf(-up[k], ps[c + 1], a);
+                a = fmaf(-um[k], ps[c - 1], a);
+                a = fmaf(-vp[k], ps[c + su], a);
+                a = fmaf(-vm[k], ps[c - su], a);
+                a = fmaf(-sp[k], ps[c + b], a);
+                a = fmaf(-sm[k], ps[c - b], a);
+                q[k] = a;
+                pq = fmaf(p[k], a, pq);
+            }
+            const float alpha = rho / sum_f(pq, 0);
+            float rho2 = 0.0f;
+#pragma unroll
+            for (int k = 0; k < kLcCells; ++k) {
+                z[k] = fmaf(alpha, p[k], z[k]);
+                r[k] = fmaf(-alpha, q[k], r[k]);
+                rho2 = fmaf(r[k], r[k], rho2);
+            }
+            rho2 = sum_f(rho2, 1);
             const float beta = rho2 / rho;
             rho = rho2;
-            for (int c = threadIdx.x; c < N; c += blockDim.x) p[c] = fmaf(beta, p[c], r[c]);
-            __syncthreads();
+#pragma unroll
+            for (int k = 0; k < kLcCells; ++k) p[k] = fmaf(beta, p[k], r[k]);
             ++iters;
         }
-        for (int c = threadIdx.x; c < N; c += blockDim.x) x[c] = fma((double)z[c], sc[c], x[c]);
+#pragma unroll
+        for (int k = 0; k < kLcCells; ++k) {
+            const int c = tid + T * k;
+            if (c < N) x[c] = fma((double)z[k], sc[c], x[c]);
+        }
         __syncthreads();
     }
     double* Xc = X + s.x_off + (long long)j * N;
-    for (int c = threadIdx.x; c < N; c += blockDim.x) Xc[c] = x[c];
-    if (threadIdx.x == 0) {
+    for (int c = tid; c < N; c += T) Xc[c] = x[c];       // (own cells)
+    if (tid == 0) {
         conv[s.rhs_off + j] = ok;
         atomicAdd(reinterpret_cast<unsigned long long*>(status + ST_CG_ITERS), (unsigned long long)iters);
     }
@@ -1232,9 +1268,12 @@ mrcm_status mrcm_net_samples(mrcm_handle* h, const mrcm_net* net, void* ws, floa
     if (!x || *n_samples == 0) return MRCM_OK;
     const mrcm::Tables& t = h->t;
     cudaStream_t s = (cudaStream_t)stream;
-    mrcm::k_gather_samples<<<(int)t.subs.size(), 256, 0, s>>>(h->d.subs, h->d.faces, soff, h->K,
+    // parts per subdomain: two CTAs per SM when the subdomains are few
+    const int nsub = (int)t.subs.size(), parts = std::max(1, std::min(32, (2 * h->d.sms + nsub - 1) / nsub));
+    const size_t sm = sizeof(float) * 4 * (size_t)net->S;
+    cudaFuncSetAttribute(mrcm::k_gather_samples, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    mrcm::k_gather_samples<<<dim3(nsub, parts), 256, sm, s>>>(h->d.subs, h->d.faces, soff, h->K,
         (const double*)((char*)ws + h->lay.X), t.cfg.nx, t.cfg.ny, t.n_cells, max_samples, x, target);
-    mrcm::k_gather_mask<<<(int)t.subs.size(), 256, 0, s>>>(h->d.subs, h->d.faces, soff, max_samples, x);
     return cudaGetLastError() == cudaSuccess ? MRCM_OK : MRCM_ERR_CUDA;
 }
 
@@ -1280,15 +1319,28 @@ mrcm_status mrcm_solve_mbf_learned(mrcm_handle* h, const mrcm_net* net, const fl
     char* w = (char*)ws;
     int* status = (int*)(w + h->lay.status);
     cudaMemsetAsync(status, 0, sizeof(int) * mrcm::ST_COUNT, st);
-    const size_t sm = (size_t)t.max_N * (2 * sizeof(double) + 8 * sizeof(float));
-    cudaFuncSetAttribute(mrcm::k_learned_column, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
     const double tol = t.cfg.ir_tol > 0 ? t.cfg.ir_tol : 1e-9;
-    if (h->n_cols > 0)
-        mrcm::k_learned_column<<<h->n_cols, 256, sm, st>>>(h->d.subs, h->d.faces, h->col_list,
-            (const double*)(w + h->lay.coef), (const double*)(w + h->lay.scale), (const double*)(w + h->lay.face_tr),
-            (const double*)(w + h->lay.face_u), (const double*)(w + h->lay.face_beta),
-            (const double*)(w + h->lay.rhs_part), f, t.cfg.nx, t.cfg.ny, t.cfg.hx * t.cfg.hy * t.cfg.hz, t.n_cells,
-            soff, pred, n_pred, cg_maxit, max_outer, tol, (double*)(w + h->lay.X), (int*)(w + h->lay.conv), status);
+    if (h->n_cols > 0) {
+        const int T = t.max_N <= 512 ? 128 : t.max_N <= 1024 ? 256 : t.max_N <= 2048 ? 512 : 1024;
+        const void* k = T == 128 ? (const void*)mrcm::k_learned_column<128> : T == 256 ? (const void*)mrcm::k_learned_column<256>
+                      : T == 512 ? (const void*)mrcm::k_learned_column<512> : (const void*)mrcm::k_learned_column<1024>;
+        size_t sm = 0;
+        for (const mrcm::SubInfo& sb : t.subs) sm = std::max(sm, (sizeof(double) + sizeof(float)) * ((size_t)sb.N + 2 * sb.b));
+        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        const int* list = h->col_list;
+        const double *coef = (const double*)(w + h->lay.coef), *scale = (const double*)(w + h->lay.scale),
+                     *ftr = (const double*)(w + h->lay.face_tr), *fu = (const double*)(w + h->lay.face_u),
+                     *fbe = (const double*)(w + h->lay.face_beta), *rp = (const double*)(w + h->lay.rhs_part);
+        double vol = t.cfg.hx * t.cfg.hy * t.cfg.hz;
+        double* X = (double*)(w + h->lay.X);
+        int* conv = (int*)(w + h->lay.conv);
+        long long nct = t.n_cells;
+        int nx = t.cfg.nx, ny = t.cfg.ny;
+        double tol_ = tol;
+        void* args[] = {&h->d.subs, &h->d.faces, &list, &coef, &scale, &ftr, &fu, &fbe, &rp, &f, &nx, &ny, &vol, &nct,
+                        &soff, &pred, &n_pred, &cg_maxit, &max_outer, &tol_, &X, &conv, &status};
+        cudaLaunchKernel(k, dim3(h->n_cols), dim3(T), args, sm, st);
+    }
     int rc = mrcm::launch_local_finish(t, h->d, h->lay, w, f, stream, h->prof);
     if (rc != 0 || cudaGetLastError() != cudaSuccess) { h->err = "mrcm_solve_mbf_learned: launch failed"; return MRCM_ERR_CUDA; }
     h->stage = 2;
