@@ -30,7 +30,12 @@
 // extend-add of the two children (subdomain blocks at the leaves), partially
 // factored by a blocked right-looking LDL^T (32-column panels, 64x64 update
 // tiles spread over the whole GPU), and leave the Schur complement on B for
-// their parent.  The solution is refined once in FP64 with CSR residuals.
+// their parent.  The right-hand side b^int goes along as one more row of every
+// front (row n: the panels turn its E part into D^{-1} L^{-1} b, the updates reduce
+// its B part for the parent), so that the solve after a factorisation has only the
+// backward substitution left: the forward one, a launch pair per level with little
+// work in each, took 0.5 of 1.0 ms at 60 x 220 x 85.  The solution can be refined in
+// FP64 with CSR residuals; those right-hand sides go through k_front_forward.
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -61,17 +66,26 @@ __global__ void k_assemble_csr(int nrows, const int* __restrict__ rowptr, const 
                                double* __restrict__ val, double* __restrict__ b, double* __restrict__ dscale,
                                int pin) {
     pdl_begin();
-    int r = blockIdx.x * blockDim.x + threadIdx.x;
+    // a warp per row (a thread per row left 100 dependent loads in a chain on a few CTAs: 64 us for
+    // 704 rows, 38 us for 32,944)
+    const int r = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (r >= nrows) return;
     double diag = 0.0, rowmax = 0.0;
-    for (int q = rowptr[r]; q < rowptr[r + 1]; ++q) {
-        double v = 0.0;
-        if (src_lo[q] >= 0) v += elem[src_lo[q]];
-        if (src_hi[q] >= 0) v += elem[src_hi[q]];
+    const bool need_max = pin && r == 0;
+    for (int q = rowptr[r] + lane; q < rowptr[r + 1]; q += 32) {
+        const long long lo = src_lo[q], hi = src_hi[q];
+        double v = lo >= 0 ? elem[lo] : hi >= 0 ? elem[hi] : 0.0;
+        if (lo >= 0 && hi >= 0) v += elem[hi];
         val[q] = v;
         if (colidx[q] == r) diag = v;
-        rowmax = fmax(rowmax, fabs(v));
+        if (need_max) rowmax = fmax(rowmax, fabs(v));
     }
+    for (int o = 16; o > 0; o >>= 1) {                    // (at most one lane holds the diagonal)
+        const double dd = __shfl_xor_sync(0xffffffffu, diag, o);
+        if (__double_as_longlong(dd) != 0) diag = dd;
+        if (need_max) rowmax = fmax(rowmax, __shfl_xor_sync(0xffffffffu, rowmax, o));
+    }
+    if (lane != 0) return;
     b[r] = elem_b[rsl[r]] + elem_b[rsh[r]];
     double ad = fabs(diag);
     // The pressure constant is removed by -c e_0 e_0^T with c = 1 / dscale[0]^2 (the factorisation
@@ -183,8 +197,9 @@ __device__ void factor_diag_block(double* __restrict__ A, int n, int k0, int nbk
 __global__ void __launch_bounds__(kThreads)
 k_front_assemble(const FrontInfo* __restrict__ fronts, const int* __restrict__ ids,
                  const int* __restrict__ inv, const int* __restrict__ dofs, const SubInfo* __restrict__ subs,
-                 const double* __restrict__ elem, const double* __restrict__ dscale, int NV,
-                 double* __restrict__ F, double* __restrict__ P, int* __restrict__ status) {
+                 const double* __restrict__ elem, const double* __restrict__ dscale,
+                 const double* __restrict__ bglob, int NV, double* __restrict__ F, double* __restrict__ P,
+                 int* __restrict__ status) {
     pdl_begin();
     const FrontInfo fr = fronts[ids[blockIdx.y]];
     const int n = fr.n;
@@ -258,12 +273,32 @@ k_front_assemble(const FrontInfo* __restrict__ fronts, const int* __restrict__ i
             const int rl = e / kTile, ql = e % kTile;
             const int r = ti * kTile + rl, q = tj * kTile + ql;
             if (e >= kTile * kTile || r >= n || q > r) continue;
-            double v = 0.0;
-#pragma unroll
-            for (int ci = 0; ci < 2; ++ci)
-                v += leaf[ci] ? dof_sign(s_fd[0][rl], NV) * x[ci][u] * s_ds[0][rl] * s_ds[1][ql] : x[ci][u];
+            // most entries come from one child only: an FP64 addition (19 cycles of the SM's FP64
+            // unit per warp, what bounds the large levels) just where both contribute
+            const bool in0 = s_iv[0][0][rl] >= 0 && s_iv[1][0][ql] >= 0, in1 = s_iv[0][1][rl] >= 0 && s_iv[1][1][ql] >= 0;
+            double v0 = x[0][u], v1 = x[1][u];
+            if (leaf[0] || leaf[1]) {
+                const double sc = s_ds[0][rl] * s_ds[1][ql];
+                const int flip = s_fd[0][rl] < NV ? 0 : (int)0x80000000u;       // J: the sign of the row
+                if (leaf[0] && in0) { v0 *= sc; v0 = __hiloint2double(__double2hiint(v0) ^ flip, __double2loint(v0)); }
+                if (leaf[1] && in1) { v1 *= sc; v1 = __hiloint2double(__double2hiint(v1) ^ flip, __double2loint(v1)); }
+            }
+            double v = in0 ? v0 : in1 ? v1 : 0.0;
+            if (in0 && in1) v = v0 + v1;
             if (r == fr.pin_row && q == fr.pin_row) v -= 1.0;
             Fm[(long long)r * n + q] = v;
+        }
+    }
+    if (ti == nt - 1 && threadIdx.x < kTile) {       // the right-hand side's entries of this tile's columns
+        const int ql = threadIdx.x, q = tj * kTile + ql;
+        if (q < n) {
+            const int d = s_fd[1][ql];
+            double v = q < fr.ne ? dof_sign(d, NV) * s_ds[1][ql] * bglob[d] : 0.0;
+            for (int ci = 0; ci < 2; ++ci) {
+                const int iq = s_iv[1][ci][ql];
+                if (!leaf[ci] && iq >= 0) v += src[ci][(long long)ld[ci] * ld[ci] + off[ci] + iq];
+            }
+            Fm[(long long)n * n + q] = v;
         }
     }
     if (t == 0 && fr.ne > 0) {              // first panel's diagonal block (inside tile (0, 0))
@@ -381,8 +416,8 @@ k_ldl_panel(const FrontInfo* __restrict__ fronts, const int* __restrict__ ids, i
     const int R = kPanel / W;                                   // rows per warp pass
     const int rows = W == kPanel ? 2 * kPanelRows : kPanelRows * R;   // rows of this CTA
     const int r0 = k1 + blockIdx.x * rows;
-    if (r0 >= n) return;
-    const int r_end = min(n, r0 + rows);
+    if (r0 > n) return;                                         // row n: the right-hand side
+    const int r_end = min(n + 1, r0 + rows);
     double* A = F + fr.f_off;
     __shared__ double Vs[kPanel][kPanel + 1];
     __shared__ double Dinv[kPanel], Dd[kPanel];
@@ -489,6 +524,8 @@ __device__ __forceinline__ double i128_scaled(__int128 v, int e) {
 // Exact integer value (|v| < 2^22) of an FP32 holding one: add 1.5 2^23 and
 // read the significand (FP32 add and integer subtract, no conversion).
 __device__ __forceinline__ int f32_int(float v) { return __float_as_int(v + 12582912.0f) - 0x4B400000; }
+// 2^7 hi + lo of two of them (|.| < 2^30: 32-bit arithmetic)
+__device__ __forceinline__ int f32_pair(float hi, float lo) { return (f32_int(hi) << 7) + f32_int(lo); }
 
 // Trailing update of the blocked LDL^T: F22 -= L21 D L21^T on 32 x 32 tiles
 // of the lower triangle (small tiles spread one front's update over many
@@ -509,7 +546,7 @@ k_ldl_update(const FrontInfo* __restrict__ fronts, const int* __restrict__ ids, 
     const int k1 = k0 + nbk;
     const int m = n - k1;
     if (m <= 0) return;
-    const int nt = (m + kPanel - 1) / kPanel;
+    const int nt = (m + 1 + kPanel - 1) / kPanel;               // rows k1 .. n (row n: the right-hand side)
     const int T = nt * (nt + 1) / 2;
     const int t = blockIdx.x;
     if (t >= T) return;
@@ -517,6 +554,7 @@ k_ldl_update(const FrontInfo* __restrict__ fronts, const int* __restrict__ ids, 
     while (ti * (ti + 1) / 2 > t) --ti;
     while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
     const int tj = t - ti * (ti + 1) / 2;
+    if (k1 + tj * kPanel >= n) return;                          // (a last tile that only row n reaches)
     double* A = F + fr.f_off;
     __shared__ __align__(16) uint32_t sbuf[2 * kPanel * kOzLd];             // 33.8 KB, reused below
     const int i0 = k1 + ti * kPanel, j0 = k1 + tj * kPanel;
@@ -528,7 +566,7 @@ k_ldl_update(const FrontInfo* __restrict__ fronts, const int* __restrict__ ids, 
         if (threadIdx.x < 2 * kPanel) {
             const int op = threadIdx.x / kPanel, rr = threadIdx.x % kPanel;
             const int gr = (op == 0 ? i0 : j0) + rr;
-            ez[threadIdx.x] = gr < n ? oz_exp[2 * ((long long)fr.s_off + gr) + op] : 0;
+            ez[threadIdx.x] = gr <= n ? oz_exp[2 * ((long long)fr.s_off + gr) + op] : 0;
         }
         const uint4* src = reinterpret_cast<const uint4*>(oz);
         for (int e = threadIdx.x; e < 2 * kPanel * (kOzLd - 4) / 4; e += blockDim.x) {
@@ -537,7 +575,7 @@ k_ldl_update(const FrontInfo* __restrict__ fronts, const int* __restrict__ ids, 
             const int rr = rem / ((kOzLd - 4) / 4), q = rem % ((kOzLd - 4) / 4);
             const int gr = (op == 0 ? i0 : j0) + rr;
             uint4 v = make_uint4(0u, 0u, 0u, 0u);
-            if (gr < n) v = src[((long long)fr.s_off + gr) * (kOzRowWords / 4) + op * ((kOzLd - 4) / 4) + q];
+            if (gr <= n) v = src[((long long)fr.s_off + gr) * (kOzRowWords / 4) + op * ((kOzLd - 4) / 4) + q];
             reinterpret_cast<uint4*>((op == 0 ? Sa : Sb) + rr * kOzLd)[q] = v;
         }
         __syncthreads();
@@ -574,12 +612,14 @@ k_ldl_update(const FrontInfo* __restrict__ fronts, const int* __restrict__ ids, 
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
             // S = sum_d P_d 2^{7(7-d)} exactly (|S| < 2^72), then one rounding to FP64
-            __int128 sum = 0;
-#pragma unroll
-            for (int d = 0; d < kOzS; ++d) sum += (__int128)f32_int(acc[d][q]) << (7 * (7 - d));
+            // pairs in 32 bits, quadruples in 64, one 128-bit sum
+            static_assert(kOzS == 8, "the sum below takes eight slices");
+            const long long hi = (long long)f32_pair(acc[0][q], acc[1][q]) * 16384 + f32_pair(acc[2][q], acc[3][q]);
+            const long long lo = (long long)f32_pair(acc[4][q], acc[5][q]) * 16384 + f32_pair(acc[6][q], acc[7][q]);
+            const __int128 sum = ((__int128)hi << 28) + lo;
             const int gi = i0 + mr + g + (q >> 1) * 8;
             const int gj = j0 + nc + 2 * tg + (q & 1);
-            if (gi < n && gj <= gi) {
+            if (gi <= n && gj <= gi && gj < n) {
                 const int e = ez[mr + g + (q >> 1) * 8] + ez[kPanel + nc + 2 * tg + (q & 1)];
                 double* c = A + (long long)gi * n + gj;
                 *c -= i128_scaled(sum, e - 63);
@@ -593,7 +633,7 @@ k_ldl_update(const FrontInfo* __restrict__ fronts, const int* __restrict__ ids, 
         __syncthreads();
         for (int a = w; a < kPanel; a += kThreads / 32) {
             const int gi = i0 + a, gj = j0 + a;
-            Li[a][lane] = (gi < n && lane < nbk) ? A[(long long)gi * n + k0 + lane] * Dk[lane] : 0.0;
+            Li[a][lane] = (gi <= n && lane < nbk) ? A[(long long)gi * n + k0 + lane] * Dk[lane] : 0.0;
             Lj[a][lane] = (gj < n && lane < nbk) ? A[(long long)gj * n + k0 + lane] : 0.0;
         }
         __syncthreads();
@@ -609,11 +649,11 @@ k_ldl_update(const FrontInfo* __restrict__ fronts, const int* __restrict__ ids, 
 #pragma unroll
         for (int p = 0; p < 2; ++p) {
             const int gi = i0 + ty + 16 * p;
-            if (gi >= n) continue;
+            if (gi > n) continue;
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
                 const int gj = j0 + tx + 16 * q;
-                if (gj <= gi) A[(long long)gi * n + gj] -= acc[p][q];
+                if (gj <= gi && gj < n) A[(long long)gi * n + gj] -= acc[p][q];
             }
         }
     }
@@ -717,7 +757,7 @@ k_front_forward_b(const FrontInfo* __restrict__ fronts, const int* __restrict__ 
 __global__ void __launch_bounds__(kThreads)
 k_front_backward_b(const FrontInfo* __restrict__ fronts, const int* __restrict__ ids, const int* __restrict__ dofs,
                    const double* __restrict__ F, const double* __restrict__ xs, double* __restrict__ frhs,
-                   double* __restrict__ bpart, unsigned* __restrict__ bcnt) {
+                   double* __restrict__ bpart, unsigned* __restrict__ bcnt, int rhs_row /* D^{-1} y from the front's row n */) {
     pdl_begin();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     double* xb = reinterpret_cast<double*>(smem_raw);
@@ -758,7 +798,7 @@ k_front_backward_b(const FrontInfo* __restrict__ fronts, const int* __restrict__
     }
     double* zr = frhs + fr.r_off;
     if (Z == 1) {
-        if (g == 0 && i < ne) zr[i] = zr[i] / A[(long long)i * n + i] - s;
+        if (g == 0 && i < ne) zr[i] = (rhs_row ? A[(long long)n * n + i] : zr[i] / A[(long long)i * n + i]) - s;
         return;
     }
     const long long slot = (long long)blockIdx.y * gridDim.x + blockIdx.x;
@@ -771,7 +811,7 @@ k_front_backward_b(const FrontInfo* __restrict__ fronts, const int* __restrict__
         __threadfence();
         double t = 0.0;
         for (int zz = 0; zz < Z; ++zz) t += __ldcg(&bpart[(slot * Z + zz) * 32 + lane]);
-        zr[i] = zr[i] / A[(long long)i * n + i] - t;
+        zr[i] = (rhs_row ? A[(long long)n * n + i] : zr[i] / A[(long long)i * n + i]) - t;
     }
 }
 
@@ -1101,8 +1141,8 @@ LevelPlan plan_level(const Tables& t, int h) {
             if (k0 >= f.ne) continue;
             int k1 = k0 + std::min(kPanel, f.ne - k0);
             int m = f.n - k1;
-            rt = std::max(rt, (m + 2 * kPanelRows - 1) / (2 * kPanelRows));   // >= 8 rows per CTA
-            int nt = (m + kPanel - 1) / kPanel;
+            rt = std::max(rt, (m + 1 + 2 * kPanelRows - 1) / (2 * kPanelRows));   // >= 8 rows per CTA
+            int nt = (m + 1 + kPanel - 1) / kPanel;                            // (with the right-hand side's row)
             ut = std::max(ut, nt * (nt + 1) / 2);
         }
         p.row_tiles.push_back(rt);
@@ -1134,7 +1174,7 @@ int launch_assemble_interface(const Tables& t, const DeviceTables& d, const Layo
     const int nd = 2 * t.NV;
     if (nd == 0) return 0;
     double* dscale = (double*)(ws + L.dscale);
-    MRCM_LAUNCH(P, "k_assemble_csr", st, launch_pdl(k_assemble_csr, dim3((nd + 127) / 128), dim3(128), 0, st, nd, d.rowptr, d.src_lo, d.src_hi, d.rhs_src_lo, d.rhs_src_hi,
+    MRCM_LAUNCH(P, "k_assemble_csr", st, launch_pdl(k_assemble_csr, dim3((nd + 7) / 8), dim3(256), 0, st, nd, d.rowptr, d.src_lo, d.src_hi, d.rhs_src_lo, d.rhs_src_hi,
                                                    d.colidx, (const double*)(ws + L.elem),
                                                    (const double*)(ws + L.elem_b), (double*)(ws + L.csr_val),
                                                    (double*)(ws + L.b_int), dscale, t.has_dirichlet ? 0 : 1));
@@ -1152,7 +1192,7 @@ int launch_assemble_interface(const Tables& t, const DeviceTables& d, const Layo
         for (int id : t.levels[h]) { int nt = (t.fronts[id].n + kTile - 1) / kTile; maxT = std::max(maxT, nt * (nt + 1) / 2); }
         dim3 ga(maxT, cnt);
         MRCM_LAUNCH(P, "k_front_assemble", st, launch_pdl(k_front_assemble, dim3(ga), dim3(kThreads), 0, st, d.fronts, ids, d.front_inv, d.front_dofs, d.subs,
-                                                  (const double*)(ws + L.elem), dscale, t.NV, F, Pv, status));
+                                                  (const double*)(ws + L.elem), dscale, (const double*)(ws + L.b_int), t.NV, F, Pv, status));
         LevelPlan p = plan_level(t, (int)h);
         for (int s = 0; s < p.steps; ++s) {
             dim3 gp(p.row_tiles[s], cnt);
@@ -1185,7 +1225,8 @@ static void launch_cluster(void (*kern)(Args...), int fronts, size_t smem, cudaS
     cudaLaunchKernelEx(&cfg, kern, args...);
 }
 
-static void multifrontal_solve(const Tables& t, const DeviceTables& d, const Layout& L, char* ws,
+// forward = false: the right-hand side is the fronts' own row n (b^int of the factorisation).
+static void multifrontal_solve(const Tables& t, const DeviceTables& d, const Layout& L, char* ws, bool forward,
                                const double* rhs, double* xs, cudaStream_t st, Prof& P) {
     double* F = (double*)(ws + L.fronts);
     const double* Pv = (const double*)(ws + L.panel);
@@ -1194,7 +1235,7 @@ static void multifrontal_solve(const Tables& t, const DeviceTables& d, const Lay
     double* bpart = (double*)(ws + L.bpart);
     unsigned* bcnt = (unsigned*)(ws + L.bcnt);
     size_t sm = sizeof(double) * (size_t)std::max(t.max_front, 1);
-    for (size_t h = 1; h < t.levels.size(); ++h) {
+    for (size_t h = 1; forward && h < t.levels.size(); ++h) {
         int cnt = (int)t.levels[h].size();
         if (!cnt) continue;
         const int* ids = d.level_ids + d.level_off[h];
@@ -1214,7 +1255,7 @@ static void multifrontal_solve(const Tables& t, const DeviceTables& d, const Lay
         const int* ids = d.level_ids + d.level_off[h];
         const LevelPlan p = plan_level(t, (int)h);
         MRCM_LAUNCH(P, "k_front_backward_b", st, launch_pdl(k_front_backward_b, dim3(p.bwd_cols, cnt, bwd_split(p.max_nb)), dim3(kThreads), sm, st, 
-                                                        d.fronts, ids, d.front_dofs, F, xs, frhs, bpart, bcnt));
+                                                        d.fronts, ids, d.front_dofs, F, xs, frhs, bpart, bcnt, forward ? 0 : 1));
         if (p.max_ne >= kSolveClMinNe && p.cl_smem <= kClSmemMax)
             MRCM_LAUNCH(P, "k_front_backward", st, launch_cluster(k_front_backward_cl, cnt, p.cl_smem, st, (const FrontInfo*)d.fronts, ids,
                                                                   (const int*)d.front_dofs, (const double*)F, Pv,
@@ -1256,13 +1297,13 @@ int launch_solve_interface(const Tables& t, const DeviceTables& d, const Layout&
         bwd_split_sizes(t.levels, t.fronts, &parts, &cnts);
         cudaMemsetAsync(ws + L.bcnt, 0, cnts * sizeof(unsigned), st);
     }
-    multifrontal_solve(t, d, L, ws, b, xs, st, P);
+    multifrontal_solve(t, d, L, ws, false, b, xs, st, P);
     MRCM_LAUNCH(P, "k_unscale", st, launch_pdl(k_unscale, dim3((nd + 255) / 256), dim3(256), 0, st, nd, xs, dscale, X, 0));
     const int refine = t.cfg.interface_refine == 0 ? 1 : std::max(0, t.cfg.interface_refine);
     for (int it = 0; it < refine; ++it) {
         MRCM_LAUNCH(P, "k_csr_residual", st, launch_pdl(k_csr_residual, dim3((nd + 127) / 128), dim3(128), 0, st, nd, d.rowptr, d.colidx, (const double*)(ws + L.csr_val),
                                                        b, X, dscale, pin, r));
-        multifrontal_solve(t, d, L, ws, r, xs, st, P);
+        multifrontal_solve(t, d, L, ws, true, r, xs, st, P);
         MRCM_LAUNCH(P, "k_unscale", st, launch_pdl(k_unscale, dim3((nd + 255) / 256), dim3(256), 0, st, nd, xs, dscale, X, 1));
     }
     return (int)cudaGetLastError();

@@ -62,7 +62,7 @@ struct FaceInfo {
 struct FrontInfo {
     int ne, nb, n;          // eliminated dofs, boundary dofs, n = ne + nb
     int nchild;             // 2
-    long long f_off;        // offset (doubles) of the n x n front (row major)
+    long long f_off;        // offset (doubles) of the (n + 1) x n front (row major; row n: right-hand side)
     int r_off;              // offset (doubles) of the front right-hand side
     int child[2];           // child front index, or -(1 + element) for a leaf
     int map_off[2];         // offset (ints) of the child -> front position maps

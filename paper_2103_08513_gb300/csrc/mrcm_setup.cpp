@@ -376,7 +376,7 @@ mrcm_status build_tables(const mrcm_config* cfg, Tables& t, std::string& err) {
         for (int id = 0; id < (int)t.fronts.size(); ++id) {
             FrontInfo& f = t.fronts[id];
             t.levels[f.height].push_back(id);
-            f.f_off = foff;  foff += (long long)f.n * f.n;
+            f.f_off = foff;  foff += (long long)(f.n + 1) * f.n;     // the last row carries the right-hand side
             f.r_off = roff;  roff += f.n;
             f.p_off = t.total_panels;  t.total_panels += (f.ne + 31) / 32;
             t.max_front = std::max(t.max_front, f.n);
@@ -420,7 +420,7 @@ mrcm_status build_tables(const mrcm_config* cfg, Tables& t, std::string& err) {
             for (int id : lv) {
                 FrontInfo& f = t.fronts[id];
                 f.s_off = -1;
-                if (f.n >= kOzMinN) { f.s_off = (int)rows; rows += f.n; }
+                if (f.n >= kOzMinN) { f.s_off = (int)rows; rows += f.n + 1; }
             }
             t.oz_rows = std::max(t.oz_rows, rows);
         }
@@ -429,7 +429,7 @@ mrcm_status build_tables(const mrcm_config* cfg, Tables& t, std::string& err) {
             for (int k0 = 0; k0 < f.ne; k0 += 32) {
                 const int nbk = std::min(32, f.ne - k0), m = f.n - k0 - nbk;
                 if (m < kOzMinM || nbk < kOzMinK) continue;
-                const double nt = (m + 31) / 32;
+                const double nt = (m + 1 + 31) / 32;       // with the right-hand side's row
                 t.ldl_update_tensor_flops += nt * (nt + 1.0) / 2.0 * kOzTileFlops;
             }
         }
