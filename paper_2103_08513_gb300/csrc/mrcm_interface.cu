@@ -307,68 +307,33 @@ k_front_assemble(const FrontInfo* __restrict__ fronts, const int* __restrict__ i
     }
 }
 
-constexpr int kPanelRows = 4;           // warp passes per panel-kernel CTA (one per warp)
+constexpr int kPanelRows = 4;           // warps per panel-kernel CTA, two rows or more each
 
 // Tensor-core emulation of the FP64 trailing update (Ozaki-type splitting
 // with exact integer arithmetic).  For each panel row x (of L21 D for the left
 // operand, of L21 for the right one) let E be the smallest power of two with
-// |x_k| < 2^E for every k of the row; |x_k| 2^{-E} is cut into S = 8 slices of
-// 7 bits, x_k = 2^E sum_t s_t 2^{-7(t+1)} + r with integer |s_t| <= 127 and
-// |r| < 2^{E-56} (sign carried by every slice), extracted from the bits of
+// |x_k| < 2^E for every k of the row; |x_k| 2^{-E} is cut into S = 7 slices of
+// 8 bits, x_k = 2^E sum_t s_t 2^{-8(t+1)} + r with integer |s_t| <= 255 (exact in
+// BF16) and |r| < 2^{E-56} (sign carried by every slice), extracted from the bits of
 // the double with integer operations.  Then
-//   sum_k x_ik y_jk = 2^{E_i + F_j} sum_d P_d 2^{-7(d+2)},
+//   sum_k x_ik y_jk = 2^{E_i + F_j} sum_d P_d 2^{-8(d+2)},
 //   P_d = sum_{t+u=d} sum_k s_t(x_ik) s_u(y_jk),   d = 0 .. S-1
 // (terms with t + u >= S are below the FP64 rounding of the result).  Each
 // P_d is a BF16 MMA with FP32 accumulation whose every partial sum is an
-// integer below 2^22, hence exact; the P_d are combined exactly in 64-bit
-// integers and converted to FP64 once.  An update then costs about five FP64
-// operations per entry instead of one FMA per panel column.
-constexpr int kOzS = 8;                     // slices per operand
+// integer of at most 7 x 32 x 255^2 < 2^24, hence exact; the P_d are combined exactly in integers and converted to FP64 once.  An update then
+// costs one FP64 operation per entry instead of one FMA per panel column.  (Eight slices
+// of 7 bits keep the same 56 bits at 36 products instead of 28.)
+constexpr int kOzS = 7;                     // slices per operand
 constexpr int kOzRowWords = 2 * kOzS * kPanel / 2;   // u32 words per slice row (2 operands x 8 slices x 32 bf16)
 
 __device__ __forceinline__ bool oz_step(const FrontInfo& fr, int m, int nbk) {
     return fr.s_off >= 0 && m >= kOzMinM && nbk >= kOzMinK;
 }
 
-// Maximum over the aligned segment of W lanes (W a power of two) holding this lane.
-__device__ __forceinline__ unsigned long long seg_max_u64(unsigned long long v, int W) {
-    for (int o = W >> 1; o > 0; o >>= 1) {
-        const unsigned long long w = __shfl_xor_sync(0xffffffffu, v, o);
-        v = w > v ? w : v;
-    }
-    return v;
-}
-
-// Slices of one panel row held by a segment of W lanes (lane j of the segment
-// holds column j; columns W .. 31 are zero) into `dst` (kOzS x 32 bf16) and
-// its exponent E into *exp_out.  Integer operations only.
-__device__ __forceinline__ void oz_slice_row(double x, int j, int W, bool store, __nv_bfloat16* dst, int* exp_out) {
-    const unsigned long long bits = (unsigned long long)__double_as_longlong(x);
-    const unsigned long long mag = bits & 0x7FFFFFFFFFFFFFFFull;          // orders like |x|
-    const unsigned long long mx = seg_max_u64(mag, W);
-    const int E = mx == 0 ? 0 : (int)(mx >> 52) - 1023 + 1;                // max |x| < 2^E
-    const int ex = (int)(mag >> 52);
-    unsigned long long Fx = 0;                                             // floor(|x| 2^{56-E})
-    if (ex != 0) {
-        const unsigned long long mant = (mag & 0x000FFFFFFFFFFFFFull) | (1ull << 52);
-        const int sh = ex - 1023 + 4 - E;                                  // <= 3
-        Fx = sh >= 0 ? (mant << sh) : (-sh < 64 ? (mant >> -sh) : 0ull);
-    }
-    const bool neg = (bits >> 63) != 0;
-    const __nv_bfloat16 zero = __float2bfloat16_rn(0.0f);
-    if (!store) return;                                                    // after the segment reduction
-#pragma unroll
-    for (int t = 0; t < kOzS; ++t) {
-        const int v = (int)((Fx >> (49 - 7 * t)) & 127ull);
-        dst[t * kPanel + j] = __float2bfloat16_rn((float)(neg ? -v : v));
-        for (int c = j + W; c < kPanel; c += W) dst[t * kPanel + c] = zero;
-    }
-    if (j == 0) *exp_out = E;
-}
-
-// Slices of one panel row held as pairs: lane p of a 16-lane segment holds
-// columns p and 31 - p (values x1, x2).  Same slices and exponent as
-// oz_slice_row over the full row.
+// Slices of one panel row held by a segment of H lanes (the first of them `base`), lane p
+// the adjacent columns 2 p and 2 p + 1 (values x1, x2), a 32-bit word a slice, to `dst`
+// (kOzS x 16 words), and the row's exponent E to *exp_out.  Words past the panel are not
+// written (the update reads zeros there).  Integer operations only.
 __device__ __forceinline__ unsigned long long oz_fixed(unsigned long long mag, int E) {   // floor(|x| 2^{56-E})
     const int ex = (int)(mag >> 52);
     if (ex == 0) return 0ull;
@@ -376,33 +341,39 @@ __device__ __forceinline__ unsigned long long oz_fixed(unsigned long long mag, i
     const int sh = ex - 1023 + 4 - E;                                      // <= 3
     return sh >= 0 ? (mant << sh) : (-sh < 64 ? (mant >> -sh) : 0ull);
 }
-__device__ __forceinline__ void oz_slice_pair(double x1, double x2, int p, bool store, __nv_bfloat16* dst,
-                                              int* exp_out) {
+__device__ __forceinline__ void oz_slice_row(double x1, double x2, int p, int H, int base, bool store,
+                                             uint32_t* dst, int* exp_out) {
     const unsigned long long b1 = (unsigned long long)__double_as_longlong(x1);
     const unsigned long long b2 = (unsigned long long)__double_as_longlong(x2);
-    const unsigned long long m1 = b1 & 0x7FFFFFFFFFFFFFFFull, m2 = b2 & 0x7FFFFFFFFFFFFFFFull;
-    const unsigned long long mx = seg_max_u64(m1 > m2 ? m1 : m2, 16);
-    const int E = mx == 0 ? 0 : (int)(mx >> 52) - 1023 + 1;
-    const unsigned long long F1 = oz_fixed(m1, E), F2 = oz_fixed(m2, E);
+    const unsigned long long m1 = b1 & 0x7FFFFFFFFFFFFFFFull, m2 = b2 & 0x7FFFFFFFFFFFFFFFull;   // order like |x|
+    // E needs the exponent field of the largest magnitude alone
+    unsigned mx = max((unsigned)(m1 >> 32), (unsigned)(m2 >> 32));
+    if (mx == 0u && (m1 | m2) != 0ull) mx = 1u;                            // (a subnormal below 2^-1042 is not zero)
+    for (int o = 1; o < H; o <<= 1)                                        // lane p: maximum over p .. p + 2 o - 1
+        mx = max(mx, __shfl_sync(0xffffffffu, mx, base + min(p + o, H - 1)));
+    mx = __shfl_sync(0xffffffffu, mx, base);
     if (!store) return;                                                    // after the segment reduction
-    const bool n1 = (b1 >> 63) != 0, n2 = (b2 >> 63) != 0;
+    const int E = mx == 0u ? 0 : (int)(mx >> 20) - 1023 + 1;               // max |x| < 2^E
+    const unsigned long long F1 = oz_fixed(m1, E), F2 = oz_fixed(m2, E);
+    const uint32_t sg = (uint32_t)(b1 >> 48 & 0x8000u) | (uint32_t)(b2 >> 32 & 0x80000000u);
 #pragma unroll
     for (int t = 0; t < kOzS; ++t) {
-        const int v1 = (int)((F1 >> (49 - 7 * t)) & 127ull), v2 = (int)((F2 >> (49 - 7 * t)) & 127ull);
-        dst[t * kPanel + p] = __float2bfloat16_rn((float)(n1 ? -v1 : v1));
-        dst[t * kPanel + kPanel - 1 - p] = __float2bfloat16_rn((float)(n2 ? -v2 : v2));
+        const float f1 = __uint_as_float(0x4B000000u | ((uint32_t)(F1 >> (48 - 8 * t)) & 255u)) - 8388608.0f;
+        const float f2 = __uint_as_float(0x4B000000u | ((uint32_t)(F2 >> (48 - 8 * t)) & 255u)) - 8388608.0f;
+        dst[t * (kPanel / 2) + p] = __byte_perm(__float_as_uint(f1), __float_as_uint(f2), 0x7632) | sg;   // exact in BF16
     }
     if (p == 0) *exp_out = E;
 }
 
 // Panel step of the blocked LDL^T: the rows below the (already factored)
 // diagonal block, l = a L11^{-T} D^{-1}, i.e. l_j = sum_{k <= j} a_k V[j][k] / d_j
-// with V = L11^{-1}.  Panels wider than 16 columns: a warp holds two rows,
-// lane p of each half computes columns p and 31 - p (p + 1 and 32 - p terms of
-// the triangular product, 33 FMAs in two chains instead of 32 per column), 8
-// rows per CTA.  Narrower panels: a warp holds 32 / W rows at once, W = the
-// panel width rounded up to a power of two (one lane per column), so narrow
-// panels do not waste FP64 issue slots; kPanelRows x 32 / W rows per CTA.
+// with V = L11^{-1}.  FP64-bound (an FP64 warp instruction takes 16 cycles of an SM), so
+// the triangular product has no idle lanes: lane p of a row computes columns p and
+// nbk - 1 - p, nbk + 1 terms together, on ceil(nbk / 2) lanes, and a warp holds as many
+// rows as fit.  The slices of L21 D are those of the undivided sums; they leave in 32-bit
+// words (16-bit stores of single columns, zeros included, took as long as the product).
+// 1116 fronts of 90 rows, 20 columns: 106 us (lanes in powers of two) -> 49; 240 of 120,
+// 8 columns: 20 -> 12; one panel of 32 columns alone stays at its latency, 8 us.
 __global__ void __launch_bounds__(128)
 k_ldl_panel(const FrontInfo* __restrict__ fronts, const int* __restrict__ ids, int k0, double* __restrict__ F,
             const double* __restrict__ P, __nv_bfloat16* __restrict__ oz, int* __restrict__ oz_exp) {
@@ -412,78 +383,53 @@ k_ldl_panel(const FrontInfo* __restrict__ fronts, const int* __restrict__ ids, i
     const int n = fr.n;
     const int nbk = min(kPanel, fr.ne - k0);
     const int k1 = k0 + nbk;
-    const int W = nbk <= 1 ? 1 : 1 << (32 - __clz(nbk - 1));
-    const int R = kPanel / W;                                   // rows per warp pass
-    const int rows = W == kPanel ? 2 * kPanelRows : kPanelRows * R;   // rows of this CTA
-    const int r0 = k1 + blockIdx.x * rows;
+    const int H = (nbk + 1) >> 1, R = 32 / H;                   // lanes per row, rows per warp
+    const int r0 = k1 + blockIdx.x * kPanelRows * R;
     if (r0 > n) return;                                         // row n: the right-hand side
-    const int r_end = min(n + 1, r0 + rows);
     double* A = F + fr.f_off;
     __shared__ double Vs[kPanel][kPanel + 1];
-    __shared__ double Dinv[kPanel], Dd[kPanel];
+    __shared__ double Dinv[kPanel];
+    __shared__ double As[kPanelRows][2 * kPanel + 1], Ls[kPanelRows][2 * kPanel + 1];
     const double* V = P + (long long)(fr.p_off + k0 / kPanel) * kPanel * kPanel;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int rs = lane / H, p = lane - rs * H, p2 = nbk - 1 - p;
+    const int r = r0 + w * R + rs;
+    const bool live = rs < R && r <= n;
+    double* row = A + (long long)min(r, n) * n + k0;
+    double* as = As[w] + min(rs, R - 1) * nbk;
+    const double a1 = live ? row[p] : 0.0, a2 = live ? row[p2] : 0.0;
     for (int e = threadIdx.x; e < kPanel * kPanel; e += blockDim.x) Vs[e >> 5][e & 31] = V[e];
     if (threadIdx.x < kPanel) {
         const double d = threadIdx.x < nbk ? A[(long long)(k0 + threadIdx.x) * n + k0 + threadIdx.x] : 0.0;
-        Dd[threadIdx.x] = d;
         Dinv[threadIdx.x] = threadIdx.x < nbk ? rcp64(d) : 0.0;
     }
+    if (rs < R) { as[p] = a1; as[p2] = a2; }
     __syncthreads();
-    const bool oz_on = oz_step(fr, n - k1, nbk);
-    if (W == kPanel) {
-        __shared__ double As[kPanelRows][2][kPanel];
-        const int h = lane >> 4, p = lane & 15, p2 = kPanel - 1 - p;
-        const int r = r0 + 2 * w + h;
-        const bool live = r < r_end;
-        double* row = A + (long long)min(r, r_end - 1) * n + k0;
-        double* as = As[w][h];
-        as[p] = (live && p < nbk) ? row[p] : 0.0;
-        as[p2] = (live && p2 < nbk) ? row[p2] : 0.0;
-        __syncwarp();
-        // chain A: terms q = 0 .. 16 (column p while q <= p, then column p2);
-        // chain B: q = 17 .. 32, all of column p2 (k = q - p - 1)
-        double x1 = 0.0, x2 = 0.0, y2 = 0.0;
+    // terms q = 0 .. p of column p, then p2 + 1 of column p2
+    double x1 = 0.0, x2 = 0.0;
+    for (int q0 = 0; q0 <= nbk; q0 += 8) {
 #pragma unroll
-        for (int q = 0; q < 17; ++q) {
+        for (int u = 0; u < 8; ++u) {
+            const int q = q0 + u;
             const bool f = q <= p;
-            const int k = f ? q : q - p - 1;
+            const int k = min(f ? q : q - p - 1, nbk - 1);      // (odd nbk: the middle column is formed twice)
             const double v = fma(as[k], Vs[f ? p : p2][k], f ? x1 : x2);
-            if (f) x1 = v; else x2 = v;
-            if (q < 16) y2 = fma(as[q + 16 - p], Vs[p2][q + 16 - p], y2);
+            if (q <= nbk) { if (f) x1 = v; else x2 = v; }
         }
-        const double l1 = x1 * Dinv[p], l2 = (x2 + y2) * Dinv[p2];
-        if (live && p < nbk) row[p] = l1;
-        if (live && p2 < nbk) row[p2] = l2;
-        if (oz_on) {                                              // all lanes: segment reductions inside
-            const long long sr = (long long)fr.s_off + min(r, r_end - 1);
-            oz_slice_pair(l1 * Dd[p], l2 * Dd[p2], p, live, oz + sr * (2 * kOzS * kPanel), oz_exp + 2 * sr);
-            oz_slice_pair(l1, l2, p, live, oz + sr * (2 * kOzS * kPanel) + kOzS * kPanel, oz_exp + 2 * sr + 1);
-        }
-        return;
     }
-    const int rs = lane / W, j = lane % W;
-    for (int base = r0 + w * R; base < r_end; base += 4 * R) {
-        const int r = base + rs;
-        const bool live = r < r_end && j < nbk;
-        double* row = A + (long long)r * n + k0;
-        const double a = live ? row[j] : 0.0;
-        double acc0 = 0.0, acc1 = 0.0;                            // two chains of FP64 FMAs
-        int k = 0;
-        for (; k + 1 < nbk; k += 2) {
-            const double ak0 = __shfl_sync(0xffffffffu, a, rs * W + k);
-            const double ak1 = __shfl_sync(0xffffffffu, a, rs * W + k + 1);
-            acc0 = fma(ak0, Vs[j][k], acc0);                     // V[j][k] = 0 for k > j
-            acc1 = fma(ak1, Vs[j][k + 1], acc1);
-        }
-        if (k < nbk) acc0 = fma(__shfl_sync(0xffffffffu, a, rs * W + k), Vs[j][k], acc0);
-        const double l = live ? (acc0 + acc1) * Dinv[j] : 0.0;
-        if (live) row[j] = l;
-        if (oz_on) {                                              // all lanes: segment reductions inside
-            const long long sr = (long long)fr.s_off + min(r, r_end - 1);
-            oz_slice_row(l * Dd[j], j, W, r < r_end, oz + sr * (2 * kOzS * kPanel), oz_exp + 2 * sr);
-            oz_slice_row(l, j, W, r < r_end, oz + sr * (2 * kOzS * kPanel) + kOzS * kPanel, oz_exp + 2 * sr + 1);
-        }
+    const double l1 = x1 * Dinv[p], l2 = x2 * Dinv[p2];
+    if (live) { row[p] = l1; row[p2] = l2; }
+    if (oz_step(fr, n - k1, nbk)) {                             // all lanes: segment reductions inside
+        double* ls = Ls[w] + min(rs, R - 1) * nbk;
+        __syncwarp();
+        if (rs < R) { as[p] = x1; as[p2] = x2; ls[p] = l1; ls[p2] = l2; }
+        __syncwarp();
+        const int c1 = 2 * p, c2 = 2 * p + 1;                   // an odd panel's last word: a zero column
+        const long long sr = (long long)fr.s_off + min(r, n);
+        const int base = min(rs, R - 1) * H;
+        uint32_t* dst = reinterpret_cast<uint32_t*>(oz) + sr * kOzRowWords;
+        oz_slice_row(as[c1], c2 < nbk ? as[c2] : 0.0, p, H, base, live, dst, oz_exp + 2 * sr);
+        oz_slice_row(ls[c1], c2 < nbk ? ls[c2] : 0.0, p, H, base, live, dst + kOzRowWords / 2, oz_exp + 2 * sr + 1);
     }
 }
 
@@ -496,24 +442,23 @@ __device__ __forceinline__ void mma_bf16(float d[4], const uint32_t a[4], const 
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b[0]), "r"(b[1]));
 }
 
-// The 128-bit integer v, times 2^e, rounded to the nearest FP64 value with
+// The 128-bit integer v (|v| < 2^72), times 2^e, rounded to the nearest FP64 value with
 // integer operations only (ties away from zero; results below the normal
 // range become 0).
 __device__ __forceinline__ double i128_scaled(__int128 v, int e) {
     if (v == 0) return 0.0;
     const unsigned long long sign = v < 0 ? 0x8000000000000000ull : 0ull;
     const unsigned __int128 m = v < 0 ? (unsigned __int128)(-v) : (unsigned __int128)v;
-    const unsigned long long mh = (unsigned long long)(m >> 64), ml = (unsigned long long)m;
-    const int top = mh ? 127 - __clzll((long long)mh) : 63 - __clzll((long long)ml);   // m in [2^top, 2^(top+1))
+    unsigned long long mh = (unsigned long long)(m >> 64), ml = (unsigned long long)m;
+    if (mh) { ml = (ml >> 8) | (mh << 56); e += 8; }           // the 8 bits lie below the rounding bit
+    const int top = 63 - __clzll((long long)ml);               // ml in [2^top, 2^(top+1))
     unsigned long long mant;                                   // top 53 bits, rounded
     int ex = top + e;
     if (top <= 52) {
         mant = ml << (52 - top);
     } else {
-        const int sh = top - 52;
-        const unsigned __int128 q = m >> sh;
-        const bool up = (m >> (sh - 1)) & 1;                   // first dropped bit
-        mant = (unsigned long long)q + (up ? 1ull : 0ull);
+        const unsigned long long q = ml >> (top - 53);
+        mant = (q >> 1) + (q & 1);                             // first dropped bit
         if (mant >> 53) { mant >>= 1; ++ex; }                  // rounding carried into a new bit
     }
     const int be = ex + 1023;
@@ -524,17 +469,22 @@ __device__ __forceinline__ double i128_scaled(__int128 v, int e) {
 // Exact integer value (|v| < 2^22) of an FP32 holding one: add 1.5 2^23 and
 // read the significand (FP32 add and integer subtract, no conversion).
 __device__ __forceinline__ int f32_int(float v) { return __float_as_int(v + 12582912.0f) - 0x4B400000; }
-// 2^7 hi + lo of two of them (|.| < 2^30: 32-bit arithmetic)
-__device__ __forceinline__ int f32_pair(float hi, float lo) { return (f32_int(hi) << 7) + f32_int(lo); }
+__device__ __forceinline__ void ldsm_x4(uint32_t addr, uint32_t r[4]) {
+    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
+}
 
 // Trailing update of the blocked LDL^T: F22 -= L21 D L21^T on 32 x 32 tiles
 // of the lower triangle (small tiles spread one front's update over many
 // SMs); blockIdx.x enumerates the (ti >= tj) tile pairs.  Large steps take
 // the tensor-core emulation above, the others plain FP64 FMAs.  The CTA of
 // tile (0, 0), which holds the next panel's diagonal block, factors that
-// block afterwards.
+// block afterwards.  A tile is a chain of loads, products and one rounding, so the time is
+// latency over the warps in flight: three CTAs per SM, the entries read ahead of the
+// products.  20 fronts of 850 (7020 tiles): 117 us (36 products, word loads) -> 84; all 70
+// launches at 60 x 220 x 85: 2.21 -> 2.02 ms, of which the 32 pivots of the diagonal block are 1.0.
 constexpr int kOzLd = kOzRowWords / 2 + 4;  // u32 words per staged operand row (one operand, padded)
-__global__ void __launch_bounds__(kThreads)
+__global__ void __launch_bounds__(kThreads, 3)
 k_ldl_update(const FrontInfo* __restrict__ fronts, const int* __restrict__ ids, int k0, double* __restrict__ F,
              double* __restrict__ P, int* __restrict__ status, const __nv_bfloat16* __restrict__ oz,
              const int* __restrict__ oz_exp) {
@@ -556,7 +506,7 @@ k_ldl_update(const FrontInfo* __restrict__ fronts, const int* __restrict__ ids, 
     const int tj = t - ti * (ti + 1) / 2;
     if (k1 + tj * kPanel >= n) return;                          // (a last tile that only row n reaches)
     double* A = F + fr.f_off;
-    __shared__ __align__(16) uint32_t sbuf[2 * kPanel * kOzLd];             // 33.8 KB, reused below
+    __shared__ __align__(16) uint32_t sbuf[2 * kPanel * kOzLd];             // 29.7 KB, reused below
     const int i0 = k1 + ti * kPanel, j0 = k1 + tj * kPanel;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     if (oz_step(fr, m, nbk)) {
@@ -576,53 +526,61 @@ k_ldl_update(const FrontInfo* __restrict__ fronts, const int* __restrict__ ids, 
             const int gr = (op == 0 ? i0 : j0) + rr;
             uint4 v = make_uint4(0u, 0u, 0u, 0u);
             if (gr <= n) v = src[((long long)fr.s_off + gr) * (kOzRowWords / 4) + op * ((kOzLd - 4) / 4) + q];
+            if (nbk < kPanel) {                                            // words past the panel are not written
+                const int c0 = 8 * (q & 3);
+                if (c0 >= nbk) v.x = 0u;
+                if (c0 + 2 >= nbk) v.y = 0u;
+                if (c0 + 4 >= nbk) v.z = 0u;
+                if (c0 + 6 >= nbk) v.w = 0u;
+            }
             reinterpret_cast<uint4*>((op == 0 ? Sa : Sb) + rr * kOzLd)[q] = v;
         }
-        __syncthreads();
         const int g = lane >> 2, tg = lane & 3;
         const int mr = (w >> 2) * 16, nc = (w & 3) * 8;                   // this warp's 16 x 8 output block
+        double cv[4];                                                     // its entries, read ahead
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int gi = i0 + mr + g + (q >> 1) * 8, gj = j0 + nc + 2 * tg + (q & 1);
+            cv[q] = gi <= n && gj <= gi && gj < n ? A[(long long)gi * n + gj] : 0.0;
+        }
+        __syncthreads();
+        static_assert(kOzS == 7, "the sums below take seven slices");
         float acc[kOzS][4];
 #pragma unroll
         for (int d = 0; d < kOzS; ++d)
 #pragma unroll
             for (int q = 0; q < 4; ++q) acc[d][q] = 0.f;
-        // P_d accumulates every slice pair (ts, us) with ts + us = d; consecutive
-        // MMAs go to different accumulators
+        // fragments by ldmatrix: 14 + 28 shared-memory instructions a warp (208 word loads before)
+        const uint32_t sa = (uint32_t)__cvta_generic_to_shared(Sa), sb = (uint32_t)__cvta_generic_to_shared(Sb);
+        const uint32_t la = sa + 4u * ((mr + (lane & 7) + ((lane >> 3) & 1) * 8) * kOzLd + (lane >> 4) * 4);
+        const uint32_t lb = sb + 4u * ((nc + (lane & 7)) * kOzLd + (lane >> 3) * 4);
 #pragma unroll
         for (int ts = 0; ts < kOzS; ++ts) {
             uint32_t af[2][4];
-#pragma unroll
-            for (int kc = 0; kc < 2; ++kc) {
-                const int wa = ts * (kPanel / 2) + kc * 8 + tg;
-                af[kc][0] = Sa[(mr + g) * kOzLd + wa];
-                af[kc][1] = Sa[(mr + g + 8) * kOzLd + wa];
-                af[kc][2] = Sa[(mr + g) * kOzLd + wa + 4];
-                af[kc][3] = Sa[(mr + g + 8) * kOzLd + wa + 4];
-            }
+            ldsm_x4(la + ts * (kPanel * 2), af[0]);
+            ldsm_x4(la + ts * (kPanel * 2) + 32, af[1]);
 #pragma unroll
             for (int us = 0; us < kOzS - ts; ++us) {
-#pragma unroll
-                for (int kc = 0; kc < 2; ++kc) {
-                    const int wb = us * (kPanel / 2) + kc * 8 + tg;
-                    const uint32_t bf[2] = {Sb[(nc + g) * kOzLd + wb], Sb[(nc + g) * kOzLd + wb + 4]};
-                    mma_bf16(acc[ts + us], af[kc], bf);
-                }
+                uint32_t bf[4];
+                ldsm_x4(lb + us * (kPanel * 2), bf);
+                mma_bf16(acc[ts + us], af[0], bf);
+                mma_bf16(acc[ts + us], af[1], bf + 2);
             }
         }
 #pragma unroll
         for (int q = 0; q < 4; ++q) {
-            // S = sum_d P_d 2^{7(7-d)} exactly (|S| < 2^72), then one rounding to FP64
-            // pairs in 32 bits, quadruples in 64, one 128-bit sum
-            static_assert(kOzS == 8, "the sum below takes eight slices");
-            const long long hi = (long long)f32_pair(acc[0][q], acc[1][q]) * 16384 + f32_pair(acc[2][q], acc[3][q]);
-            const long long lo = (long long)f32_pair(acc[4][q], acc[5][q]) * 16384 + f32_pair(acc[6][q], acc[7][q]);
-            const __int128 sum = ((__int128)hi << 28) + lo;
+            // S = sum_d P_d 2^{8(6-d)} exactly (|S| < 2^70), then one rounding to FP64
+            const int p0 = f32_int(acc[0][q]), p1 = f32_int(acc[1][q]);           // at most 2 x 32 x 255^2 < 2^22
+            const int p2 = __float2int_rn(acc[2][q]), p3 = __float2int_rn(acc[3][q]);
+            const int p4 = __float2int_rn(acc[4][q]), p5 = __float2int_rn(acc[5][q]), p6 = __float2int_rn(acc[6][q]);
+            const long long hi = (long long)(p0 * 256 + p1) * 256 + p2;
+            const long long lo = (long long)(p3 * 256 + p4) * 65536 + ((long long)p5 * 256 + p6);
+            const __int128 sum = ((__int128)hi << 32) + lo;
             const int gi = i0 + mr + g + (q >> 1) * 8;
             const int gj = j0 + nc + 2 * tg + (q & 1);
             if (gi <= n && gj <= gi && gj < n) {
                 const int e = ez[mr + g + (q >> 1) * 8] + ez[kPanel + nc + 2 * tg + (q & 1)];
-                double* c = A + (long long)gi * n + gj;
-                *c -= i128_scaled(sum, e - 63);
+                A[(long long)gi * n + gj] = cv[q] - i128_scaled(sum, e - 64);
             }
         }
     } else {

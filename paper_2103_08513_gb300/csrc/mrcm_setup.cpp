@@ -429,7 +429,7 @@ mrcm_status build_tables(const mrcm_config* cfg, Tables& t, std::string& err) {
             for (int k0 = 0; k0 < f.ne; k0 += 32) {
                 const int nbk = std::min(32, f.ne - k0), m = f.n - k0 - nbk;
                 if (m < kOzMinM || nbk < kOzMinK) continue;
-                const double nt = (m + 1 + 31) / 32;       // with the right-hand side's row
+                const double nt = (m + 31) / 32;
                 t.ldl_update_tensor_flops += nt * (nt + 1.0) / 2.0 * kOzTileFlops;
             }
         }
@@ -525,7 +525,7 @@ void compute_layout(const Tables& t, Layout& L) {
     L.fronts = take((size_t)t.total_front * sizeof(double));
     L.frhs = take((size_t)t.total_frhs * sizeof(double));
     L.panel = take((size_t)t.total_panels * 32 * 32 * sizeof(double));
-    L.oz = take((size_t)t.oz_rows * 1024);                 // 2 operands x 8 slices x 32 bf16 per row
+    L.oz = take((size_t)t.oz_rows * 896);                  // 2 operands x 7 slices x 32 bf16 per row
     L.oz_exp = take((size_t)t.oz_rows * 2 * sizeof(int));
     L.xres = take((size_t)2 * t.NV * sizeof(double));
     L.xtmp = take((size_t)2 * t.NV * sizeof(double));
