@@ -1,5 +1,5 @@
 // Device arithmetic helpers shared by the libmrcm kernels: FP64 <-> FP32
-// conversions and an FP64 reciprocal that avoid the FP64 unit's slow paths.
+// conversions, an FP64 reciprocal and maxima that stay off the FP64 unit.
 #pragma once
 #include <cuda_runtime.h>
 
@@ -34,49 +34,44 @@ __device__ __forceinline__ double f32_to_f64(float x) {
     return __longlong_as_double((long long)b);
 }
 
-// 1 / d by Newton-Raphson iteration y <- y + y (1 - d y) from an FP32 seed
-// (FP32 reciprocal of d truncated to FP32, both conversions done with bit
-// operations): each step squares the relative error, so two steps take the
-// seed's ~2^-22 to the FP64 rounding level.  On this GPU an FP64 division is
-// a ~470-cycle dependent chain on the FP64 unit, this one four FMAs.  Values
-// whose reciprocal leaves the FP32 range fall back to the division.
+// 1 / d with integer operations: the FP32 reciprocal Y 2^-24 of the significand M 2^-52, its
+// error e = 1 - M Y 2^-76 exactly (below 2^-22, so 64 bits hold it), then Y (1 + e + e^2)
+// rounded to 53 bits: within 0.5 ulp over 4e7 random d (1 ulp at d = 2 - ulp).  An FP64 warp
+// instruction takes 16 cycles of an SM here and 66 of a dependent chain, so the four FMAs of
+// two Newton steps cost a per-cell kernel 64 cycles and a pivot chain 270; these ~30 integer
+// instructions cost 8 and 130.  Zero, subnormal, infinite and NaN d, and d whose reciprocal is
+// subnormal, take the division.
 __device__ __forceinline__ double rcp64(double d) {
-    const unsigned long long bd = (unsigned long long)__double_as_longlong(d);
-    const int e = (int)((bd >> 52) & 0x7FF) - 1023;
-    if (e < -125 || e > 125) return 1.0 / d;
-    const float df = __uint_as_float((unsigned int)(bd >> 32) & 0x80000000u |
-                                     (unsigned int)(e + 127) << 23 | (unsigned int)((bd >> 29) & 0x7FFFFFu));
+    const unsigned hi = (unsigned)__double2hiint(d), lo = (unsigned)__double2loint(d);
+    const unsigned ex = (hi >> 20) & 0x7FFu;
+    if (ex - 1u > 2042u) return 1.0 / d;
     float yf;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(df));
-    const unsigned int fy = __float_as_uint(yf);
-    const int ey = (int)((fy >> 23) & 0xFF);
-    double y = __longlong_as_double((long long)((unsigned long long)(fy & 0x80000000u) << 32 |
-                                                (unsigned long long)(ey - 127 + 1023) << 52 |
-                                                (unsigned long long)(fy & 0x7FFFFFu) << 29));
-    double r = fma(-d, y, 1.0);
-    y = fma(y, r, y);
-    r = fma(-d, y, 1.0);
-    return fma(y, r, y);
+    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(__uint_as_float(0x3F800000u | (hi & 0xFFFFFu) << 3 | lo >> 29)));
+    const unsigned fy = __float_as_uint(yf);                  // in [1/2, 1]
+    const unsigned Y = ((fy & 0x7FFFFFu) | 0x800000u) << ((fy >> 23) - 126u);
+    const long long E = -(long long)((unsigned long long)lo * Y + ((unsigned long long)(((hi & 0xFFFFFu) | 0x100000u) * Y) << 32));
+    const int Eh = (int)(E >> 32);
+    const long long c1 = (long long)(int)Y * Eh + (long long)__umulhi(Y, (unsigned)E);            // Y e, in 2^-68
+    const unsigned t = (unsigned)(((long long)Eh * Eh) >> 20);                                     // e^2
+    const long long R = ((long long)Y << 38) + ((c1 + (long long)(((unsigned long long)Y * t) >> 24)) >> 6);
+    const unsigned long long mant = (unsigned long long)(R + 256) >> 9;
+    return __longlong_as_double((long long)((((unsigned long long)(2044u - ex) << 52) + mant) |
+                                            (unsigned long long)(hi & 0x80000000u) << 32));
 }
 
-// 1 / d from the same FP32 seed by one third-order step, y (1 + e + e^2) with
-// e = 1 - d y: the seed's ~2^-22 error cubed lies below the FP64 rounding, at
-// three dependent FMAs instead of four (for pivot chains).
-__device__ __forceinline__ double rcp64c(double d) {
-    const unsigned long long bd = (unsigned long long)__double_as_longlong(d);
-    const int e = (int)((bd >> 52) & 0x7FF) - 1023;
-    if (e < -125 || e > 125) return 1.0 / d;
-    const float df = __uint_as_float((unsigned int)(bd >> 32) & 0x80000000u |
-                                     (unsigned int)(e + 127) << 23 | (unsigned int)((bd >> 29) & 0x7FFFFFu));
-    float yf;
-    asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(yf) : "f"(df));
-    const unsigned int fy = __float_as_uint(yf);
-    const int ey = (int)((fy >> 23) & 0xFF);
-    const double y = __longlong_as_double((long long)((unsigned long long)(fy & 0x80000000u) << 32 |
-                                                      (unsigned long long)(ey - 127 + 1023) << 52 |
-                                                      (unsigned long long)(fy & 0x7FFFFFu) << 29));
-    const double r = fma(-d, y, 1.0);
-    return fma(y, fma(r, r, r), y);
+// n / d from r = 1 / d by one correction step (the quotient's residual is exact in an FMA):
+// three FP64 operations
+__device__ __forceinline__ double div64(double n, double d, double r) {
+    const double q = n * r;
+    const double e = fma(-q, d, n);
+    return fma(e, r, q);
+}
+
+// Maximum of |x| as bits of a non-negative double (integer operations: an FP64 comparison
+// occupies the FP64 unit like an FMA); a NaN counts as infinity.
+__device__ __forceinline__ unsigned long long abs_bits(double x) {
+    const unsigned long long b = (unsigned long long)__double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFull;
+    return b > 0x7FF0000000000000ull ? 0x7FF0000000000000ull : b;
 }
 
 }  // namespace mrcm

@@ -92,7 +92,9 @@ __global__ void k_assemble_csr(int nrows, const int* __restrict__ rowptr, const 
     // subtracts 1 from the scaled pinned entry); any c > 0 gives the solution with pi^p_0 = 0.  c is
     // the row's largest entry: |A_00| itself unless A_00 vanishes, which it does when the
     // subdomains around basis 0 carry no other basis (their P-MBF is the constant 1, no flux).
-    if (pin && r == 0) ad = rowmax;
+    // A_00 <= 0 (see above); a positive one is the rounding error of such a row, and the scaled
+    // entry 1 less c would vanish: a larger c then.
+    if (pin && r == 0) ad = __double2hiint(diag) >= 0 ? 4.0 * rowmax : rowmax;
     dscale[r] = ad > 0.0 ? rsqrt(ad) : 1.0;
 }
 
@@ -110,7 +112,7 @@ __device__ __forceinline__ double dof_sign(int dof, int NV) { return dof < NV ? 
 // of V is final at step k).  Block column k is not written after step k - 1,
 // so L = T[i][k] / d_k is formed once at the end: one barrier per pivot.  One
 // lane per column: a row costs one FP64 FMA per step.  Warp 0 updates row
-// k + 1 alone; its lane k + 1 computes 1 / d_{k+1} (one cubic Newton step)
+// k + 1 alone; its lane k + 1 computes 1 / d_{k+1} (integer operations)
 // from the fresh diagonal, and the warp forms the next step's multipliers
 // from the row it holds (the upper triangle is kept for that) into one of two
 // shared vectors, so the other warps, which update the remaining rows, read
@@ -146,7 +148,7 @@ __device__ void factor_diag_block(double* __restrict__ A, int n, int k0, int nbk
         double d = T[0][0];
         const bool z = zero_or_nan(d);
         if (z) d = 1.0;
-        const double inv0 = rcp64c(d);
+        const double inv0 = rcp64(d);
         swc[lane] = (lane == 0 ? 1.0 : T[0][lane]) * inv0;
         if (lane == 0) {
             *zero = z ? 1 : 0;
@@ -167,7 +169,7 @@ __device__ void factor_diag_block(double* __restrict__ A, int n, int k0, int nbk
             double inv = 0.0;
             if (c == i) {                                     // the next pivot, straight from the register
                 if (zero_or_nan(v)) { v = 1.0; *zero = 1; }
-                inv = rcp64c(v);
+                inv = rcp64(v);
                 sinv[i] = inv;
             }
             *dst = v;

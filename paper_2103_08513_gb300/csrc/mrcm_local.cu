@@ -61,7 +61,7 @@ __device__ __forceinline__ long long global_cell(const SubInfo& s, const int lc[
 
 // Robin coefficient of a face with normal permeability Kn: beta (the constant,
 // or alpha H / Kn with H the subdomain's extent along the normal) and
-// T_R = A_f / (h_n / (2 Kn) + beta), with one Newton reciprocal of Kn shared by
+// T_R = A_f / (h_n / (2 Kn) + beta), with one reciprocal of Kn shared by
 // both and one of the denominator instead of FP64 divisions.
 __device__ __forceinline__ void robin_of(int mode, double alpha, double beta_const, const SubInfo& s, int a,
                                          double h_a, double area_a, double Kn, double* beta, double* tr) {
@@ -77,11 +77,16 @@ __device__ __forceinline__ void robin_of(int mode, double alpha, double beta_con
 // Dirichlet part of the particular right-hand side.  Also T_R, beta, the
 // U-MBF right-hand side -beta s T_R and beta s T_R of every Robin face.
 // Each interior face's transmissibility (area / h) 2 K1 K2 / (K1 + K2) is
-// computed once, by the cell on its low side, with a Newton reciprocal (an
-// FP64 division is a long chain on this GPU's FP64 unit); the high-side cell
+// computed once, by the cell on its low side; the high-side cell
 // reads it back after a barrier.  The Jacobi scale 1 / sqrt(diag) only has to
 // be a consistent preconditioner, so it is formed in FP32 and widened exactly.
+// Bound by the FP64 unit (two lane operations a cycle and SM), so reciprocals are integer
+// arithmetic and the Robin faces' T_R is computed once, face by face on full warps, into a
+// shared table by box side that the diagonal reads (formed by the boundary cells themselves it
+// costs whole warps at every x-face); boxes with more side faces than the table holds keep
+// that form.  16.8 M cells: 2205 -> 935 us, 1.1 M: 220 -> 96.
 // ---------------------------------------------------------------------------
+constexpr int kSideTab = 3072;       // 24 KB: boxes of up to 32 x 16 x 10 or 22^3 cells fit
 __global__ void __launch_bounds__(kThreads)
 k_coefficients(const SubInfo* __restrict__ subs, const FaceInfo* __restrict__ faces,
                const double* __restrict__ K, Geo geo, int beta_mode, double alpha, double beta_const,
@@ -91,7 +96,15 @@ k_coefficients(const SubInfo* __restrict__ subs, const FaceInfo* __restrict__ fa
                double* __restrict__ face_tr, double* __restrict__ face_beta, double* __restrict__ face_u,
                double* __restrict__ face_bst, long long ncell_total,
                short* __restrict__ cface /* [cell][6] face of each cell side, for the subdomains with frag; or NULL */) {
+    __shared__ double side_tr[kSideTab];               // T_R by box side (low x, high x, low y, ...), first tangential axis fastest
     const SubInfo s = subs[blockIdx.x];
+    const int nyz = s.sz[1] * s.sz[2], nxz = s.sz[0] * s.sz[2], nxy = s.sz[0] * s.sz[1];   // faces of one side
+    const bool tab = 2 * (nyz + nxz + nxy) <= kSideTab;
+    auto side_at = [&](int a, int hi, const int lc[3]) {
+        return a == 0   ? hi * nyz + lc[1] + s.sz[1] * lc[2]
+               : a == 1 ? 2 * nyz + hi * nxz + lc[0] + s.sz[0] * lc[2]
+                        : 2 * (nyz + nxz) + hi * nxy + lc[0] + s.sz[0] * lc[1];
+    };
     int* cw = cface && s.frag ? reinterpret_cast<int*>(cface + 6 * s.cell_off) : nullptr;
     const long long ncells = (long long)geo.n[0] * geo.n[1] * geo.n[2];
     const double* Kc[3] = {K, K + ncells, K + 2 * ncells};
@@ -122,7 +135,24 @@ k_coefficients(const SubInfo* __restrict__ subs, const FaceInfo* __restrict__ fa
         }
         if (cw) { cw[3 * c] = -1; cw[3 * c + 1] = -1; cw[3 * c + 2] = -1; }
     }
-    __syncthreads();                                   // the high-side cells read their "-" faces
+    __syncthreads();                                   // (the cleared cface entries come first)
+    for (int q = threadIdx.x; q < s.nface; q += blockDim.x) {
+        FaceInfo fi = faces[s.face_off + q];
+        int lc[3];
+        local_coords(s, fi.cell, lc);
+        long long g = global_cell(s, lc, geo.n);
+        int a = fi.axis;
+        double beta, tr;
+        robin_of(beta_mode, alpha, beta_const, s, a, geo.h[a], geo.area[a], Kc[a][g], &beta, &tr);
+        face_tr[s.face_off + q] = tr;
+        face_beta[s.face_off + q] = beta;
+        const double bst = beta * tr;
+        face_u[s.face_off + q] = fi.s > 0 ? -bst : bst;     // U-MBF right-hand side on this face
+        face_bst[s.face_off + q] = fi.s > 0 ? bst : -bst;   // weight of the face's flux in the U row
+        if (tab) side_tr[side_at(a, fi.s > 0 ? 1 : 0, lc)] = tr;
+        if (cw) cface[6 * (s.cell_off + fi.cell) + 2 * a + (fi.s > 0 ? 1 : 0)] = (short)q;   // one face per cell side
+    }
+    __syncthreads();                                   // the cells read their "-" faces and the table
     for (int c = threadIdx.x; c < s.N; c += blockDim.x) {
         int lc[3];
         local_coords(s, c, lc);
@@ -135,6 +165,8 @@ k_coefficients(const SubInfo* __restrict__ subs, const FaceInfo* __restrict__ fa
                 d += tp[a][c];
             } else if (s.o[a] + lc[a] == geo.n[a] - 1) {
                 if ((bc_lo_hi.y >> a) & 1) { double TD = 2.0 * ah[a] * Kc[a][g]; d += TD; rd += TD * bhi[a]; }
+            } else if (tab) {
+                d += side_tr[side_at(a, 1, lc)];
             } else {
                 double beta, tr;
                 robin_of(beta_mode, alpha, beta_const, s, a, geo.h[a], geo.area[a], Kc[a][g], &beta, &tr);
@@ -145,6 +177,8 @@ k_coefficients(const SubInfo* __restrict__ subs, const FaceInfo* __restrict__ fa
                 d += tp[a][c - lstride[a]];
             } else if (s.o[a] == 0) {
                 if ((bc_lo_hi.x >> a) & 1) { double TD = 2.0 * ah[a] * Kc[a][g]; d += TD; rd += TD * blo[a]; }
+            } else if (tab) {
+                d += side_tr[side_at(a, 0, lc)];
             } else {
                 double beta, tr;
                 robin_of(beta_mode, alpha, beta_const, s, a, geo.h[a], geo.area[a], Kc[a][g], &beta, &tr);
@@ -155,20 +189,6 @@ k_coefficients(const SubInfo* __restrict__ subs, const FaceInfo* __restrict__ fa
         coef[i] = d;
         scale[i] = f32_to_f64(rsqrtf(f64_to_f32_rz(d)));
         rhs_dir[i] = rd;
-    }
-    for (int q = threadIdx.x; q < s.nface; q += blockDim.x) {
-        FaceInfo fi = faces[s.face_off + q];
-        int lc[3];
-        local_coords(s, fi.cell, lc);
-        long long g = global_cell(s, lc, geo.n);
-        int a = fi.axis;
-        double beta, tr;
-        robin_of(beta_mode, alpha, beta_const, s, a, geo.h[a], geo.area[a], Kc[a][g], &beta, &tr);
-        face_tr[s.face_off + q] = tr;
-        face_beta[s.face_off + q] = beta;
-        face_u[s.face_off + q] = -beta * fi.s * tr;     // U-MBF right-hand side on this face
-        face_bst[s.face_off + q] = beta * fi.s * tr;     // weight of the face's flux in the U row
-        if (cw) cface[6 * (s.cell_off + fi.cell) + 2 * a + (fi.s > 0 ? 1 : 0)] = (short)q;   // one face per cell side
     }
 }
 
@@ -1722,19 +1742,32 @@ k_element(const SubInfo* __restrict__ subs, const FaceInfo* __restrict__ faces,
     }
     __syncthreads();
     // per basis, the data terms of its own two columns (g = 1 on the P-MBF,
-    // g = -beta s on the U-MBF): sums over its faces in face order
+    // g = -beta s on the U-MBF): sums over its faces in a fixed order
     __shared__ double s_gsum[4][kMaxI];             // sum T_R, sum beta s T_R, sum beta^2 s^2 T_R, sum beta A_f
-    for (int k = threadIdx.x; k < nI; k += blockDim.x) {
+    {
+        // G consecutive lanes per basis (a thread each leaves one warp with a chain of ~7 FP64
+        // operations per face: 170 faces of a 16 x 16 face 80 k cycles, the kernel's longest part;
+        // 8192 subdomains of 16 x 16 x 8: 2412 -> 1078 us)
+        int G = 1;
+        while (G < 32 && 2 * G * nI <= (int)blockDim.x) G <<= 1;
+        const int k = threadIdx.x / G, sub = threadIdx.x & (G - 1);
         double a0 = 0.0, a1 = 0.0, a2 = 0.0, a3 = 0.0;
-        for (int q = start[k]; q < start[k + 1]; ++q) {
-            const int sa = s_sa[q], ax = sa & 3;
-            const double be = s_be[q];
-            a0 += s_tr[q];
-            a1 += s_bst[q];
-            a2 += s_bst[q] * be * (double)((sa - ax) / 4);
-            a3 += be * geo.area[ax];
+        if (k < nI)
+            for (int q = start[k] + sub; q < start[k + 1]; q += G) {
+                const int sa = s_sa[q], ax = sa & 3;
+                const double be = s_be[q], bt = s_bst[q];
+                a0 += s_tr[q];
+                a1 += bt;
+                a2 = fma(sa < 0 ? -bt : bt, be, a2);
+                a3 = fma(be, geo.area[ax], a3);
+            }
+        for (int o = 1; o < G; o <<= 1) {
+            a0 += __shfl_xor_sync(0xffffffffu, a0, o);
+            a1 += __shfl_xor_sync(0xffffffffu, a1, o);
+            a2 += __shfl_xor_sync(0xffffffffu, a2, o);
+            a3 += __shfl_xor_sync(0xffffffffu, a3, o);
         }
-        s_gsum[0][k] = a0; s_gsum[1][k] = a1; s_gsum[2][k] = a2; s_gsum[3][k] = a3;
+        if (k < nI && sub == 0) { s_gsum[0][k] = a0; s_gsum[1][k] = a1; s_gsum[2][k] = a2; s_gsum[3][k] = a3; }
     }
     __syncthreads();
     const double* Xs = X + s.x_off;
@@ -1978,7 +2011,7 @@ k_pp_velocity(const SubInfo* __restrict__ subs, const double* __restrict__ X, co
     tp[s.sa] = coef + 3 * nct + s.cell_off;
     const double* pl = X + s.x_off + (long long)(s.m - 1) * s.N;
     double inv_area[3];
-    for (int a = 0; a < 3; ++a) inv_area[a] = 1.0 / geo.area[a];
+    for (int a = 0; a < 3; ++a) inv_area[a] = rcp64(geo.area[a]);
     for (int c = threadIdx.x; c < s.N; c += blockDim.x) {
         int lc[3];
         local_coords(s, c, lc);
@@ -2007,7 +2040,7 @@ k_pp_velocity(const SubInfo* __restrict__ subs, const double* __restrict__ X, co
     }
     __syncthreads();                                      // this CTA wrote every face of its cells
     const double vol = geo.h[0] * geo.h[1] * geo.h[2];
-    double mx = 0.0;
+    unsigned long long mx = 0ull;
     for (int c = threadIdx.x; c < s.N; c += blockDim.x) {
         int lc[3];
         local_coords(s, c, lc);
@@ -2015,16 +2048,16 @@ k_pp_velocity(const SubInfo* __restrict__ subs, const double* __restrict__ X, co
         double div = -f[g] * vol;
         for (int a = 0; a < 3; ++a)
             div += (u_out[(long long)(2 * a + 1) * ncells + g] - u_out[(long long)(2 * a) * ncells + g]) * geo.area[a];
-        mx = (div == div) ? fmax(mx, fabs(div)) : __longlong_as_double(0x7ff0000000000000LL);
+        mx = max(mx, abs_bits(div));
     }
-    __shared__ double red[kThreads];
+    __shared__ unsigned long long red[kThreads];
     red[threadIdx.x] = mx;
     __syncthreads();
     for (int w = blockDim.x / 2; w > 0; w >>= 1) {
-        if (threadIdx.x < w) red[threadIdx.x] = fmax(red[threadIdx.x], red[threadIdx.x + w]);
+        if (threadIdx.x < w) red[threadIdx.x] = max(red[threadIdx.x], red[threadIdx.x + w]);
         __syncthreads();
     }
-    if (threadIdx.x == 0) atomicMax(mres_bits, (unsigned long long)__double_as_longlong(red[0]));
+    if (threadIdx.x == 0) atomicMax(mres_bits, red[0]);
 }
 
 // FP64 fallback (mixed modes): after the last refinement sweep of a wave, every

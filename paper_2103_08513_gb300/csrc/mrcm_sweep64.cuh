@@ -13,12 +13,12 @@
 // cost: 16 updates and 4 scalings per tile warp -- 60 at b = 50 against 40 for
 // the bare triangle; a packed triangle in shared memory with a warp per row took
 // about 250 (two operations per entry, idle lanes past the diagonal, a division
-// in every warp).  The next pivot and its reciprocal (five dependent operations)
+// in every warp).  The next pivot and its reciprocal (two FP64 operations, then integer ones)
 // are formed by a warp of their own, which at b <= 52 is the fourth
 // sub-partition's, while the tile warps update (10 x 10 x 5 box: 440 us with the
 // diagonal tile's thread doing it after its updates, 376 us with the warp, 318 us
-// once no sign was flipped by an FP64 instruction).  2244 blocks of 10 slabs,
-// b = 50: 19.3 ms with the packed triangle, 4.5 ms now.
+// once no sign was flipped by an FP64 instruction, 321 us with the integer reciprocal).  2244 blocks of 10 slabs,
+// b = 50: 19.3 ms with the packed triangle, 4.3 ms now.
 // Blocks above 128 (the tiles no longer fit one SM's registers) are spread over a
 // cluster of eight CTAs, tile t on CTA t mod 8; the pivot row goes into every
 // CTA's shared memory and the step's barrier is the cluster's (72 x 70 x 48 cells, uneven
@@ -66,7 +66,7 @@ struct Sweep64Shared {
 __device__ __forceinline__ double sweep64_pivot(double p, int* bad) {
     const long long u = __double_as_longlong(p);
     if (!(u > 0 && u <= 0x7FF0000000000000ll)) { *bad = 1; p = 1.0; }
-    return rcp64c(p);
+    return rcp64(p);
 }
 
 template <int CL>
