@@ -1260,11 +1260,50 @@ __device__ __forceinline__ void block_gemm_tc(const float* __restrict__ Wsm, con
     }
 }
 
+// The product of few columns, a thread per entry; KS > 1: that many adjacent lanes share an
+// entry, each taking every KS-th k, and add their sums by a butterfly.
+template <typename T, typename Store>
+__device__ __forceinline__ void block_gemm_entry(const T* __restrict__ Wsm, const T* __restrict__ Z, int b, int na,
+                                                 int mpad, int KS, Store store) {
+    const int tot = b * na * KS;
+    for (int e0 = threadIdx.x & ~31; e0 < tot; e0 += blockDim.x) {       // (whole warps: the butterfly's)
+        const int e = min(e0 + (int)(threadIdx.x & 31), tot - 1);
+        const int ks = e & (KS - 1), task = e / KS;
+        const int jj = task / b, i = task - jj * b;
+        const T* zc = Z + jj;
+        T acc = (T)0;
+#pragma unroll 4
+        for (int k = ks; k < b; k += KS) acc += Wsm[k * b + i] * zc[k * mpad];
+        for (int o = 1; o < KS; o <<= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+        if (ks == 0 && e0 + (int)(threadIdx.x & 31) < tot) store(i, jj, acc);
+    }
+}
+
 // Dispatch: RT > 0 selects the SIMT tile with RT rows per thread, RT == 0 the
 // 3xTF32 tensor-core path (FP32 operands only), RT < 0 the pair tile (odd b:
-// the one-row tile).
+// the one-row tile).  Few columns leave those tiles on a warp or two, and the FP64 unit of
+// the other schedulers idle.  A pass over one column alone (`single`: the post-processing)
+// shares each entry's k among lanes, b = 50 in FP64: 170 -> 45 us a pass over 126
+// subdomains.  FP64 products of up to two entries a thread take a thread per entry; k
+// stays in order there, so that a column's bits do not depend on how many are active
+// with it (40 x 40 x 8, 4 columns a CTA: with the groups of column_groups, 319 -> 143 us).
 template <typename T, int RT, typename Store>
-__device__ __forceinline__ void block_product(const T* Wsm, const T* Z, int b, int na, int mpad, Store store) {
+__device__ __forceinline__ void block_product(const T* Wsm, const T* Z, int b, int na, int mpad, bool single,
+                                              Store store) {
+    if constexpr (RT != 0) {
+        if (single) {
+            int KS = 1;
+            while (KS < 16 && 2 * KS * b <= (int)blockDim.x) KS <<= 1;
+            block_gemm_entry<T>(Wsm, Z, b, na, mpad, KS, store);
+            return;
+        }
+        if constexpr (std::is_same<T, double>::value) {
+            if (b * na <= 2 * (int)blockDim.x) {
+                block_gemm_entry<T>(Wsm, Z, b, na, mpad, 1, store);
+                return;
+            }
+        }
+    }
     if constexpr (RT < 0) {
         if (b & 1) block_gemm<T, 1>(Wsm, Z, b, na, mpad, store);
         else block_gemm_pair<T>(Wsm, Z, b, na, mpad, store);
@@ -1561,7 +1600,7 @@ __device__ __forceinline__ void solve_one(const LocalArgs& g, const T* __restric
         }
         const T* Wsm = wblock(sl);
         __syncthreads();
-        block_product<T, RT>(Wsm, Z, b, na, mpad, [&](int i, int jj, T v) {
+        block_product<T, RT>(Wsm, Z, b, na, mpad, g.last_only != 0, [&](int i, int jj, T v) {
             Yp[i * mpad + jj] = v;
             Ys[(g.last_only ? 0 : (long long)cols[jj] * N) + base + i] = v;
         });
@@ -1590,7 +1629,7 @@ __device__ __forceinline__ void solve_one(const LocalArgs& g, const T* __restric
             }
             const T* Wsm = wblock(q);
             __syncthreads();
-            block_product<T, RT>(Wsm, Z, b, na, mpad, finish);
+            block_product<T, RT>(Wsm, Z, b, na, mpad, g.last_only != 0, finish);
             __syncthreads();
             refill(q);
         } else {
@@ -2343,14 +2382,25 @@ static LocalArgs local_args(const Tables& t, const DeviceTables& d, const Layout
 }
 
 // CTAs that share a subdomain (by columns) when there are too few subdomains to
-// fill the SMs: as many as give every SM two CTAs, each with eight columns or more.
-// The columns are independent, so the results are those of one CTA.  40 x 40 x 8
-// cells in FP64 (32 subdomains, 53 columns: 7 groups): first solve 769 -> 317 us,
-// sweep 838 -> 342 us; 45 x 38 x 27 (100 subdomains, mixed, 3 groups): 453 -> 259
-// and 1313 -> 698 us.
-static int column_groups(const DeviceTables& d, const LocalArgs& g, int max_m) {
+// fill the SMs.  The columns are independent, so the results are those of one CTA.
+// FP32 (latency-bound): as many as give every SM two CTAs, each with eight columns or
+// more.  FP64 (bound by the SM's FP64 unit, which its CTAs share): the count that minimises
+// the four-column tiles of the fullest SM, at most three CTAs per SM; the larger of
+// equals, which overlaps more.  40 x 40 x 8 cells in FP64 (32 subdomains, 53 columns): one
+// CTA each 769 us (first solve) and 838 (sweep), 6 groups by the FP32 rule (40 SMs with two
+// CTAs, 24 columns) 319 and 340, 14 groups (12 columns) 143 and 159; 45 x 38 x 27 (100
+// subdomains, mixed, 3 groups): 453 -> 259 and 1313 -> 698 us.
+static int column_groups(const DeviceTables& d, const LocalArgs& g, int max_m, bool f64) {
     if (g.last_only || g.nlist <= 0) return 1;
-    return std::max(1, std::min(2 * d.sms / g.nlist, max_m / 8));
+    if (!f64) return std::max(1, std::min(2 * d.sms / g.nlist, max_m / 8));
+    const int top = std::min(3 * d.sms / g.nlist, (max_m + 3) / 4);
+    int best = 1;
+    long long cost = -1;
+    for (int G = 1; G <= top; ++G) {
+        const long long rounds = ((long long)g.nlist * G + d.sms - 1) / d.sms, quads = ((max_m + G - 1) / G + 3) / 4;
+        if (cost < 0 || rounds * quads <= cost) { cost = rounds * quads; best = G; }
+    }
+    return best;
 }
 
 // Launch one local-solve pass (first solve or refinement sweeps) over g.list, whose
@@ -2364,7 +2414,7 @@ static void launch_local_pass(const Tables& t, const DeviceTables& d, const Loca
         BigArgs a;
         a.g = g0;
         a.g.nlist = nbig;
-        a.g.col_groups = column_groups(d, a.g, t.max_m);
+        a.g.col_groups = column_groups(d, a.g, t.max_m, false);
         a.stages = big.stages();
         a.stage_bytes = big.nt * 1024;
         size_t o = (size_t)a.stages * a.stage_bytes;
@@ -2383,7 +2433,7 @@ static void launch_local_pass(const Tables& t, const DeviceTables& d, const Loca
         LocalArgs g = g0;
         g.list += nbig;
         g.nlist -= nbig;
-        g.col_groups = column_groups(d, g, t.max_m);
+        g.col_groups = column_groups(d, g, t.max_m, f64);
         const void* k = f64 ? (sweep ? solve_kernel<double, false, true>(v) : solve_kernel<double, false, false>(v))
                             : (sweep ? solve_kernel<float, true, true>(v) : solve_kernel<float, true, false>(v));
         const int occ = sweep ? d.sweep_occ[v] : d.solve_occ[v];
