@@ -130,12 +130,14 @@ struct Tables {
     int root = -1;
     int pin_front = -1;
 
-    // mixed modes: the FP64 post-processing factors the Neumann problems into
-    // the W region in FP64 waves (pp_wave_off into solve_list; pp_subs are the
-    // subdomain records with the FP64 block offsets and one forward-value
-    // column per cell); pp_ok is false when some block cannot take it
+    // mixed modes: the FP64 post-processing factors the Neumann problems that its FP32 pass
+    // leaves unconverged into the W region, pp_cap slots of pp_stride doubles at a time
+    // (pp_subs: the subdomain records with one forward-value column per cell); pp_ok is false
+    // when some block cannot take it
     std::vector<SubInfo> pp_subs;
-    std::vector<int> pp_wave_off;
+    long long pp_stride = 1;
+    int pp_cap = 1;
+    int pp_chunks() const { return ((int)subs.size() + pp_cap - 1) / pp_cap; }
     bool pp_ok = true;
 };
 
@@ -146,7 +148,8 @@ struct Layout {
     size_t elem, elem_b, csr_val, b_int, dscale, fronts, frhs, panel, oz, oz_exp, xres, xtmp, psum, status;
     size_t bpart, bcnt;    // row-chunk partial sums and counters of the split boundary back substitution
     size_t fb_W, fb_Y, fb_subs, fb_list;   // FP64 fallback: block factors, forward values, subdomain records, slots
-    size_t pp_list;                        // post-processing (mixed): the subdomains its FP32 pass left unconverged
+    size_t pp_list, pp_slots, pp_cnt;      // post-processing (mixed): the subdomains its FP32 pass left unconverged
+                                           // (slot numbers, records), their number in each chunk of slots
     size_t total;
 };
 

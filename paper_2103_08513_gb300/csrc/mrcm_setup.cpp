@@ -297,25 +297,17 @@ mrcm_status build_tables(const mrcm_config* cfg, Tables& t, std::string& err) {
             t.wave_class_off.push_back((int)t.class_list.size());
         }
         for (int k = 0; k < 4; ++k) t.class_off[k] = t.wave_class_off[k];
-        // FP64 post-processing waves of the mixed modes (the W region holds total_w floats)
+        // FP64 post-processing slots of the mixed modes (the W region holds total_w floats)
         if (cfg->precision != MRCM_FP64) {
             t.pp_subs = t.subs;
-            t.pp_wave_off.assign(1, 0);
             const long long cap_d = t.total_w * (long long)sizeof(float) / (long long)sizeof(double);
-            long long cur = 0;
-            for (int q = 0; q < nsub; ++q) {
-                SubInfo& s = t.pp_subs[t.solve_list[q]];
+            for (SubInfo& s : t.pp_subs) {
                 const long long need = (long long)s.ns * wstride<double>(s.b);
                 if (s.b > kMaxBlock64 || need > cap_d) t.pp_ok = false;
-                if (q > t.pp_wave_off.back() && cur + need > cap_d) {
-                    t.pp_wave_off.push_back(q);
-                    cur = 0;
-                }
-                s.w_off = cur;
+                t.pp_stride = std::max(t.pp_stride, need);
                 s.y_off = s.cell_off;      // one column of forward values per cell
-                cur += need;
             }
-            t.pp_wave_off.push_back(nsub);
+            t.pp_cap = (int)std::max(1LL, std::min((long long)nsub, cap_d / t.pp_stride));
         }
     }
     t.total_x = x_off;
@@ -547,6 +539,8 @@ void compute_layout(const Tables& t, Layout& L) {
         L.fb_list = take((size_t)cap * sizeof(int));
     }
     L.pp_list = take((size_t)std::max<size_t>(t.subs.size(), 1) * sizeof(int));
+    L.pp_slots = take(std::max<size_t>(t.pp_subs.size(), 1) * sizeof(SubInfo));
+    L.pp_cnt = take((size_t)(t.pp_chunks() + 1) * sizeof(int));
     L.total = off;
 }
 
