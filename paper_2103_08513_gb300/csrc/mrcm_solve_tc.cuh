@@ -22,10 +22,11 @@
 //     threads on consecutive cells; the product's result passes through shared
 //     memory (P) once.  Two CTAs per SM overlap one's FP64 with the other's products.
 //
-// 256 x 256 x 128 cells, uneven blocks of 64 to 256: first solve 11.5 -> 4.1 ms, six
-// sweeps 37.8 -> 13.6 ms; 256 x 512 x 128 cells, blocks of 128: 11.0 -> 7.4 and
-// 39.5 -> 27.6 ms (there each warp issues an instruction every ~9 cycles at 4.5 warps
-// per scheduler; half of the instructions cut W and feed the products).
+// 256 x 256 x 128 cells, uneven blocks of 64 to 256: first solve 11.5 -> 3.8 ms, six
+// sweeps 37.8 -> 11.6 ms; 256 x 512 x 128 cells, blocks of 128: 11.0 -> 6.5 and
+// 39.5 -> 23.0 ms.  A CTA spends about half of a pass on the entries and a third on the
+// products; neither the instructions that cut W (stored ready cut it was no faster) nor
+// the chain of the six products bounds it.
 #pragma once
 
 constexpr int kBigWarps = 8;                          // consumer warps; one producer warp after them
@@ -271,16 +272,24 @@ k_solve_big(BigArgs a, const float* __restrict__ Wall) {
                         }
                     }
                 };
-                auto put_z = [&](int jj, int i, float z) {
+                auto put_z2 = [&](int jj, int i, float za, float zb) {      // cells i (even) and i + 1
                     uint32_t p1, p2, p3;
-                    cut3(z, 0.0f, p1, p2, p3);
+                    cut3(za, zb, p1, p2, p3);
                     unsigned char* q = Zp + (uint32_t)jj * zs + 2 * i;
-                    *reinterpret_cast<unsigned short*>(q) = (unsigned short)p1;
-                    *reinterpret_cast<unsigned short*>(q + zpl) = (unsigned short)p2;
-                    *reinterpret_cast<unsigned short*>(q + 2 * zpl) = (unsigned short)p3;
+                    *reinterpret_cast<uint32_t*>(q) = p1;
+                    *reinterpret_cast<uint32_t*>(q + zpl) = p2;
+                    *reinterpret_cast<uint32_t*>(q + 2 * zpl) = p3;
                 };
-                // entry walk: (column jj, slab cell i), consecutive threads on consecutive cells
-                const int jj0 = tid / b, i0 = tid - jj0 * b, dj = 256 / b, di = 256 - dj * b;
+                auto particular = [&](int c) {                    // right-hand side of the particular column
+                    int lc[3];
+                    local_coords(s, c, lc);
+                    return g.rhs_dir[s.cell_off + c] + g.f[global_cell(s, lc, g.geo.n)] * vol;
+                };
+                // entry walk: (column jj, slab cells i, i + 1), consecutive threads on consecutive
+                // pairs: the index and address arithmetic, the cut and the stores of Z serve two cells
+                // (the two entry phases were half of a pass, ~100 instructions a cell)
+                const int bp = (b + 1) >> 1;
+                const int jj0 = tid / bp, i0 = tid - jj0 * bp, dj = 256 / bp, di = 256 - dj * bp;
                 stage_load(0, true);
                 stage_store(true);
                 bar_consumers();
@@ -288,52 +297,65 @@ k_solve_big(BigArgs a, const float* __restrict__ Wall) {
                 for (int sl = 0; sl < ns; ++sl) {
                     const int base = sl * b;
                     {
-                        int jj = jj0, i = i0;
-                        for (int e = tid; e < na * b; e += 256) {
+                        int jj = jj0, i = 2 * i0;
+                        for (int e = tid; e < na * bp; e += 256) {
                             const int j = cols[jj];
                             const int c = base + i;
-                            const unsigned mk = msk_s[i];
-                            double r;
+                            const bool two = i + 1 < b;
+                            const long long o = (long long)j * N + c;
+                            const int i1 = two ? i + 1 : i;       // (a lone last cell twice, its second result dropped)
+                            const unsigned mk0 = msk_s[i], mk1 = msk_s[i1];
+                            double r0 = 0.0, r1 = 0.0;
                             if (j == m - 1) {
-                                int lc[3];
-                                local_coords(s, c, lc);
-                                r = g.rhs_dir[s.cell_off + c] + g.f[global_cell(s, lc, g.geo.n)] * vol;
+                                r0 = particular(c);
+                                r1 = two ? particular(c + 1) : 0.0;
                             } else {
-                                r = 0.0;
                                 const int kb = j < nI ? j : j - nI;
-                                if ((mk >> (kb & 15)) & 1u) {
+                                if (((mk0 | mk1) >> (kb & 15)) & 1u) {
+                                    const double* fv = (j < nI ? g.face_tr : g.face_u) + s.face_off;
 #pragma unroll
-                                    for (int q = 0; q < 6; ++q)
-                                        if (fcol_s[6 * i + q] == kb) {
-                                            const int f = s.face_off + fq_s[6 * i + q];
-                                            r = j < nI ? g.face_tr[f] : g.face_u[f];
-                                        }
+                                    for (int q = 0; q < 6; ++q) {
+                                        if (fcol_s[6 * i + q] == kb) r0 = fv[fq_s[6 * i + q]];
+                                        if (fcol_s[6 * i1 + q] == kb) r1 = fv[fq_s[6 * i1 + q]];
+                                    }
                                 }
                             }
-                            if (kSweep) {                     // r - A x as one FMA chain
-                                const double* x = Xs + (long long)j * N;
-                                r = fma(-co_d[i], x[c], r);
-                                if (mk & kNbUp) r = fma(co_u[i], x[c + 1], r);
-                                if (mk & kNbUm) r = fma(co_u[i - 1], x[c - 1], r);
-                                if (mk & kNbVp) r = fma(co_v[i], x[c + su], r);
-                                if (mk & kNbVm) r = fma(co_v[i - su], x[c - su], r);
-                                if (c + b < N) r = fma(co_sp[i], x[c + b], r);
-                                if (sl > 0) r = fma(co_sm[i], x[c - b], r);
+                            if (kSweep) {                     // r - A x as one FMA chain each
+                                const double* x = Xs + o;
+                                const double xa = x[0], xb = two ? x[1] : 0.0;
+                                r0 = fma(-co_d[i], xa, r0);
+                                if (mk0 & kNbUp) r0 = fma(co_u[i], xb, r0);
+                                if (mk0 & kNbUm) r0 = fma(co_u[i - 1], x[-1], r0);
+                                if (mk0 & kNbVp) r0 = fma(co_v[i], x[su], r0);
+                                if (mk0 & kNbVm) r0 = fma(co_v[i - su], x[-su], r0);
+                                if (sl + 1 < ns) r0 = fma(co_sp[i], x[b], r0);
+                                if (sl > 0) r0 = fma(co_sm[i], x[-b], r0);
+                                if (two) {
+                                    r1 = fma(-co_d[i1], xb, r1);
+                                    if (mk1 & kNbUp) r1 = fma(co_u[i1], x[2], r1);
+                                    if (mk1 & kNbUm) r1 = fma(co_u[i], xa, r1);
+                                    if (mk1 & kNbVp) r1 = fma(co_v[i1], x[su + 1], r1);
+                                    if (mk1 & kNbVm) r1 = fma(co_v[i1 - su], x[1 - su], r1);
+                                    if (sl + 1 < ns) r1 = fma(co_sp[i1], x[b + 1], r1);
+                                    if (sl > 0) r1 = fma(co_sm[i1], x[1 - b], r1);
+                                }
                             }
-                            const float rf = f64_to_f32_rz(r);
-                            float z = rf * sc_s[i];
-                            float* pp = &P[jj * ldp + i];
+                            const float f0 = f64_to_f32_rz(r0), f1 = two ? f64_to_f32_rz(r1) : 0.0f;
+                            float z0 = f0 * sc_s[i], z1 = f1 * sc_s[i1];
+                            float2* pp = reinterpret_cast<float2*>(&P[jj * ldp + i]);
                             if (sl > 0) {
-                                const float y = *pp;          // Y of the previous slab
-                                Ys[(g.last_only ? 0 : (long long)j * N) + c - b] = y;
-                                z = fmaf(t_s[i], y, z);
+                                const float2 y = *pp;         // Y of the previous slab
+                                float* yo = Ys + (g.last_only ? (long long)c : o) - b;
+                                yo[0] = y.x;
+                                z0 = fmaf(t_s[i], y.x, z0);
+                                if (two) { yo[1] = y.y; z1 = fmaf(t_s[i1], y.y, z1); }
                             }
-                            const float rn = rf * rsb[jj];
-                            *pp = rn * rn;                    // parked for the column's norm
-                            put_z(jj, i, z);
-                            i += di;
+                            const float sb = rsb[jj], n0 = f0 * sb, n1 = f1 * sb;
+                            *pp = make_float2(n0 * n0, n1 * n1);    // parked for the column's norm
+                            put_z2(jj, i, z0, z1);
+                            i += 2 * di;
                             jj += dj;
-                            if (i >= b) { i -= b; ++jj; }
+                            if (i >= 2 * bp) { i -= 2 * bp; ++jj; }
                         }
                     }
                     bar_consumers();
@@ -353,18 +375,25 @@ k_solve_big(BigArgs a, const float* __restrict__ Wall) {
                 // ---- backward sweep: P holds x of the last slab, then W_s (t x_{s+1})
                 for (int sl = ns - 1; sl >= 0; --sl) {
                     const int base = sl * b;
-                    int jj = jj0, i = i0;
-                    for (int e = tid; e < na * b; e += 256) {
-                        const int j = cols[jj];
-                        float x = P[jj * ldp + i];
-                        if (sl + 1 < ns) x += Ys[(g.last_only ? 0 : (long long)j * N) + base + i];
-                        double* xp = Xs + (long long)j * N + base + i;
-                        const double xo = f32_to_f64(x * sc_s[i]);
-                        if (kSweep) *xp += xo; else *xp = xo;
-                        if (sl > 0) put_z(jj, i, t_s[i] * x);
-                        i += di;
+                    int jj = jj0, i = 2 * i0;
+                    for (int e = tid; e < na * bp; e += 256) {
+                        const bool two = i + 1 < b;
+                        const int i1 = two ? i + 1 : i;
+                        const long long o = (long long)cols[jj] * N + base + i;
+                        float2 x = *reinterpret_cast<const float2*>(&P[jj * ldp + i]);
+                        if (sl + 1 < ns) {
+                            const float* y = Ys + (g.last_only ? (long long)(base + i) : o);
+                            x.x += y[0];
+                            if (two) x.y += y[1];
+                        }
+                        double* xp = Xs + o;
+                        const double x0 = f32_to_f64(x.x * sc_s[i]), x1 = f32_to_f64(x.y * sc_s[i1]);
+                        if (kSweep) { xp[0] += x0; if (two) xp[1] += x1; }
+                        else { xp[0] = x0; if (two) xp[1] = x1; }
+                        if (sl > 0) put_z2(jj, i, t_s[i] * x.x, two ? t_s[i1] * x.y : 0.0f);
+                        i += 2 * di;
                         jj += dj;
-                        if (i >= b) { i -= b; ++jj; }
+                        if (i >= 2 * bp) { i -= 2 * bp; ++jj; }
                     }
                     if (sl == 0) break;
                     bar_consumers();
