@@ -335,6 +335,7 @@ enum StatusWord { ST_NOT_SPD = 0, ST_UNCONVERGED = 1, ST_ZERO_PIVOT = 2, ST_SWEE
                   ST_FB_TOTAL = 7 /* subdomains re-solved in FP64 */,
                   ST_SWEPT = 8 /* 64-bit counter at words 8-9 */,
                   ST_FB_LOST = 10 /* subdomains that needed the fallback and could not have it */,
+                  ST_QUEUE2 = 14 /* work-queue counter of the pass's second launch */,
                   ST_CG_ITERS = 12 /* 64-bit counter at words 12-13: CG iterations of the learned form */,
                   ST_COUNT = 16 };
 

@@ -1722,6 +1722,8 @@ k_local_solve(LocalArgs g, const T* __restrict__ Wall) {
                                                   g.count_unconverged && ps + 1 == np, smem_raw, pipe);
     }
     drain_pipe(pipe, bar);
+    // launched beside k_solve_big (launch_local_pass): not complete before it is
+    asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 #include "mrcm_solve_tc.cuh"
@@ -2453,6 +2455,7 @@ static void launch_local_pass(const Tables& t, const DeviceTables& d, const Loca
         a.bars = (int)o;
         const int grid = std::max(1, std::min(nbig * a.g.col_groups, d.sms * d.big_occ[sweep]));
         MRCM_LAUNCH(P, "k_set_int", st, k_set_int<<<1, 1, 0, st>>>(g0.queue, 0));
+        if (g0.nlist > nbig) MRCM_LAUNCH(P, "k_set_int", st, k_set_int<<<1, 1, 0, st>>>(g0.queue + (ST_QUEUE2 - ST_QUEUE), 0));
         void* args[] = {(void*)&a, (void*)&W};
         MRCM_LAUNCH(P, name, st, cudaLaunchKernel(big_kernel(sweep, big.units), dim3(grid), dim3(kBigThreads), args, big.total(), st));
     }
@@ -2465,9 +2468,28 @@ static void launch_local_pass(const Tables& t, const DeviceTables& d, const Loca
                             : (sweep ? solve_kernel<float, true, true>(v) : solve_kernel<float, true, false>(v));
         const int occ = sweep ? d.sweep_occ[v] : d.solve_occ[v];
         const int grid = std::max(1, std::min(g.nlist * g.col_groups, d.sms * occ));
-        MRCM_LAUNCH(P, "k_set_int", st, k_set_int<<<1, 1, 0, st>>>(g.queue, 0));
         void* args[] = {(void*)&g, (void*)&W};
-        MRCM_LAUNCH(P, name, st, cudaLaunchKernel(k, dim3(grid), dim3(variant_threads(v)), args, d.solve_smem, st));
+        if (nbig > 0) {
+            // beside k_solve_big, on other subdomains with a queue of its own (programmatic launch: it
+            // starts once every CTA of k_solve_big has, and ends after it).  Few subdomains of both kinds
+            // are two chains of slabs: 69 x 81 x 23 cells in 12 x 12 x 8, whole solve 2.00 ms one after
+            // the other, 1.54 so (1.86 when one kernel took both kinds)
+            g.queue += ST_QUEUE2 - ST_QUEUE;
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3(grid);
+            cfg.blockDim = dim3(variant_threads(v));
+            cfg.dynamicSmemBytes = d.solve_smem;
+            cfg.stream = st;
+            cudaLaunchAttribute at[1];
+            at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+            at[0].val.programmaticStreamSerializationAllowed = 1;
+            cfg.attrs = at;
+            cfg.numAttrs = 1;
+            MRCM_LAUNCH(P, name, st, cudaLaunchKernelExC(&cfg, k, args));
+        } else {
+            MRCM_LAUNCH(P, "k_set_int", st, k_set_int<<<1, 1, 0, st>>>(g.queue, 0));
+            MRCM_LAUNCH(P, name, st, cudaLaunchKernel(k, dim3(grid), dim3(variant_threads(v)), args, d.solve_smem, st));
+        }
     }
 }
 

@@ -65,6 +65,7 @@ template <bool kSweep, int U>
 __global__ void __launch_bounds__(kBigThreads, U <= 2 ? 2 : 1)
 k_solve_big(BigArgs a, const float* __restrict__ Wall) {
     extern __shared__ __align__(128) unsigned char smem_ls[];
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the pass's launch for the smaller blocks may join
     const LocalArgs& g = a.g;
     unsigned char* sm = smem_ls;
     unsigned long long* full = reinterpret_cast<unsigned long long*>(sm + a.bars);
