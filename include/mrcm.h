@@ -109,8 +109,8 @@ enum {
  *                     wave (their FP64 block factors take a workspace region
  *                     of that many slots); 0 = default max(16, n_sub / 64)
  *                     (at most n_sub), -1 = no fallback.  Subdomains beyond
- *                     the cap, or with slab blocks above 224 (the FP64 factor's
- *                     limit), stay unconverged and are counted by
+ *                     the cap, or with slab blocks above 224 (the largest a
+ *                     slot is sized for), stay unconverged and are counted by
  *                     mrcm_read_status */
 typedef struct {
     int nx, ny, nz;
@@ -214,7 +214,7 @@ mrcm_status mrcm_solve_mbf(mrcm_handle* h, const double* f, void* ws, void* stre
 mrcm_status mrcm_assemble_interface(mrcm_handle* h, void* ws, void* stream);
 
 /* Solve the interface system with the factor of mrcm_assemble_interface and
- * two FP64 iterative-refinement steps (CSR residuals).
+ * interface_refine FP64 iterative-refinement steps (CSR residuals).
  *  X   device, FP64 [2*NV], output */
 mrcm_status mrcm_solve_interface(mrcm_handle* h, double* X, void* ws, void* stream);
 
@@ -338,8 +338,9 @@ mrcm_status mrcm_read_tuning_times(const mrcm_handle* h, float* solve_ms, float*
 /* The kernel variants the handle uses (host only; after mrcm_autotune or a
  * tune-cache hit, else the defaults): local solve first pass and refinement
  * sweep (0-11), factor for blocks with b <= 64 (0 a row per thread, 1 8x8
- * register tiles, 2 4x4 tiles) and for 64 < b <= 128 (0 register tiles,
- * 1 tensor cores with the block in tensor memory).  Any pointer may be NULL. */
+ * register tiles, 2 4x4 tiles) and for 64 < b <= 128 (0 tensor cores with the
+ * block in registers, 1 with the block in tensor memory).  The solve variants
+ * serve blocks with b <= 64 and FP64; larger mixed blocks have one solve kernel.  Any pointer may be NULL. */
 mrcm_status mrcm_query_tuning(const mrcm_handle* h, int* solve_variant, int* sweep_variant, int* factor_small,
                               int* factor_mid);
 
