@@ -338,9 +338,11 @@ mrcm_status mrcm_read_tuning_times(const mrcm_handle* h, float* solve_ms, float*
 /* The kernel variants the handle uses (host only; after mrcm_autotune or a
  * tune-cache hit, else the defaults): local solve first pass and refinement
  * sweep (0-11), factor for blocks with b <= 64 (0 a row per thread, 1 8x8
- * register tiles, 2 4x4 tiles) and for 64 < b <= 128 (0 tensor cores with the
- * block in registers, 1 with the block in tensor memory).  The solve variants
- * serve blocks with b <= 64 and FP64; larger mixed blocks have one solve kernel.  Any pointer may be NULL. */
+ * register tiles, 2 4x4 tiles) and for 64 < b <= 128 (0 register tiles,
+ * 1 tensor cores with the block in tensor memory).  The solve variants serve
+ * blocks with b <= 64, FP64 and the larger mixed blocks whose right-hand sides
+ * do not fit one CTA; the other mixed blocks have one solve kernel.  Any pointer
+ * may be NULL. */
 mrcm_status mrcm_query_tuning(const mrcm_handle* h, int* solve_variant, int* sweep_variant, int* factor_small,
                               int* factor_mid);
 

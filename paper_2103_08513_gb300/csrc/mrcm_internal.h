@@ -43,7 +43,7 @@ struct SubInfo {
     long long cell_off;   // offset into per-cell arrays
     long long x_off;      // offset (doubles) into the MBF array [m][N]
     long long y_off;      // offset (elements) of the forward-sweep values Y (= x_off; a slot for the FP64 fallback)
-    int frag;             // FP32 block factor in fragment order (frag_off), solved by k_solve_big
+    int stream;           // mixed modes: solved by k_solve_big, which streams the block factors (big_ok)
     long long w_off;      // offset (elements) into the block factor array
     long long el_off;     // offset (doubles) into element matrices
     int elb_off;          // offset (doubles) into element right-hand sides
@@ -97,10 +97,10 @@ struct Tables {
     // (offsets into class_list); block factors are stored per wave (w_off is
     // relative to the wave) so one W region serves every wave
     std::vector<int> wave_off;
-    std::vector<int> wave_big;         // per wave: its first so many subdomains have SubInfo::frag
+    std::vector<int> wave_big;         // per wave: its first so many subdomains have SubInfo::stream
     std::vector<int> wave_class_off;   // 4 entries per wave (class boundaries)
     int n_waves = 1;
-    int class_off[4] = {0, 0, 0, 0};  // class 0: b <= kRegBlock, 1: fragment-order factors, 2: the other larger blocks (mixed); FP64: all in 2
+    int class_off[4] = {0, 0, 0, 0};  // class 0: b <= kRegBlock, 1: b <= kTileBlock, 2: larger (mixed); FP64: all in 2
     long long n_cells = 0, total_x = 0, total_w = 0, total_el = 0;
     int total_elb = 0;
     int max_m = 0, max_b = 0, max_el = 0, max_N = 0;
@@ -144,7 +144,7 @@ struct Tables {
 // Workspace layout (byte offsets into the caller's workspace).
 struct Layout {
     size_t coef, scale, scf, tsc, rhs_part, face_tr, face_beta, face_u, face_bst, W, X, R, colnorm, conv;
-    size_t cface;          // [cell][6] face of each cell side (mixed modes with fragment-order factors)
+    size_t cface;          // [cell][6] face of each cell side (mixed modes with k_solve_big)
     size_t elem, elem_b, csr_val, b_int, dscale, fronts, frhs, panel, oz, oz_exp, xres, xtmp, psum, status;
     size_t bpart, bcnt;    // row-chunk partial sums and counters of the split boundary back substitution
     size_t fb_W, fb_Y, fb_subs, fb_list;   // FP64 fallback: block factors, forward values, subdomain records, slots
@@ -258,42 +258,24 @@ inline SolveSmem solve_smem_layout(int b, int mpad, int N) {
     return L;
 }
 
-// Fragment order of an FP32 block factor (SubInfo::frag): nt x nt tiles of 16 x 16
-// entries (nt = ceil(b / 16), zero past b), stored as panels of 16 columns j, each
-// the nt tiles of its rows; inside a tile the two halves of eight columns, and in
-// each the 32 lanes' four values as mma.m16n8k16 takes its A operand (rows g and
-// g + 8, columns 2t and 2t + 1 for lane 4 g + t): one conflict-free 16-byte shared
-// load per lane and half, and a contiguous panel per bulk copy.
-#ifdef __CUDACC__
-__host__ __device__
-#endif
-inline long long frag_stride(int b) { const long long nt = (b + 15) >> 4; return 256 * nt * nt; }
-#ifdef __CUDACC__
-__host__ __device__
-#endif
-inline int frag_off(int nt, int i, int j) {
-    return ((j >> 4) * nt + (i >> 4)) * 256 + ((j >> 3) & 1) * 128 + ((i & 7) * 4 + ((j & 7) >> 1)) * 4 + ((i >> 3) & 1) * 2 + (j & 1);
-}
-
-// Shared memory of k_solve_big for blocks up to b and m right-hand sides: per 16
-// columns the three BF16 planes of Z and the product P, one slab's staged data, the
-// column lists, and a ring of W panels.
-constexpr int kBigMinB = 65;       // smaller blocks keep the SIMT products (k_local_solve)
-constexpr int kBigUnits = 64;      // most 16 x 16 output tiles of a product
+// Shared memory of k_solve_big for blocks up to b and m right-hand sides: per column Z
+// and the product P, one slab's staged data, the column lists, and a ring of W panels
+// of 16 rows.
+constexpr int kBigMinB = 65;       // smaller blocks take k_local_solve
+constexpr int kBigUnits = 64;      // most 16 x 16 tiles of a product (eight a warp)
 struct BigSmem {
-    size_t zp = 0, p = 0, co = 0, cols = 0;    // sizes (bytes)
+    size_t zp = 0, co = 0, cols = 0;           // sizes (bytes); zp: of Z, and of P
     int nt = 0, units = 0;
     void add(int b, int m) {
-        const size_t t = (b + 15) / 16, nc = (size_t)(m + 15) / 16 * 16;
-        zp = std::max(zp, 3 * nc * (32 * t + 16));
-        p = std::max(p, nc * (16 * t + 4) * sizeof(float));
+        const size_t t = (b + 15) / 16, nc = (size_t)(m + 7) / 8 * 8;
+        zp = std::max(zp, nc * (16 * t + 4) * sizeof(float));
         co = std::max(co, (size_t)b * (5 * sizeof(double) + 2 * sizeof(float) + sizeof(unsigned) + 6 * sizeof(short) + 6));
         cols = std::max(cols, nc * (sizeof(int) + 2 * sizeof(float)));
         nt = std::max(nt, (int)t);
-        units = std::max(units, (int)(t * nc / 16));
+        units = std::max(units, (int)t * ((m + 15) / 16));
     }
     static size_t al(size_t v) { return (v + 127) & ~size_t(127); }
-    size_t rest() const { return al(zp) + al(p) + al(co) + al(cols) + 256; }
+    size_t rest() const { return 2 * al(zp) + al(co) + al(cols) + 256; }
     // ring stages: eight if two CTAs then fit an SM, at least three of them; more shared memory for one CTA otherwise
     int stages() const {
         const size_t st = (size_t)nt * 1024;

@@ -95,7 +95,7 @@ k_coefficients(const SubInfo* __restrict__ subs, const FaceInfo* __restrict__ fa
                double* __restrict__ coef, double* __restrict__ scale, double* __restrict__ rhs_dir,
                double* __restrict__ face_tr, double* __restrict__ face_beta, double* __restrict__ face_u,
                double* __restrict__ face_bst, long long ncell_total,
-               short* __restrict__ cface /* [cell][6] face of each cell side, for the subdomains with frag; or NULL */) {
+               short* __restrict__ cface /* [cell][6] face of each cell side, for the subdomains with stream; or NULL */) {
     __shared__ double side_tr[kSideTab];               // T_R by box side (low x, high x, low y, ...), first tangential axis fastest
     const SubInfo s = subs[blockIdx.x];
     const int nyz = s.sz[1] * s.sz[2], nxz = s.sz[0] * s.sz[2], nxy = s.sz[0] * s.sz[1];   // faces of one side
@@ -105,7 +105,7 @@ k_coefficients(const SubInfo* __restrict__ subs, const FaceInfo* __restrict__ fa
                : a == 1 ? 2 * nyz + hi * nxz + lc[0] + s.sz[0] * lc[2]
                         : 2 * (nyz + nxz) + hi * nxy + lc[0] + s.sz[0] * lc[1];
     };
-    int* cw = cface && s.frag ? reinterpret_cast<int*>(cface + 6 * s.cell_off) : nullptr;
+    int* cw = cface && s.stream ? reinterpret_cast<int*>(cface + 6 * s.cell_off) : nullptr;
     const long long ncells = (long long)geo.n[0] * geo.n[1] * geo.n[2];
     const double* Kc[3] = {K, K + ncells, K + 2 * ncells};
     const long long stride[3] = {1, geo.n[0], (long long)geo.n[0] * geo.n[1]};
@@ -688,20 +688,11 @@ k_block_factor_tc(const SubInfo* __restrict__ subs, const int* __restrict__ list
         if (stop_s) break;
         // W_s: row i of the swept matrix (every lane loads: the TMEM loads are warp-collective)
         {
-            const int nt16 = (b + 15) >> 4;
-            float* Wf = W + (long long)sl * frag_stride(b);
             float* row = W + (long long)sl * wstride<float>(b) + (long long)min(i, b - 1) * b;
             for (int c0 = 0; c0 < kTcN; c0 += 16) {
                 float v[16];
                 tm_ld16(trow + c0, v);
-                if (s.frag) {
-                    if (i < 16 * nt16 && c0 < 16 * nt16) {
-#pragma unroll
-                        for (int q = 0; q < 16; q += 2)
-                            *reinterpret_cast<float2*>(Wf + frag_off(nt16, i, c0 + q)) =
-                                make_float2(i < b && c0 + q < b ? v[q] : 0.0f, i < b && c0 + q + 1 < b ? v[q + 1] : 0.0f);
-                    }
-                } else if (i < b) {
+                if (i < b) {
 #pragma unroll
                     for (int q = 0; q < 16; ++q)
                         if (c0 + q < b) row[c0 + q] = v[q];
@@ -1363,7 +1354,7 @@ struct LocalArgs {
     const int* nlist_dev; // when set: the list holds min(nlist, *nlist_dev) subdomains (written by an earlier kernel)
     int col_groups;       // > 1: up to this many CTAs share a subdomain, each taking the columns j = grp mod G
                           // (G = min(col_groups, grid / subdomains)); 1: one CTA per subdomain
-    const short* cface;   // [cell][6] face of each cell side (fragment-order subdomains)
+    const short* cface;   // [cell][6] face of each cell side (subdomains of k_solve_big)
     int passes;           // refinement sweeps run back to back on each subdomain by one launch (sweeps only)
 };
 
@@ -1726,8 +1717,7 @@ k_local_solve(LocalArgs g, const T* __restrict__ Wall) {
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
-#include "mrcm_solve_tc.cuh"
-#include "mrcm_factor_tc.cuh"
+#include "mrcm_solve_stream.cuh"
 
 // Tunable variants of the local solve: threads per CTA x block-product path
 // (SIMT with 2, 1 or 4 rows per thread, the pair tile, or 3xTF32 tensor
@@ -2199,17 +2189,6 @@ static void launch_factor64(const SubInfo* subs, const int* list, int n, int bma
     MRCM_LAUNCH(P, name, st, cudaLaunchKernelExC(&cfg, k, args));
 }
 
-// CTA shape of k_block_factor_mma by the number of tile rows: as few warps as hold the
-// tiles in registers, so that as many blocks as possible are in flight on an SM (the step
-// is a chain; 8 warps of 5 tiles for b = 128, three CTAs, took 17.3 ms where 4 of 9, four
-// CTAs, take 16.0): nt <= 8: 4 warps of 2 + 7, nt = 9: 8 of 2 + 5, nt <= 12: 16 of 1 + 5,
-// nt <= 16: 16 of 1 + 8.
-static int factor_mma_shape(int b) { return b <= 128 ? 0 : b <= 144 ? 1 : b <= 192 ? 2 : 3; }
-static const void* factor_mma_kernel(int shape) {
-    return shape == 0 ? (const void*)k_block_factor_mma<4, 9, 2, 4> : shape == 1 ? (const void*)k_block_factor_mma<8, 7, 2, 2>
-         : shape == 2 ? (const void*)k_block_factor_mma<16, 6, 1, 1> : (const void*)k_block_factor_mma<16, 9, 1, 1>;
-}
-
 static void launch_factor_wave(const Tables& t, const DeviceTables& d, const Layout& L, char* ws, int precision,
                                int w, cudaStream_t st, Prof& P) {
     double* coef = (double*)(ws + L.coef);
@@ -2217,9 +2196,8 @@ static void launch_factor_wave(const Tables& t, const DeviceTables& d, const Lay
     int* status = (int*)(ws + L.status);
     const int* wc = &t.wave_class_off[4 * w];
     const int o0 = wc[0], o1 = wc[1], o2 = wc[2], o3 = wc[3];
-    const int n_small = o1 - o0, n_mid = o2 - o1, n_large = o3 - o2;
+    const int n_small = o1 - o0, n_mid = o2 - o1;
     if (precision == MRCM_FP64) {
-        (void)n_large;
         // ordered by b, largest first: one launch per run of subdomains that share a CTA size
         for (int q = o2; q < o3;) {
             const int b0 = t.subs[t.class_list[q]].b, nth = sweep64_threads(b0);
@@ -2241,41 +2219,26 @@ static void launch_factor_wave(const Tables& t, const DeviceTables& d, const Lay
                 MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_tile<4, 16><<<n_small, 256, 0, st>>>(d.subs, d.class_list + o0, coef, scale,
                     (float*)(ws + L.W), status, t.n_cells, (float*)(ws + L.scf), (float*)(ws + L.tsc)));
         }
-        // 64 < b: fragment-order factors first (ordered by b, largest first, one launch per CTA
-        // shape; up to b = 128 the tuner may choose the kernel with the block in tensor memory),
-        // then the blocks with too many right-hand sides for k_solve_big
-        float* W = (float*)(ws + L.W);
-        float* scf = (float*)(ws + L.scf);
-        float* tsc = (float*)(ws + L.tsc);
-        int q = o1;
-        while (q < o3 && t.subs[t.class_list[q]].frag) {
-            const int b0 = t.subs[t.class_list[q]].b, shape = factor_mma_shape(b0);
-            int e = q + 1;
-            while (e < o3 && t.subs[t.class_list[e]].frag && factor_mma_shape(t.subs[t.class_list[e]].b) == shape) ++e;
-            const int n = e - q;
-            const int* lst = d.class_list + q;
-            const size_t sm = factor_mma_smem(b0);
-            if (shape == 0 && d.factor_mid_variant == 1)    // its shared memory keeps <= 4 CTAs (4 x 128 TMEM columns) per SM
-                MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_tc<<<n, kTcN, kTcSmem, st>>>(d.subs, lst, coef, scale, W, status, t.n_cells, scf, tsc));
-            else {
-                const void* k = factor_mma_kernel(shape);
-                void* args[] = {(void*)&d.subs, (void*)&lst, (void*)&coef, (void*)&scale, (void*)&W, (void*)&status, (void*)&t.n_cells, (void*)&scf, (void*)&tsc};
-                MRCM_LAUNCH(P, "k_block_factor", st, cudaLaunchKernel(k, dim3(n), dim3(shape == 0 ? 128 : shape == 1 ? 256 : 512), args, sm, st));
-            }
-            q = e;
+        if (n_mid > 0) {
+            if (d.factor_mid_variant == 1)       // tensor cores; its shared memory keeps <= 4 CTAs (4 x 128 TMEM columns) per SM
+                MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_tc<<<n_mid, kTcN, kTcSmem, st>>>(d.subs, d.class_list + o1, coef, scale,
+                    (float*)(ws + L.W), status, t.n_cells, (float*)(ws + L.scf), (float*)(ws + L.tsc)));
+            else
+                MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_tile<8, 16><<<n_mid, 256, 0, st>>>(d.subs, d.class_list + o1, coef, scale,
+                    (float*)(ws + L.W), status, t.n_cells, (float*)(ws + L.scf), (float*)(ws + L.tsc)));
         }
-        (void)n_mid;
         // the large class is ordered by b, largest first: one launch per run of
         // subdomains that share a thread count
-        while (q < o3) {
-            auto cta = [&](int k) { const int b = t.subs[t.class_list[k]].b; return b <= kTileBlock ? 256 : tri_threads(b); };
-            const int nth = cta(q);
+        for (int q = o2; q < o3;) {
+            const int nth = tri_threads(t.subs[t.class_list[q]].b);
             int e = q + 1;
-            while (e < o3 && cta(e) == nth) ++e;
+            while (e < o3 && tri_threads(t.subs[t.class_list[e]].b) == nth) ++e;
             const int n = e - q;
             const int* lst = d.class_list + q;
+            float* W = (float*)(ws + L.W);
+            float* scf = (float*)(ws + L.scf);
+            float* tsc = (float*)(ws + L.tsc);
             switch (nth) {
-            case 256: MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_tile<8, 16><<<n, 256, 0, st>>>(d.subs, lst, coef, scale, W, status, t.n_cells, scf, tsc)); break;
             case 192: MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_tri<192><<<n, 192, 0, st>>>(d.subs, lst, coef, scale, W, status, t.n_cells, scf, tsc)); break;
             case 320: MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_tri<320><<<n, 320, 0, st>>>(d.subs, lst, coef, scale, W, status, t.n_cells, scf, tsc)); break;
             case 512: MRCM_LAUNCH(P, "k_block_factor", st, k_block_factor_tri<512><<<n, 512, 0, st>>>(d.subs, lst, coef, scale, W, status, t.n_cells, scf, tsc)); break;
@@ -2317,22 +2280,20 @@ static size_t solve_smem_bytes(const Tables& t, int precision) {
     const int mpad = (t.max_m + 3) & ~3;
     size_t sm = 0;
     for (const SubInfo& sb : t.subs)
-        if (!sb.frag) sm = std::max(sm, precision == MRCM_FP64 ? solve_smem_layout<double>(sb.b, mpad, sb.N).total
+        if (!sb.stream) sm = std::max(sm, precision == MRCM_FP64 ? solve_smem_layout<double>(sb.b, mpad, sb.N).total
                                                  : solve_smem_layout<float>(sb.b, mpad, sb.N).total);
     return sm + 16;                                // + the two mbarriers, after the largest layout
 }
 
 static BigSmem big_smem(const Tables& t) {
     BigSmem b;
-    for (const SubInfo& s : t.subs) if (s.frag) b.add(s.b, s.m);
+    for (const SubInfo& s : t.subs) if (s.stream) b.add(s.b, s.m);
     return b;
 }
 static const void* big_kernel(bool sweep, int units) {
-    const int U = (units + kBigWarps - 1) / kBigWarps;
-    if (sweep) return U <= 1 ? (const void*)k_solve_big<true, 1> : U <= 2 ? (const void*)k_solve_big<true, 2>
-                    : U <= 4 ? (const void*)k_solve_big<true, 4> : (const void*)k_solve_big<true, 8>;
-    return U <= 1 ? (const void*)k_solve_big<false, 1> : U <= 2 ? (const void*)k_solve_big<false, 2>
-         : U <= 4 ? (const void*)k_solve_big<false, 4> : (const void*)k_solve_big<false, 8>;
+    const int U = (units + 2 * kBigWarps - 1) / (2 * kBigWarps);     // pairs of 16 x 16 tiles a warp
+    if (sweep) return U <= 1 ? (const void*)k_solve_big<true, 1> : U <= 2 ? (const void*)k_solve_big<true, 2> : (const void*)k_solve_big<true, 4>;
+    return U <= 1 ? (const void*)k_solve_big<false, 1> : U <= 2 ? (const void*)k_solve_big<false, 2> : (const void*)k_solve_big<false, 4>;
 }
 
 // One-time kernel configuration (dynamic shared memory limits, persistent
@@ -2381,8 +2342,6 @@ int configure_local(const Tables& t, DeviceTables& d) {
         d.f64_occ = std::max(1, occ);
     }
     cudaFuncSetAttribute(k_block_factor_tc, cudaFuncAttributeMaxDynamicSharedMemorySize, kTcSmem);
-    for (int b : {128, 144, 192, 256})
-        cudaFuncSetAttribute(factor_mma_kernel(factor_mma_shape(b)), cudaFuncAttributeMaxDynamicSharedMemorySize, (int)factor_mma_smem(b));
     return (int)cudaGetLastError();
 }
 
@@ -2433,7 +2392,7 @@ static int column_groups(const DeviceTables& d, const LocalArgs& g, int max_m, b
 }
 
 // Launch one local-solve pass (first solve or refinement sweeps) over g.list, whose
-// first nbig subdomains have fragment-order factors; v: variant of the others.
+// first nbig subdomains are k_solve_big's; v: variant of the others.
 static void launch_local_pass(const Tables& t, const DeviceTables& d, const LocalArgs& g0, int nbig, const void* W,
                               bool sweep, int v, cudaStream_t st, Prof& P) {
     const bool f64 = t.cfg.precision == MRCM_FP64;
@@ -2448,8 +2407,8 @@ static void launch_local_pass(const Tables& t, const DeviceTables& d, const Loca
         a.stage_bytes = big.nt * 1024;
         size_t o = (size_t)a.stages * a.stage_bytes;
         a.ring = 0;
-        a.zp = (int)o; o += BigSmem::al(big.zp);
-        a.p = (int)o; o += BigSmem::al(big.p);
+        a.z = (int)o; o += BigSmem::al(big.zp);
+        a.p = (int)o; o += BigSmem::al(big.zp);
         a.co = (int)o; o += BigSmem::al(big.co);
         a.cols = (int)o; o += BigSmem::al(big.cols);
         a.bars = (int)o;

@@ -257,9 +257,8 @@ mrcm_status build_tables(const mrcm_config* cfg, Tables& t, std::string& err) {
         long long wcur = 0, wmax = 0;
         for (int q = 0; q < nsub; ++q) {
             SubInfo& s = t.subs[t.solve_list[q]];
-            s.frag = cfg->precision != MRCM_FP64 && big_ok(s.b, s.m) ? 1 : 0;
-            const long long need = (long long)s.ns * (t.cfg.precision == MRCM_FP64 ? wstride<double>(s.b)
-                                                      : s.frag ? frag_stride(s.b) : wstride<float>(s.b));
+            s.stream = cfg->precision != MRCM_FP64 && big_ok(s.b, s.m) ? 1 : 0;
+            const long long need = (long long)s.ns * (t.cfg.precision == MRCM_FP64 ? wstride<double>(s.b) : wstride<float>(s.b));
             if (cfg->wave_bytes > 0 && q > t.wave_off.back() && (size_t)(wcur + need) * welem > cfg->wave_bytes) {
                 t.wave_off.push_back(q);
                 wcur = 0;
@@ -271,10 +270,10 @@ mrcm_status build_tables(const mrcm_config* cfg, Tables& t, std::string& err) {
         t.wave_off.push_back(nsub);
         t.n_waves = (int)t.wave_off.size() - 1;
         t.total_w = wmax;
-        // within a wave, the fragment-order subdomains first (each kind has its own solve kernel)
+        // within a wave, the subdomains of k_solve_big first (each kind has its own solve kernel)
         for (int w = 0; w < t.n_waves; ++w) {
             const auto mid = std::stable_partition(t.solve_list.begin() + t.wave_off[w], t.solve_list.begin() + t.wave_off[w + 1],
-                                                   [&](int l) { return t.subs[l].frag != 0; });
+                                                   [&](int l) { return t.subs[l].stream != 0; });
             t.wave_big.push_back((int)(mid - t.solve_list.begin()) - t.wave_off[w]);
         }
         t.class_list.clear();
@@ -284,10 +283,10 @@ mrcm_status build_tables(const mrcm_config* cfg, Tables& t, std::string& err) {
                 const int l = t.solve_list[q];
                 const SubInfo& s = t.subs[l];
                 const double cost = (double)s.ns * s.b * s.b * s.b;
-                // small blocks; fragment-order factors; the others (and FP64).  The last two are ordered
-                // by b first (their factors launch one CTA shape per run of b), then by cost
-                const int k = cfg->precision == MRCM_FP64 ? 2 : s.b <= kRegBlock ? 0 : s.frag ? 1 : 2;
-                cls[k].push_back({k > 0 ? -s.b : 0, -cost, l});
+                const int k = cfg->precision == MRCM_FP64 ? 2 : s.b <= kRegBlock ? 0 : s.b <= kTileBlock ? 1 : 2;
+                // large class and FP64: ordered by b first (its factor launches
+                // one CTA size per run of b), then by cost
+                cls[k].push_back({k == 2 ? -s.b : 0, -cost, l});
             }
             for (int k = 0; k < 3; ++k) {
                 std::sort(cls[k].begin(), cls[k].end());
@@ -497,9 +496,9 @@ void compute_layout(const Tables& t, Layout& L) {
     L.scf = take(nc * sizeof(float));
     L.tsc = take(nc * sizeof(float));
     L.rhs_part = take(nc * sizeof(double));
-    bool any_frag = false;
-    for (const SubInfo& s : t.subs) any_frag = any_frag || s.frag;
-    L.cface = take(any_frag ? 6 * nc * sizeof(short) : 0);
+    bool any_stream = false;
+    for (const SubInfo& s : t.subs) any_stream = any_stream || s.stream;
+    L.cface = take(any_stream ? 6 * nc * sizeof(short) : 0);
     L.face_tr = take(t.faces.size() * sizeof(double));
     L.face_beta = take(t.faces.size() * sizeof(double));
     L.face_u = take(t.faces.size() * sizeof(double));

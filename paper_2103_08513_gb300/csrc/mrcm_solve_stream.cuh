@@ -1,54 +1,38 @@
-// Local solve of the mixed modes with the block products on the tensor cores
-// (one launch: the first solve, or the FP64-residual refinement passes), for the
-// subdomains whose block factor is stored in fragment order (SubInfo::frag).
-// Included by mrcm_local.cu inside its anonymous namespace.
+// Local solve of the mixed modes for slab blocks above 64 (one launch: the first
+// solve, or the FP64-residual refinement passes), for the subdomains with
+// SubInfo::stream.  Included by mrcm_local.cu inside its anonymous namespace.
 //
 // The slab recursion is the one of solve_one (forward Y_s = W_s Z_s, backward
 // x_s = Y_s + W_s (t x_{s+1})), built around three things:
 //
-//   * W streams.  A block is stored as panels of 16 k-columns, each a row of
-//     16 x 16 tiles in the order of the MMA's A fragments (frag_off), and one
-//     producer warp keeps a ring of panels filled by bulk copies through the whole
-//     pass -- over slab and sweep boundaries -- while eight warps consume them
-//     (mbarriers full / empty).  Before, a block was fetched whole into one or two
-//     buffers between barriers, with one CTA per SM at b >= 128 (or read from L2
-//     above 192), and the copy, the FP64 residual and the product took turns.
-//   * Products by mma.sync (m16n8k16, BF16): FP32 operands are cut into three BF16
-//     pieces (24 bits), the six piece products down to 2^-24 relative are summed
-//     per panel in a fresh accumulator and added in FP32 (the tensor core
-//     truncates its running sum).  W is cut in registers as it is consumed, Z once
-//     per slab by the thread that forms it.
+//   * W streams.  One producer warp keeps a ring of panels (16 rows k of W_s, row
+//     major) filled by bulk copies through the whole pass -- over slab and sweep
+//     boundaries -- while eight warps consume them (mbarriers full / empty).  Before,
+//     a block was fetched whole into one or two buffers between barriers, with one CTA
+//     per SM at b >= 128 (or read from L2 above 192), and the copy, the FP64 residual
+//     and the product took turns.
+//   * Products by FP32 FMAs, a warp's tile of 32 or 16 rows x 4, 8 or 16 columns, k in order:
+//     the sums of k_local_solve, bit for bit, so that a column does not depend on the
+//     route.  The refinement stops on the residual before a column's last correction,
+//     hence the rounding of the correction solve decides what is left in an
+//     ill-conditioned column: with factor and products in three BF16 pieces on the
+//     tensor cores X of 256 x 512 x 128 cells (sigma 3, stop 1e-10) moved by up to 2.6e-9.
 //   * Everything per entry (FP64 residual, Y and X traffic) is done by consecutive
 //     threads on consecutive cells; the product's result passes through shared
 //     memory (P) once.  Two CTAs per SM overlap one's FP64 with the other's products.
 //
-// 256 x 256 x 128 cells, uneven blocks of 64 to 256: first solve 11.5 -> 3.8 ms, six
-// sweeps 37.8 -> 11.6 ms; 256 x 512 x 128 cells, blocks of 128: 11.0 -> 6.5 and
-// 39.5 -> 23.0 ms.  A CTA spends about half of a pass on the entries and a third on the
-// products; neither the instructions that cut W (stored ready cut it was no faster) nor
-// the chain of the six products bounds it.
+// 256 x 256 x 128 cells, uneven blocks of 64 to 256, 13 columns: first solve 11.5 -> 4.3 ms,
+// six sweeps 37.8 -> 14.1 ms; 256 x 512 x 128 cells, blocks of 128: 11.0 -> 7.6 and
+// 39.5 -> 28.2 ms.  Bound by issue (54 % of the cycles in the first solve, 46 % in a sweep) and
+// by the alternation of the two phases: a third of the instructions are the products' FMAs, a
+// consumer warp has one of them in flight per scheduler at 13 columns, and the FP64 residual
+// of the entries takes the FP64 unit a fifth of the time.  (In three BF16 pieces on the tensor
+// cores 6.5 and 23.0 ms, but see above; 16 rows a tile, two a lane, 9.0 and 32.2.)
 #pragma once
 
 constexpr int kBigWarps = 8;                          // consumer warps; one producer warp after them
 constexpr int kBigThreads = 32 * (kBigWarps + 1);
 
-__device__ __forceinline__ void ldsm4(uint32_t addr, uint32_t r[4]) {
-    asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr) : "memory");
-}
-__device__ __forceinline__ void mma_16816(float d[4], const uint32_t a[4], uint32_t b0, uint32_t b1) {
-    asm volatile("mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-                 : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
-                 : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-// (a, b) = p1 + p2 + p3, BF16 pairs (a in the low half)
-__device__ __forceinline__ void cut3(float a, float b, uint32_t& p1, uint32_t& p2, uint32_t& p3) {
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p1) : "f"(b), "f"(a));
-    const float a1 = a - __uint_as_float(p1 << 16), b1 = b - __uint_as_float(p1 & 0xFFFF0000u);
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p2) : "f"(b1), "f"(a1));
-    const float a2 = a1 - __uint_as_float(p2 << 16), b2 = b1 - __uint_as_float(p2 & 0xFFFF0000u);
-    asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(p3) : "f"(b2), "f"(a2));
-}
 __device__ __forceinline__ void bar_consumers() { asm volatile("bar.sync 1, 256;" ::: "memory"); }
 __device__ __forceinline__ void mbar_arrive(unsigned long long* bar) {
     asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" :: "r"(smem_u32(bar)) : "memory");
@@ -57,12 +41,140 @@ __device__ __forceinline__ void mbar_arrive(unsigned long long* bar) {
 struct BigArgs {
     LocalArgs g;
     int stages, stage_bytes;
-    int ring, zp, p, co, cols, bars;   // shared-memory offsets (BigSmem)
+    int ring, z, p, co, cols, bars;    // shared-memory offsets (BigSmem)
 };
+
+// What a product needs besides the panel sequence.
+struct BigProduct {
+    const unsigned char* ring;
+    unsigned long long *full, *empty;
+    int stages, stage_bytes, b, na, ld;
+    const float* Z;                    // [column][k]
+    float* P;                          // [column][row]
+    int* abort_s;
+    int* status;
+};
+
+// P[column][row] = sum_k W[k][row] Z[column][k] of one slab, the panels as they arrive.  A
+// warp takes U tiles of 8 R rows x 4 C columns, lane (rl, cl) of 8 x 4 the rows R rl .. (b a
+// multiple of R: one vector load of W; R = 2 with odd b: the rows rl and rl + 8) and the
+// columns cl, cl + 4, ...  The lanes that share a row, or a column, are neighbours, which
+// makes a load of W one pass of the shared memory and four k of Z two.  With `park` P is
+// still read by the others until all consumers are here.
+template <int R, int C, int U, bool kOdd>
+__device__ __forceinline__ void big_product(const BigProduct& g, bool park, uint32_t& stage, uint32_t& parity) {
+    static_assert(R == 4 || R == 2, "rows a lane");
+    const int b = g.b, rt = (b + 8 * R - 1) / (8 * R), tiles = rt * ((g.na + 4 * C - 1) / (4 * C));
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int cl = (lane & 1) | ((lane >> 1) & 2), rl = ((lane >> 1) & 1) | ((lane >> 2) & 6);
+    float acc[U][R][C];
+    int wo[U], zo[U];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int x = min(warp + kBigWarps * u, tiles - 1), cb = x / rt, i0 = 8 * R * (x - cb * rt);
+        wo[u] = kOdd ? min(i0 + rl, b - 1) : min(i0 + R * rl, b - R);        // (rows past the block: never stored)
+        zo[u] = 4 * C * cb + cl;
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+            for (int c = 0; c < C; ++c) acc[u][r][c] = 0.0f;
+    }
+    const uint32_t zbase = smem_u32(g.Z), rbase = smem_u32(g.ring), b4 = 4u * (uint32_t)b;
+    for (int k0 = 0; k0 < b; k0 += 16) {
+        if (!mbar_try_wait(&g.full[stage], parity) && !*g.abort_s && !mbar_wait(&g.full[stage], parity)) {
+            if (lane == 0) { *g.abort_s = 1; atomicAdd(&g.status[ST_TIMEOUT], 1); }
+        }
+        const uint32_t pan = rbase + stage * (uint32_t)g.stage_bytes;
+        const int rows = min(16, b - k0);
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            if (warp + kBigWarps * u >= tiles) break;
+            uint32_t zc[C];                                   // shared addresses (32 bits, immediate offsets)
+#pragma unroll
+            for (int c = 0; c < C; ++c) zc[c] = zbase + 4u * (uint32_t)(min(zo[u] + 4 * c, g.na - 1) * g.ld + k0);
+            uint32_t w = pan + 4u * (uint32_t)wo[u];
+            const uint32_t w8 = kOdd ? 4u * (uint32_t)(min(wo[u] + 8, b - 1) - wo[u]) : 0u;
+            auto load_w = [&](float (&v)[R]) {
+                if constexpr (kOdd) {
+                    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v[0]) : "r"(w));
+                    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v[1]) : "r"(w + w8));
+                } else if constexpr (R == 4) {
+                    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                                 : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]) : "r"(w));
+                } else {
+                    asm volatile("ld.shared.v2.f32 {%0, %1}, [%2];" : "=f"(v[0]), "=f"(v[1]) : "r"(w));
+                }
+                w += b4;
+            };
+            auto group = [&](int k) {
+                float z[C][4], v[4][R];
+#pragma unroll
+                for (int c = 0; c < C; ++c)
+                    asm volatile("ld.shared.v4.f32 {%0, %1, %2, %3}, [%4];"
+                                 : "=f"(z[c][0]), "=f"(z[c][1]), "=f"(z[c][2]), "=f"(z[c][3]) : "r"(zc[c] + 4u * k));
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk) load_w(v[kk]);
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk)
+#pragma unroll
+                    for (int c = 0; c < C; ++c)
+#pragma unroll
+                        for (int r = 0; r < R; ++r) acc[u][r][c] = fmaf(v[kk][r], z[c][kk], acc[u][r][c]);
+            };
+            if (rows == 16) {
+#pragma unroll
+                for (int k = 0; k < 16; k += 4) group(k);
+            } else {
+                int k = 0;
+#pragma unroll 1
+                for (; k + 4 <= rows; k += 4) group(k);
+                if constexpr (R != 4) {                       // (b a multiple of four: none left)
+#pragma unroll 1
+                    for (; k < rows; ++k) {
+                        float v[R];
+                        load_w(v);
+#pragma unroll
+                        for (int c = 0; c < C; ++c) {
+                            float zz;
+                            asm volatile("ld.shared.f32 %0, [%1];" : "=f"(zz) : "r"(zc[c] + 4u * k));
+#pragma unroll
+                            for (int r = 0; r < R; ++r) acc[u][r][c] = fmaf(v[r], zz, acc[u][r][c]);
+                        }
+                    }
+                }
+            }
+        }
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&g.empty[stage]);
+        if (++stage == (uint32_t)g.stages) { stage = 0; parity ^= 1u; }
+    }
+    if (park) bar_consumers();
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        const int x = warp + kBigWarps * u;
+        if (x >= tiles) break;
+        const int i = 8 * R * (x % rt) + (kOdd ? rl : R * rl);
+        if (i >= b) continue;
+#pragma unroll
+        for (int c = 0; c < C; ++c) {
+            const int jj = zo[u] + 4 * c;
+            if (jj >= g.na) break;
+            float* q = g.P + jj * g.ld + i;
+            if constexpr (kOdd) {
+                q[0] = acc[u][0][c];
+                if (i + 8 < b) q[8] = acc[u][1][c];
+            } else if constexpr (R == 4) {
+                *reinterpret_cast<float4*>(q) = make_float4(acc[u][0][c], acc[u][1][c], acc[u][2][c], acc[u][3][c]);
+            } else {
+                *reinterpret_cast<float2*>(q) = make_float2(acc[u][0][c], acc[u][1][c]);
+            }
+        }
+    }
+}
 
 // One panel sequence state per thread: the count of panels consumed (produced) so far.
 template <bool kSweep, int U>
-__global__ void __launch_bounds__(kBigThreads, U <= 2 ? 2 : 1)
+__global__ void __launch_bounds__(kBigThreads, U == 1 ? 2 : 1)
 k_solve_big(BigArgs a, const float* __restrict__ Wall) {
     extern __shared__ __align__(128) unsigned char smem_ls[];
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the pass's launch for the smaller blocks may join
@@ -96,10 +208,9 @@ k_solve_big(BigArgs a, const float* __restrict__ Wall) {
         const int grp = it % G;
         const SubInfo s = g.subs[g.list[it / G]];
         const int b = s.b, m = s.m, N = s.N, su = s.su, nI = s.nI, ns = s.ns;
-        const int nt = (b + 15) >> 4, ldp = 16 * nt + 4, zs = 32 * nt + 16;
-        const int ncap = (((m + G - 1) / G + 15) >> 4) << 4;   // columns the planes hold
-        const uint32_t zpl = (uint32_t)ncap * zs;         // bytes of one piece's plane
-        unsigned char* Zp = sm + a.zp;                    // [piece][column][k] BF16
+        const int nt = (b + 15) >> 4, ld = 16 * nt + 4;
+        const int ncap = (((m + G - 1) / G + 7) >> 3) << 3;    // columns that Z and P hold
+        float* Z = reinterpret_cast<float*>(sm + a.z);    // [column][k]
         float* P = reinterpret_cast<float*>(sm + a.p);    // [column][row]
         double* co_d = reinterpret_cast<double*>(sm + a.co);
         double* co_u = co_d + b;
@@ -124,7 +235,7 @@ k_solve_big(BigArgs a, const float* __restrict__ Wall) {
         double* Xs = g.X + s.x_off;
         float* Ys = reinterpret_cast<float*>(g.Ybuf) + s.y_off;
         int* conv = g.conv + s.rhs_off;
-        const long long wst = frag_stride(b);
+        const long long wst = wstride<float>(b);
         const int np_pass = kSweep ? max(1, g.passes) : 1;
         for (int ps = 0; ps < np_pass; ++ps) {
             // ---- active columns (deterministic compaction by one warp)
@@ -142,16 +253,15 @@ k_solve_big(BigArgs a, const float* __restrict__ Wall) {
             __syncthreads();
             const int na = na_s;
             if (na == 0 || abort_s) { __syncthreads(); break; }
-            const int npair = (na + 15) >> 4;             // 16-column groups of the products
             if (producer) {
                 // ---- W panels W_0 .. W_{ns-1}, W_{ns-2} .. W_0 into the ring
                 if (lane == 0) {
-                    const uint32_t bytes = (uint32_t)nt * 1024u;
+                    const uint32_t whole = 64u * (uint32_t)b, rest = (uint32_t)(4 * wst) - (uint32_t)(nt - 1) * whole;
                     for (int q = 0; q < 2 * ns - 1 && !abort_s; ++q) {
                         const float* src = W + (q < ns ? q : 2 * ns - 2 - q) * wst;
                         for (int k = 0; k < nt; ++k) {
                             if (!mbar_wait(&empty[stage], parity ^ 1u)) { abort_s = 1; atomicAdd(&g.status[ST_TIMEOUT], 1); break; }
-                            bulk_load(sm + a.ring + stage * a.stage_bytes, src + (long long)k * nt * 256, bytes, &full[stage]);
+                            bulk_load(sm + a.ring + stage * a.stage_bytes, src + 16 * k * b, k + 1 < nt ? whole : rest, &full[stage]);
                             if (++stage == (uint32_t)S) { stage = 0; parity ^= 1u; }
                         }
                     }
@@ -161,7 +271,6 @@ k_solve_big(BigArgs a, const float* __restrict__ Wall) {
                 parity = __shfl_sync(0xffffffffu, parity, 0);
             } else {
                 // ---- consumers
-                for (uint32_t e = tid; e < 3 * zpl / 16; e += 256) reinterpret_cast<uint4*>(Zp)[e] = make_uint4(0u, 0u, 0u, 0u);
                 for (int e = tid; e < na; e += 256) {
                     nrm[e] = 0.0f;
                     float sc = 1.0f;
@@ -208,78 +317,21 @@ k_solve_big(BigArgs a, const float* __restrict__ Wall) {
                     }
                     msk_s[tid] = mk;
                 };
-                // P[column][row] = W_q Z for every 16-row tile and 16-column group: the products of
-                // the panels as they arrive, then (after `before_store`) the results
-                float acc[U][8];
-                auto product = [&]() {
-                    const int units = nt * npair;
-                    int mi[U], nj[U];
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const int x = warp + kBigWarps * u;
-                        nj[u] = x < units ? x / nt : -1;
-                        mi[u] = x - (x / nt) * nt;
-#pragma unroll
-                        for (int q = 0; q < 8; ++q) acc[u][q] = 0.0f;
+                const BigProduct bp_ = {sm + a.ring, full, empty, S, a.stage_bytes, b, na, ld, Z, P, &abort_s, g.status};
+                auto product = [&](bool park) {
+                    // four rows a lane where b allows it and the tiles of 32 rows fit the warps
+                    const bool wide = !(b & 3) && (b + 31) / 32 * ((na + 15) / 16) <= kBigWarps * U;
+                    if (b & 1) {
+                        if (na <= 4) big_product<2, 1, 2, true>(bp_, park, stage, parity);
+                        else big_product<2, 4, 2 * U, true>(bp_, park, stage, parity);
+                    } else if (!wide) {
+                        if (na <= 4) big_product<2, 1, 2, false>(bp_, park, stage, parity);
+                        else big_product<2, 4, 2 * U, false>(bp_, park, stage, parity);
+                    } else {
+                        if (na <= 4) big_product<4, 1, 1, false>(bp_, park, stage, parity);
+                        else if (na <= 8) big_product<4, 2, 1, false>(bp_, park, stage, parity);
+                        else big_product<4, 4, U, false>(bp_, park, stage, parity);
                     }
-                    const uint32_t zb = smem_u32(Zp) + (uint32_t)((lane & 7) + ((lane >> 4) & 1) * 8) * zs + ((lane >> 3) & 1) * 16;
-                    for (int k = 0; k < nt; ++k) {
-                        if (!abort_s && !mbar_wait(&full[stage], parity)) {
-                            if (lane == 0) { abort_s = 1; atomicAdd(&g.status[ST_TIMEOUT], 1); }
-                        }
-                        const unsigned char* pan = sm + a.ring + stage * a.stage_bytes;
-#pragma unroll
-                        for (int u = 0; u < U; ++u) {
-                            if (nj[u] < 0) break;
-                            const float4* at = reinterpret_cast<const float4*>(pan + mi[u] * 1024) + lane;
-                            const float4 w0 = at[0], w1 = at[32];
-                            uint32_t af[3][4];
-                            cut3(w0.x, w0.y, af[0][0], af[1][0], af[2][0]);
-                            cut3(w0.z, w0.w, af[0][1], af[1][1], af[2][1]);
-                            cut3(w1.x, w1.y, af[0][2], af[1][2], af[2][2]);
-                            cut3(w1.z, w1.w, af[0][3], af[1][3], af[2][3]);
-                            uint32_t bf[3][4];
-#pragma unroll
-                            for (int p = 0; p < 3; ++p) ldsm4(zb + p * zpl + (uint32_t)(16 * nj[u]) * zs + k * 32, bf[p]);
-                            float t0[4] = {0.f, 0.f, 0.f, 0.f}, t1[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll
-                            for (int d = 2; d >= 0; --d)
-#pragma unroll
-                                for (int pa = d; pa >= 0; --pa) {
-                                    mma_16816(t0, af[pa], bf[d - pa][0], bf[d - pa][1]);
-                                    mma_16816(t1, af[pa], bf[d - pa][2], bf[d - pa][3]);
-                                }
-#pragma unroll
-                            for (int q = 0; q < 4; ++q) { acc[u][q] += t0[q]; acc[u][4 + q] += t1[q]; }
-                        }
-                        __syncwarp();
-                        if (lane == 0) mbar_arrive(&empty[stage]);
-                        if (++stage == (uint32_t)S) { stage = 0; parity ^= 1u; }
-                    }
-                };
-                auto store_p = [&]() {
-                    const int units = nt * npair;
-#pragma unroll
-                    for (int u = 0; u < U; ++u) {
-                        const int x = warp + kBigWarps * u;
-                        if (x >= units) break;
-                        float* q0 = P + (16 * (x / nt) + 2 * (lane & 3)) * ldp + 16 * (x % nt) + (lane >> 2);
-#pragma unroll
-                        for (int h = 0; h < 2; ++h) {
-                            q0[8 * h * ldp] = acc[u][4 * h];
-                            q0[(8 * h + 1) * ldp] = acc[u][4 * h + 1];
-                            q0[8 * h * ldp + 8] = acc[u][4 * h + 2];
-                            q0[(8 * h + 1) * ldp + 8] = acc[u][4 * h + 3];
-                        }
-                    }
-                };
-                auto put_z2 = [&](int jj, int i, float za, float zb) {      // cells i (even) and i + 1
-                    uint32_t p1, p2, p3;
-                    cut3(za, zb, p1, p2, p3);
-                    unsigned char* q = Zp + (uint32_t)jj * zs + 2 * i;
-                    *reinterpret_cast<uint32_t*>(q) = p1;
-                    *reinterpret_cast<uint32_t*>(q + zpl) = p2;
-                    *reinterpret_cast<uint32_t*>(q + 2 * zpl) = p3;
                 };
                 auto particular = [&](int c) {                    // right-hand side of the particular column
                     int lc[3];
@@ -287,7 +339,7 @@ k_solve_big(BigArgs a, const float* __restrict__ Wall) {
                     return g.rhs_dir[s.cell_off + c] + g.f[global_cell(s, lc, g.geo.n)] * vol;
                 };
                 // entry walk: (column jj, slab cells i, i + 1), consecutive threads on consecutive
-                // pairs: the index and address arithmetic, the cut and the stores of Z serve two cells
+                // pairs: the index and address arithmetic and the stores of Z serve two cells
                 // (the two entry phases were half of a pass, ~100 instructions a cell)
                 const int bp = (b + 1) >> 1;
                 const int jj0 = tid / bp, i0 = tid - jj0 * bp, dj = 256 / bp, di = 256 - dj * bp;
@@ -343,7 +395,7 @@ k_solve_big(BigArgs a, const float* __restrict__ Wall) {
                             }
                             const float f0 = f64_to_f32_rz(r0), f1 = two ? f64_to_f32_rz(r1) : 0.0f;
                             float z0 = f0 * sc_s[i], z1 = f1 * sc_s[i1];
-                            float2* pp = reinterpret_cast<float2*>(&P[jj * ldp + i]);
+                            float2* pp = reinterpret_cast<float2*>(&P[jj * ld + i]);
                             if (sl > 0) {
                                 const float2 y = *pp;         // Y of the previous slab
                                 float* yo = Ys + (g.last_only ? (long long)c : o) - b;
@@ -353,7 +405,7 @@ k_solve_big(BigArgs a, const float* __restrict__ Wall) {
                             }
                             const float sb = rsb[jj], n0 = f0 * sb, n1 = f1 * sb;
                             *pp = make_float2(n0 * n0, n1 * n1);    // parked for the column's norm
-                            put_z2(jj, i, z0, z1);
+                            *reinterpret_cast<float2*>(&Z[jj * ld + i]) = make_float2(z0, z1);
                             i += 2 * di;
                             jj += dj;
                             if (i >= 2 * bp) { i -= 2 * bp; ++jj; }
@@ -363,13 +415,11 @@ k_solve_big(BigArgs a, const float* __restrict__ Wall) {
                     if (sl + 1 < ns) stage_load(sl + 1, true);
                     for (int jj = warp; jj < na; jj += kBigWarps) {     // fixed order per column
                         float rr = 0.0f;
-                        for (int i = lane; i < b; i += 32) rr += P[jj * ldp + i];
+                        for (int i = lane; i < b; i += 32) rr += P[jj * ld + i];
                         for (int o = 16; o > 0; o >>= 1) rr += __shfl_down_sync(0xffffffffu, rr, o);
                         if (lane == 0) nrm[jj] += rr;
                     }
-                    product();
-                    bar_consumers();                          // the parked norms are read
-                    store_p();
+                    product(true);                            // (the parked norms are read)
                     if (sl + 1 < ns) stage_store(true);
                     bar_consumers();
                 }
@@ -381,7 +431,7 @@ k_solve_big(BigArgs a, const float* __restrict__ Wall) {
                         const bool two = i + 1 < b;
                         const int i1 = two ? i + 1 : i;
                         const long long o = (long long)cols[jj] * N + base + i;
-                        float2 x = *reinterpret_cast<const float2*>(&P[jj * ldp + i]);
+                        float2 x = *reinterpret_cast<const float2*>(&P[jj * ld + i]);
                         if (sl + 1 < ns) {
                             const float* y = Ys + (g.last_only ? (long long)(base + i) : o);
                             x.x += y[0];
@@ -391,7 +441,7 @@ k_solve_big(BigArgs a, const float* __restrict__ Wall) {
                         const double x0 = f32_to_f64(x.x * sc_s[i]), x1 = f32_to_f64(x.y * sc_s[i1]);
                         if (kSweep) { xp[0] += x0; if (two) xp[1] += x1; }
                         else { xp[0] = x0; if (two) xp[1] = x1; }
-                        if (sl > 0) put_z2(jj, i, t_s[i] * x.x, two ? t_s[i1] * x.y : 0.0f);
+                        if (sl > 0) *reinterpret_cast<float2*>(&Z[jj * ld + i]) = make_float2(t_s[i] * x.x, two ? t_s[i1] * x.y : 0.0f);
                         i += 2 * di;
                         jj += dj;
                         if (i >= 2 * bp) { i -= 2 * bp; ++jj; }
@@ -399,8 +449,7 @@ k_solve_big(BigArgs a, const float* __restrict__ Wall) {
                     if (sl == 0) break;
                     bar_consumers();
                     stage_load(sl - 1, false);
-                    product();
-                    store_p();
+                    product(false);
                     stage_store(false);
                     bar_consumers();
                 }
