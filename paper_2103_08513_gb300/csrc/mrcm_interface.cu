@@ -326,7 +326,8 @@ constexpr int kPanelRows = 4;           // warps per panel-kernel CTA, two rows 
 // costs one FP64 operation per entry instead of one FMA per panel column.  (Eight slices
 // of 7 bits keep the same 56 bits at 36 products instead of 28.)
 constexpr int kOzS = 7;                     // slices per operand
-constexpr int kOzRowWords = 2 * kOzS * kPanel / 2;   // u32 words per slice row (2 operands x 8 slices x 32 bf16)
+constexpr int kOzRowWords = 2 * kOzS * kPanel / 2;   // u32 words per slice row (2 operands x 7 slices x 32 bf16)
+constexpr int kOzNotFinite = 1 << 20;       // exponent of a row that holds an infinity or a NaN: its products are NaN
 
 __device__ __forceinline__ bool oz_step(const FrontInfo& fr, int m, int nbk) {
     return fr.s_off >= 0 && m >= kOzMinM && nbk >= kOzMinK;
@@ -355,7 +356,7 @@ __device__ __forceinline__ void oz_slice_row(double x1, double x2, int p, int H,
         mx = max(mx, __shfl_sync(0xffffffffu, mx, base + min(p + o, H - 1)));
     mx = __shfl_sync(0xffffffffu, mx, base);
     if (!store) return;                                                    // after the segment reduction
-    const int E = mx == 0u ? 0 : (int)(mx >> 20) - 1023 + 1;               // max |x| < 2^E
+    const int E = mx == 0u ? 0 : mx >= 0x7FF00000u ? kOzNotFinite : (int)(mx >> 20) - 1023 + 1;   // max |x| < 2^E
     const unsigned long long F1 = oz_fixed(m1, E), F2 = oz_fixed(m2, E);
     const uint32_t sg = (uint32_t)(b1 >> 48 & 0x8000u) | (uint32_t)(b2 >> 32 & 0x80000000u);
 #pragma unroll
@@ -446,7 +447,7 @@ __device__ __forceinline__ void mma_bf16(float d[4], const uint32_t a[4], const 
 
 // The 128-bit integer v (|v| < 2^72), times 2^e, rounded to the nearest FP64 value with
 // integer operations only (ties away from zero; results below the normal
-// range become 0).
+// range become 0, above it infinite).
 __device__ __forceinline__ double i128_scaled(__int128 v, int e) {
     if (v == 0) return 0.0;
     const unsigned long long sign = v < 0 ? 0x8000000000000000ull : 0ull;
@@ -465,6 +466,7 @@ __device__ __forceinline__ double i128_scaled(__int128 v, int e) {
     }
     const int be = ex + 1023;
     if (be <= 0) return 0.0;
+    if (be >= 2047) return __longlong_as_double((long long)(sign | 0x7FF0000000000000ull));
     return __longlong_as_double((long long)(sign | ((unsigned long long)be << 52) | (mant & 0x000FFFFFFFFFFFFFull)));
 }
 
@@ -582,7 +584,8 @@ k_ldl_update(const FrontInfo* __restrict__ fronts, const int* __restrict__ ids, 
             const int gj = j0 + nc + 2 * tg + (q & 1);
             if (gi <= n && gj <= gi && gj < n) {
                 const int e = ez[mr + g + (q >> 1) * 8] + ez[kPanel + nc + 2 * tg + (q & 1)];
-                A[(long long)gi * n + gj] = cv[q] - i128_scaled(sum, e - 64);
+                const double prod = e >= kOzNotFinite / 2 ? __longlong_as_double(0x7FF8000000000000ll) : i128_scaled(sum, e - 64);
+                A[(long long)gi * n + gj] = cv[q] - prod;
             }
         }
     } else {
