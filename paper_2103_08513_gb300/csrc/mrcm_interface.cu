@@ -1233,15 +1233,15 @@ int configure_interface(const Tables& t, DeviceTables& d) {
     // opt in to the dynamic shared memory each substitution kernel may take
     // (static + dynamic above 48 KB needs it)
     d.front_smem = sizeof(double) * (size_t)std::max(t.max_front, 1);
-    cudaFuncSetAttribute(k_front_forward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d.front_smem);
-    cudaFuncSetAttribute(k_front_backward, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d.front_smem);
-    cudaFuncSetAttribute(k_front_backward_b, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d.front_smem);
+    allow_smem((const void*)k_front_forward, d.front_smem);
+    allow_smem((const void*)k_front_backward, d.front_smem);
+    allow_smem((const void*)k_front_backward_b, d.front_smem);
     size_t cl = 0;
     for (const FrontInfo& f : t.fronts)
         if (f.ne >= kSolveClMinNe) cl = std::max(cl, cl_smem_bytes(f.n, f.ne));
     const int lim = (int)std::max<size_t>(std::min(cl, kClSmemMax), 1);
-    cudaFuncSetAttribute(k_front_forward_cl, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
-    cudaFuncSetAttribute(k_front_backward_cl, cudaFuncAttributeMaxDynamicSharedMemorySize, lim);
+    allow_smem((const void*)k_front_forward_cl, lim);
+    allow_smem((const void*)k_front_backward_cl, lim);
     return (int)cudaGetLastError();
 }
 

@@ -291,6 +291,20 @@ inline bool big_ok(int b, int m) {
     return b >= kBigMinB && s.units <= kBigUnits && s.stages() >= 3;
 }
 
+// Opt in to `need` bytes of dynamic shared memory for a kernel.  The limit belongs to the function,
+// not to a handle: another handle or thread, with smaller blocks, would lower it under this one's
+// next launch.  So it is always set to all that the device allows beside the kernel's static part.
+inline cudaError_t allow_smem(const void* kernel, size_t need) {
+    int dev = 0, most = 0;
+    cudaFuncAttributes at;
+    cudaError_t e = cudaGetDevice(&dev);
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (e == cudaSuccess) e = cudaFuncGetAttributes(&at, kernel);
+    if (e != cudaSuccess) return e;
+    return cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                std::max((int)need, most - (int)at.sharedSizeBytes));
+}
+
 // Row chunks of the boundary back substitution for a level whose fronts have
 // at most max_nb boundary rows (about 128 rows per chunk, at most 8 chunks).
 inline int bwd_split(int max_nb) { return std::max(1, std::min(8, (max_nb + 127) / 128)); }

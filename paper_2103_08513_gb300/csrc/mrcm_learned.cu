@@ -682,15 +682,15 @@ mrcm_status mrcm_net_create(int in_channels, int hidden, int layers, int D, int 
     n->act_per_sample = aoff;
     const size_t sm = std::max(mrcm::conv_smem(hidden, hidden, n->S), mrcm::conv_smem(in_channels, hidden, n->S));
     if (sm > 227 * 1024) { delete n; return MRCM_ERR_NOT_IMPLEMENTED; }
-    cudaFuncSetAttribute(mrcm::k_conv_forward<mrcm::kMaxCh>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    cudaFuncSetAttribute(mrcm::k_conv_forward<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    mrcm::allow_smem((const void*)mrcm::k_conv_forward<mrcm::kMaxCh>, sm);
+    mrcm::allow_smem((const void*)mrcm::k_conv_forward<1>, sm);
     {
         const size_t smm = mrcm::conv_mma_smem(mrcm::ConvShape{n->D, n->H, n->W, n->S});
         n->mma_ok = smm <= 227 * 1024 &&
-                    cudaFuncSetAttribute(mrcm::k_conv_forward_mma, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smm) == cudaSuccess;
+                    mrcm::allow_smem((const void*)mrcm::k_conv_forward_mma, smm) == cudaSuccess;
         cudaGetLastError();
     }
-    cudaFuncSetAttribute(mrcm::k_conv_backward_data, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    mrcm::allow_smem((const void*)mrcm::k_conv_backward_data, sm);
     {
         const mrcm::TcGeo g(D, H, W);
         n->C = hidden > 16 ? 32 : 16;
@@ -1271,7 +1271,7 @@ mrcm_status mrcm_net_samples(mrcm_handle* h, const mrcm_net* net, void* ws, floa
     // parts per subdomain: two CTAs per SM when the subdomains are few
     const int nsub = (int)t.subs.size(), parts = std::max(1, std::min(32, (2 * h->d.sms + nsub - 1) / nsub));
     const size_t sm = sizeof(float) * 4 * (size_t)net->S;
-    cudaFuncSetAttribute(mrcm::k_gather_samples, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    mrcm::allow_smem((const void*)mrcm::k_gather_samples, sm);
     mrcm::k_gather_samples<<<dim3(nsub, parts), 256, sm, s>>>(h->d.subs, h->d.faces, soff, h->K,
         (const double*)((char*)ws + h->lay.X), t.cfg.nx, t.cfg.ny, t.n_cells, max_samples, x, target);
     return cudaGetLastError() == cudaSuccess ? MRCM_OK : MRCM_ERR_CUDA;
@@ -1326,7 +1326,7 @@ mrcm_status mrcm_solve_mbf_learned(mrcm_handle* h, const mrcm_net* net, const fl
                       : T == 512 ? (const void*)mrcm::k_learned_column<512> : (const void*)mrcm::k_learned_column<1024>;
         size_t sm = 0;
         for (const mrcm::SubInfo& sb : t.subs) sm = std::max(sm, (sizeof(double) + sizeof(float)) * ((size_t)sb.N + 2 * sb.b));
-        cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+        mrcm::allow_smem(k, sm);
         const int* list = h->col_list;
         const double *coef = (const double*)(w + h->lay.coef), *scale = (const double*)(w + h->lay.scale),
                      *ftr = (const double*)(w + h->lay.face_tr), *fu = (const double*)(w + h->lay.face_u),
@@ -1368,7 +1368,7 @@ mrcm_status mrcm_pcg_mbf(mrcm_handle* h, const mrcm_net* net, void* ws, const fl
     const mrcm::Tables& t = h->t;
     if (net->S > 1024) return MRCM_ERR_NOT_IMPLEMENTED;
     const size_t sm = sizeof(float) * 8 * (size_t)net->S;
-    cudaFuncSetAttribute(mrcm::k_pcg_sample, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    mrcm::allow_smem((const void*)mrcm::k_pcg_sample, sm);
     const char* w = (const char*)ws;
     mrcm::k_pcg_sample<<<n_samples, 512, sm, (cudaStream_t)stream>>>(h->d.subs, h->d.faces, slist,
         (const double*)(w + h->lay.coef), (const double*)(w + h->lay.scale), (const double*)(w + h->lay.face_tr),

@@ -2303,13 +2303,13 @@ int configure_local(const Tables& t, DeviceTables& d) {
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&d.sms, cudaDevAttrMultiProcessorCount, dev);
     const bool f64 = t.cfg.precision == MRCM_FP64;
-    cudaFuncSetAttribute(k_element, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)element_smem(t));
+    allow_smem((const void*)k_element, element_smem(t));
     d.solve_smem = solve_smem_bytes(t, t.cfg.precision);
     for (int v = 0; v < kNumSolveVariants; ++v) {
         const void* k0 = f64 ? solve_kernel<double, false, false>(v) : solve_kernel<float, true, false>(v);
         const void* k1 = f64 ? solve_kernel<double, false, true>(v) : solve_kernel<float, true, true>(v);
-        cudaFuncSetAttribute(k0, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d.solve_smem);
-        cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d.solve_smem);
+        allow_smem(k0, d.solve_smem);
+        allow_smem(k1, d.solve_smem);
         int occ0 = 0, occ1 = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ0, k0, variant_threads(v), d.solve_smem);
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ1, k1, variant_threads(v), d.solve_smem);
@@ -2320,7 +2320,7 @@ int configure_local(const Tables& t, DeviceTables& d) {
     if (big.units > 0) {
         for (int sw = 0; sw < 2; ++sw) {
             const void* k = big_kernel(sw == 1, big.units);
-            cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)big.total());
+            allow_smem(k, big.total());
             int occ = 0;
             cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k, kBigThreads, big.total());
             d.big_occ[sw] = std::max(1, occ);
@@ -2335,8 +2335,8 @@ int configure_local(const Tables& t, DeviceTables& d) {
         d.f64_solve_smem = sm + 16;
         const void* k0 = solve_kernel<double, false, false>(0);
         const void* k1 = solve_kernel<double, false, true>(0);
-        cudaFuncSetAttribute(k0, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d.f64_solve_smem);
-        cudaFuncSetAttribute(k1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)d.f64_solve_smem);
+        allow_smem(k0, d.f64_solve_smem);
+        allow_smem(k1, d.f64_solve_smem);
         int occ = 0;
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, k1, variant_threads(0), d.f64_solve_smem);
         d.f64_occ = std::max(1, occ);

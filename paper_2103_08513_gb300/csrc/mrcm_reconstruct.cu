@@ -180,8 +180,7 @@ __global__ void k_zero_u64(unsigned long long* x) { *x = 0ull; }
 }  // namespace
 
 int configure_reconstruct(const Tables& t) {
-    cudaFuncSetAttribute(k_reconstruct, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                         (int)(sizeof(double) * ((size_t)kMaxCells + t.max_m)));
+    allow_smem((const void*)k_reconstruct, (sizeof(double) * ((size_t)kMaxCells + t.max_m)));
     return (int)cudaGetLastError();
 }
 
