@@ -276,7 +276,9 @@ struct BigSmem {
     }
     static size_t al(size_t v) { return (v + 127) & ~size_t(127); }
     size_t rest() const { return 2 * al(zp) + al(co) + al(cols) + 256; }
-    // ring stages: eight if two CTAs then fit an SM, at least three of them; more shared memory for one CTA otherwise
+    // ring stages: eight if two CTAs then fit an SM, at least three of them; more shared memory for one
+    // CTA otherwise.  Any mixture of subdomains that big_ok admits one by one keeps at least three
+    // (Z and P of 64 tiles are about 65 KB each for every b; all mixed together: four).
     int stages() const {
         const size_t st = (size_t)nt * 1024;
         const long long two = ((long long)kSolveTwoCta - (long long)rest()) / (long long)st;
