@@ -324,7 +324,8 @@ mrcm_status mrcm_autotune(mrcm_handle* h, const double* f, void* ws, void* strea
 /* Median times (ms) of every local-solve variant in the last mrcm_autotune
  * of this handle (host only): solve_ms[v] the first solve, sweep_ms[v] the
  * cfg.ir_max_sweeps refinement sweeps in one launch (-1 where not timed: FP64
- * handles time no sweeps), and the resident CTAs per SM of each
+ * handles time no sweeps, and a handle whose blocks all have the one solve kernel
+ * of the larger ones times entry 0 only), and the resident CTAs per SM of each
  * (solve_ctas[v], sweep_ctas[v]).  Writes min(*n, cap) entries of each
  * non-NULL array; *n = the number of variants (0 before any autotune).
  * *sweeps_separate = 1 when the handle runs one launch per sweep (the

@@ -2687,7 +2687,7 @@ int launch_local_finish(const Tables& t, const DeviceTables& d, const Layout& L,
 // the fastest; (2) for every variant, after an untimed first solve, time the
 // whole refinement sequence as the solve runs it (ir_max_sweeps sweeps with
 // the configured tolerance, so retired columns shrink the later sweeps) and
-// keep the fastest.  Tuned on the first wave.
+// keep the fastest.  The factors are tuned on the first wave.
 int autotune_local(const Tables& t, DeviceTables& d, const Layout& L, char* ws, const double* f,
                    void* stream, int reps, int* best_solve, int* best_sweep, int* best_factor, int* best_factor_mid,
                    float* ms_out) {
@@ -2696,7 +2696,7 @@ int autotune_local(const Tables& t, DeviceTables& d, const Layout& L, char* ws, 
     g.tol2 = t.cfg.ir_tol * t.cfg.ir_tol;
     const void* W = (const void*)(ws + L.W);
     Prof dummy;
-    g.list = d.solve_list;                      // tune on the first wave
+    g.list = d.solve_list;
     g.nlist = t.wave_off[1];
     if (t.n_waves > 1) launch_factor_wave(t, d, L, ws, t.cfg.precision, 0, st, dummy);
     const bool mixed = t.cfg.precision != MRCM_FP64;
@@ -2761,14 +2761,23 @@ int autotune_local(const Tables& t, DeviceTables& d, const Layout& L, char* ws, 
         d.factor_mid_variant = *best_factor_mid;
         launch_factor_wave(t, d, L, ws, t.cfg.precision, 0, st, dummy);
     }
+    // the solve variants: on the first wave with a subdomain that takes one (the largest blocks, which
+    // come first, may all take k_solve_big); a handle without any keeps variant 0
+    int wv = 0;
+    while (wv < t.n_waves && t.wave_big[wv] == t.wave_off[wv + 1] - t.wave_off[wv]) ++wv;
+    const int nv = wv < t.n_waves ? kNumSolveVariants : 1;
+    if (wv == t.n_waves) wv = 0;
+    if (wv > 0) launch_factor_wave(t, d, L, ws, t.cfg.precision, wv, st, dummy);
+    g.list = d.solve_list + t.wave_off[wv];
+    g.nlist = t.wave_off[wv + 1] - t.wave_off[wv];
     float best0 = 1e30f, best1 = 1e30f;
     *best_solve = 0;
     *best_sweep = 0;
-    for (int v = 0; v < kNumSolveVariants; ++v) {
+    for (int v = 0; v < nv; ++v) {
         std::vector<float> t0;
         for (int r = 0; r < reps; ++r) {
             cudaEventRecord(e0, st);
-            launch_local_pass(t, d, g, t.wave_big[0], W, false, v, st, dummy);
+            launch_local_pass(t, d, g, t.wave_big[wv], W, false, v, st, dummy);
             cudaEventRecord(e1, st);
             cudaEventSynchronize(e1);
             float ms = 0.f;
@@ -2780,13 +2789,13 @@ int autotune_local(const Tables& t, DeviceTables& d, const Layout& L, char* ws, 
         if (m0 < best0) { best0 = m0; *best_solve = v; }
     }
     if (mixed) {
-        for (int v = 0; v < kNumSolveVariants; ++v) {
+        for (int v = 0; v < nv; ++v) {
             std::vector<float> t1;
             for (int r = 0; r < reps; ++r) {
-                launch_local_pass(t, d, g, t.wave_big[0], W, false, *best_solve, st, dummy);
+                launch_local_pass(t, d, g, t.wave_big[wv], W, false, *best_solve, st, dummy);
                 cudaEventRecord(e0, st);
                 g.passes = t.cfg.ir_max_sweeps;          // all sweeps in one launch
-                if (g.passes > 0) launch_local_pass(t, d, g, t.wave_big[0], W, true, v, st, dummy);
+                if (g.passes > 0) launch_local_pass(t, d, g, t.wave_big[wv], W, true, v, st, dummy);
                 g.passes = 1;
                 cudaEventRecord(e1, st);
                 cudaEventSynchronize(e1);
@@ -2801,9 +2810,9 @@ int autotune_local(const Tables& t, DeviceTables& d, const Layout& L, char* ws, 
         // the chosen variant with one launch per sweep
         std::vector<float> t2;
         for (int r = 0; r < reps && t.cfg.ir_max_sweeps > 0; ++r) {
-            launch_local_pass(t, d, g, t.wave_big[0], W, false, *best_solve, st, dummy);
+            launch_local_pass(t, d, g, t.wave_big[wv], W, false, *best_solve, st, dummy);
             cudaEventRecord(e0, st);
-            for (int it = 0; it < t.cfg.ir_max_sweeps; ++it) launch_local_pass(t, d, g, t.wave_big[0], W, true, *best_sweep, st, dummy);
+            for (int it = 0; it < t.cfg.ir_max_sweeps; ++it) launch_local_pass(t, d, g, t.wave_big[wv], W, true, *best_sweep, st, dummy);
             cudaEventRecord(e1, st);
             cudaEventSynchronize(e1);
             float ms = 0.f;
