@@ -183,13 +183,19 @@ def oracle_sample(w, K, f, n_sub_sample, seed=0, pool=None):
 
 
 # ------------------------------------------------------------------ roofline
+# slice pairs that k_ldl_update executes (seven 8-bit slices per operand: those with t + u < 7) of
+# those that ldl_update_tensor_flops counts (eight 7-bit slices)
+LDL_EXECUTED = 28.0 / 36.0
+
+
 def kernel_work(name, sizes, swept, precision, peaks, sweeps=0):
     """Algorithmic work of one solve step for a kernel: (work, bound, unit, peak)."""
     f32 = precision != "fp64"
     alu32 = peaks["fp32_tflops"] if f32 else peaks["fp64_tflops"]
     if name == "k_ldl_update":
         # the emulated FP64 trailing update runs its products on the BF16 tensor cores: the BF16
-        # flops of its slice products against the sustained BF16 peak (timed inside the solve)
+        # flops of its slice products, counted with eight slices per operand, against the sustained
+        # BF16 peak (timed inside the solve); what the kernel executes of them is given beside it
         return sizes["ldl_update_tensor_flops"], "tensor", "TFLOP/s", peaks["bf16_tflops_sustained"]
     if name == "k_ldl_panel":
         return sizes["ldl_flops"] - sizes["ldl_update_flops"], "alu", "TFLOP/s", peaks["fp64_tflops"]
@@ -226,8 +232,11 @@ def roofline(name, total_ms, launches, steps, sizes, swept, precision, peaks, wo
     per_step_s = total_ms / 1e3 / steps
     scale = 1e12 if unit == "TFLOP/s" else 1e9
     achieved = work / per_step_s / scale
+    executed = {}
+    if name == "k_ldl_update":                       # seven slices: the tensor cores' own rate
+        executed = {"executed": round(achieved * LDL_EXECUTED, 4), "executed_frac": round(achieved * LDL_EXECUTED / peak, 4)}
     return {"kernel": name, "bound": bound, "achieved": round(achieved, 4), "peak": round(peak, 2), "unit": unit,
-            "frac": round(achieved / peak, 4),
+            "frac": round(achieved / peak, 4), **executed,
             "traffic": traffic_per_launch(workload_key, name) if workload_key else None, "launches": launches,
             "avg_launch_ms": round(total_ms / max(launches, 1), 4),
             "work_per_step": work,

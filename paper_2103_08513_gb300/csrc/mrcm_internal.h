@@ -18,9 +18,10 @@ constexpr int kNumFactorVariants = 3;  // factor kernels for blocks with b <= 64
 constexpr int kOzMinN = 32;        // fronts with n >= kOzMinN may take the tensor-core emulated FP64 update
 constexpr int kOzMinM = 24;        // a step emulates when the trailing block has >= kOzMinM rows
 constexpr int kOzMinK = 4;         // and the panel >= kOzMinK columns
-// BF16 flops that the emulated update of one 32 x 32 tile is counted as: eight slices of 7 bits
-// per operand, 8 warps x 36 slice pairs x 2 halves of the panel x m16n8k16 MMAs (the reported
-// figure; the kernel gets the same 56 bits from seven slices of 8 bits, 28 pairs)
+// BF16 flops that the emulated update of one 32 x 32 tile is counted as, a fixed measure of its
+// work: eight slices of 7 bits per operand, 8 warps x 36 slice pairs x 2 halves of the panel x
+// m16n8k16 MMAs.  The kernel gets the same 56 bits from seven slices of 8 bits and executes 28
+// pairs: 28 / 36 of this count
 constexpr double kOzTileFlops = 8.0 * 36.0 * 2.0 * (2.0 * 16 * 8 * 16);
 constexpr int kTileBlock = 128;     // 64 < b <= kTileBlock: register-tiled FP32 factor (8 x 8 per thread)
 constexpr int kMaxI = 128;          // largest |I^l| (basis functions touching one subdomain)

@@ -420,8 +420,10 @@ mrcm_status build_tables(const mrcm_config* cfg, Tables& t, std::string& err) {
             for (int k0 = 0; k0 < f.ne; k0 += 32) {
                 const int nbk = std::min(32, f.ne - k0), m = f.n - k0 - nbk;
                 if (m < kOzMinM || nbk < kOzMinK) continue;
-                const double nt = (m + 31) / 32;
-                t.ldl_update_tensor_flops += nt * (nt + 1.0) / 2.0 * kOzTileFlops;
+                // rows of the trailing block and the right-hand side's; a last tile that only that row
+                // reaches on the diagonal has no entry
+                const double nt = (m + 1 + 31) / 32;
+                t.ldl_update_tensor_flops += (nt * (nt + 1.0) / 2.0 - (m % 32 == 0 ? 1.0 : 0.0)) * kOzTileFlops;
             }
         }
         t.total_front = foff;
