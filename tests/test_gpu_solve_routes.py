@@ -61,3 +61,17 @@ def test_a_column_has_the_same_bits_on_every_route(edge, b, patches, streams):
             assert all(np.isfinite(x).all() and np.abs(x[:2]).max() > 0 for x in got)
         for x, y in zip(got, first):
             assert np.array_equal(x, y)
+
+
+def test_both_routes_above_64_in_one_handle(streams):
+    """Subdomains of 16 x 16 x 16 cells past the limit (b 256, 65 right-hand sides) beside
+    16 x 9 x 16 below it (b 144, 57): the two kernels of a pass side by side, against the
+    oracle (1e-8 relative L2, the mixed bar of the parity tests)."""
+    from gpu_helpers import rel_l2, run_gpu
+    assert not streams(256, 65) and streams(144, 57)
+    w = small(n=(32, 25, 16), edges=([16, 16], [16, 9], [16]), patch=((4, 4),) * 3, sigma=1.5, lam=4.0)
+    prob = oracle.from_workload(w)
+    r = oracle.solve_mrcm(prob)
+    s, p, u, X, mres, code, st = run_gpu(w, prob.K, prob.f, "fp32_ir", ir_max_sweeps=8, ir_tol=1e-13)
+    assert s.sizes["max_rhs"] == 65 and st["not_spd"] == 0 and st["unconverged"] == 0
+    assert rel_l2(p, r.p) < 1e-8 and rel_l2(u.ravel(), r.u.ravel()) < 1e-8 and rel_l2(X, r.X) < 1e-8
