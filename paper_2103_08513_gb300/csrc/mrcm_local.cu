@@ -2042,7 +2042,7 @@ __global__ void k_pp_unconverged(const SubInfo* __restrict__ subs, int n, const 
     }
 }
 
-// The number of taken slots in each chunk, from the total at cnt[chunks] (also added to *total).
+// The number of taken slots in each chunk, from the total at cnt[chunks] (which *total gets too).
 __global__ void k_pp_chunks(int* __restrict__ cnt, int chunks, int cap, int* __restrict__ total) {
     const int n = cnt[chunks];
     for (int q = threadIdx.x; q < chunks; q += blockDim.x) cnt[q] = (int)max(0LL, min((long long)cap, n - (long long)q * cap));

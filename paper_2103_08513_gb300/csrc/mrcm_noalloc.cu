@@ -52,7 +52,7 @@ __device__ __forceinline__ int side_face(const BoxArgs& a, int axis, const int l
 }
 
 // Transmissibility of the face between cells of permeability k1 and k2, and the
-// Robin and Dirichlet half-cell ones (Newton reciprocals instead of divisions).
+// Robin and Dirichlet half-cell ones (reciprocals in integers instead of divisions).
 __device__ __forceinline__ double t_inner(double ah, double k1, double k2) { return 2.0 * ah * k1 * k2 * mrcm::rcp64(k1 + k2); }
 __device__ __forceinline__ double t_robin(double area, double h, double k, double beta) {
     return area * mrcm::rcp64(fma(0.5 * h, mrcm::rcp64(k), beta));

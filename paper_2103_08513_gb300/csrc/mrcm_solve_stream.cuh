@@ -22,12 +22,12 @@
 //     memory (P) once.  Two CTAs per SM overlap one's FP64 with the other's products.
 //
 // 256 x 256 x 128 cells, uneven blocks of 64 to 256, 13 columns: first solve 11.5 -> 4.3 ms,
-// six sweeps 37.8 -> 14.1 ms; 256 x 512 x 128 cells, blocks of 128: 11.0 -> 7.6 and
-// 39.5 -> 28.2 ms.  Bound by issue (54 % of the cycles in the first solve, 46 % in a sweep) and
-// by the alternation of the two phases: a third of the instructions are the products' FMAs, a
-// consumer warp has one of them in flight per scheduler at 13 columns, and the FP64 residual
-// of the entries takes the FP64 unit a fifth of the time.  (In three BF16 pieces on the tensor
-// cores 6.5 and 23.0 ms, but see above; 16 rows a tile, two a lane, 9.0 and 32.2.)
+// six sweeps 37.8 -> 13.9 ms; 256 x 512 x 128 cells, blocks of 128: 11.0 -> 7.6 and
+// 39.5 -> 28.0 ms.  No pipe or memory is near its limit (issue 55 % of the cycles in the first
+// solve, 51 % in the sweeps; FMA pipe 26 and 22, FP64 27 in the sweeps, DRAM 31 and 26): the
+// entries and the products take turns on the same warps, and at 13 columns half of the warps
+// have a tile.  (In three BF16 pieces on the tensor cores 6.5 and 23.0 ms, but see above;
+// tiles of 16 rows 9.0 and 32.2, tiles of 8 columns, which give every warp one, 7.7 and 27.8.)
 #pragma once
 
 constexpr int kBigWarps = 8;                          // consumer warps; one producer warp after them

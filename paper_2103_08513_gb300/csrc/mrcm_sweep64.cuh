@@ -10,8 +10,8 @@
 // What bounds it: the FP64 units.  A warp's FP64 instruction holds the unit of
 // its SM sub-partition for about 64 cycles whatever its active lanes (19 cycles
 // per SM over the four), so the count of FP64 warp instructions per pivot is the
-// cost: 16 updates and 4 scalings per tile warp -- 60 at b = 50 against 40 for
-// the bare triangle; a packed triangle in shared memory with a warp per row took
+// cost: 16 updates and 4 scalings per tile warp -- 60 at b = 50 (64 with the pivot warp's)
+// against 40 for the bare triangle; a packed triangle in shared memory with a warp per row took
 // about 250 (two operations per entry, idle lanes past the diagonal, a division
 // in every warp).  The next pivot and its reciprocal (two FP64 operations, then integer ones)
 // are formed by a warp of their own, which at b <= 52 is the fourth
