@@ -1290,8 +1290,11 @@ __device__ __forceinline__ void block_gemm_entry(const T* __restrict__ Wsm, cons
 // 3xTF32 tensor-core path (FP32 operands only), RT < 0 the pair tile (odd b:
 // the one-row tile).  Few columns leave those tiles on a warp or two, and the FP64 unit of
 // the other schedulers idle.  A pass over one column alone (`single`: the post-processing)
-// shares each entry's k among lanes, b = 50 in FP64: 170 -> 45 us a pass over 126
-// subdomains.  FP64 products of up to two entries a thread take a thread per entry; k
+// takes a thread per entry, in FP64 shared by lanes over k, b = 50: 170 -> 45 us a pass over
+// 126 subdomains.  (Not in FP32: no faster, and the refinement leaves the rounding of these
+// sums in ill-conditioned columns, which another order moved by up to 8.5e-10 of the
+// saturation of a two-phase run, seed 118 of 24; 1.8e-12 with k in order.)  FP64 products of
+// up to two entries a thread take a thread per entry; k
 // stays in order there, so that a column's bits do not depend on how many are active
 // with it (40 x 40 x 8, 4 columns a CTA: with the groups of column_groups, 319 -> 143 us).
 template <typename T, int RT, typename Store>
@@ -1300,7 +1303,8 @@ __device__ __forceinline__ void block_product(const T* Wsm, const T* Z, int b, i
     if constexpr (RT != 0) {
         if (single) {
             int KS = 1;
-            while (KS < 16 && 2 * KS * b <= (int)blockDim.x) KS <<= 1;
+            if constexpr (std::is_same<T, double>::value)
+                while (KS < 16 && 2 * KS * b <= (int)blockDim.x) KS <<= 1;
             block_gemm_entry<T>(Wsm, Z, b, na, mpad, KS, store);
             return;
         }

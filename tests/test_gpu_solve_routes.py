@@ -75,3 +75,23 @@ def test_both_routes_above_64_in_one_handle(streams):
     s, p, u, X, mres, code, st = run_gpu(w, prob.K, prob.f, "fp32_ir", ir_max_sweeps=8, ir_tol=1e-13)
     assert s.sizes["max_rhs"] == 65 and st["not_spd"] == 0 and st["unconverged"] == 0
     assert rel_l2(p, r.p) < 1e-8 and rel_l2(u.ravel(), r.u.ravel()) < 1e-8 and rel_l2(X, r.X) < 1e-8
+
+
+def test_post_processing_has_the_same_bits_on_either_route(streams):
+    """The one column of the post-processing's FP32 pass: subdomains of 6 x 11 x 12 cells below the
+    limit and, with 96 patches, past it, on the same multiscale velocity."""
+    from paper_2103_08513_gb300 import MRCM
+    assert streams(66, 5) and not streams(66, 193)
+    first = None
+    for patch, m in ((((0, 0), (0, 0), (0, 0)), 5), (((3, 2), (1, 1), (0, 0)), 193)):
+        w = small(n=(12, 22, 12), edges=([6, 6], [11, 11], [12]), patch=patch, sigma=2.5, lam=6.0)
+        prob = oracle.from_workload(w)
+        s = MRCM(w.n, w.edges, w.patch, precision="fp32_ir", ir_max_sweeps=8, ir_tol=1e-12)
+        assert s.sizes["max_rhs"] == m and s.sizes["max_block"] == 66
+        p, u, X, _ = s.solve(torch.from_numpy(prob.K).cuda(), torch.from_numpy(prob.f).cuda())
+        if first is None:
+            given = u.clone()
+        up, _ = s.postprocess_velocity(given.clone())
+        torch.cuda.synchronize()
+        first = up if first is None else first
+        assert torch.isfinite(up).all() and torch.equal(up, first)
